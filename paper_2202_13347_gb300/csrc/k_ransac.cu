@@ -13,21 +13,33 @@
 // are refitted by least squares (two equations per point, normal equations)
 // and recounted, `refits` times.
 //
-//   k_ransac_frames  one block: the two normalising frames (fixed-order sums)
-//   k_ransac_hyp     one warp per 8 hypotheses: each of 8 lanes solves one,
-//                    then the warp counts inliers for each model in turn
-//   k_ransac_final   one block: argmax, refits (normal equations reduced in a
-//                    fixed order: warp shuffles, then the warps in order)
+//   k_ransac_frames  one cluster: the two normalising frames (fixed-order sums)
+//   k_ransac_solve   8 lanes per hypothesis: the minimal system, a row per lane
+//   k_ransac_score   inlier counts of every model: FP32 with an error bound,
+//                    FP64 only for points the bound cannot decide
+//   k_ransac_final   one cluster: argmax, refits (normal equations reduced in
+//                    a fixed order), inlier mask
+// FP64 runs at two lanes per clock and SM here (1/64 of FP32), so it sets
+// the time of every step that uses it: the steps below either take it off
+// the per-(point, hypothesis) path or spread it over more SMs.  1000 points,
+// 4096 hypotheses: 556 us before, 115 us now (frames 14, solve 32, score 22, final 45).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace sfoc {
 
 namespace {
 
 constexpr int kRsThreads = 256;
-constexpr int kHpw = 8;  // hypotheses per warp (one warp per CTA)
+constexpr int kRsCtas = 8;     // CTAs of the cluster of the frame and final kernels (the portable size)
+constexpr int kSolveThreads = 32;  // one warp per CTA, so that the warps spread over the SMs
+constexpr int kScoreHyps = 16;  // hypotheses per scoring CTA
+constexpr int kScorePts = 1024;  // points staged at a time
+constexpr int kScoreList = 2048;  // undecided tests listed per CTA and turn (more are decided in place)
 
 struct Frames {
     double s[3];  // source: scale, cx, cy  (p -> s (p - c))
@@ -37,57 +49,83 @@ struct Frames {
 
 __device__ __forceinline__ bool is_valid(const uint8_t* valid, int i) { return !valid || valid[i] != 0; }
 
-// sum over the block of v (fixed order: strided per thread, shuffles, warps in order)
-__device__ double block_sum(double v, double* sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+// K sums over the block (fixed order: strided per thread, shuffles, warps in
+// order), left in tot[0 .. K-1].  `part`: K doubles per warp.
+template <int K>
+__device__ void block_sums(double (&v)[K], double* part, double* tot) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+    if (l == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) part[w * K + k] = v[k];
     __syncthreads();
-    if (l == 0) sh[w] = v;
+    if (threadIdx.x < K) {
+        double t = 0.0;
+        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += part[i * K + threadIdx.x];
+        tot[threadIdx.x] = t;
+    }
     __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += sh[i];
-    __syncthreads();
-    if (threadIdx.x == 0) sh[0] = t;
-    __syncthreads();
-    const double r = sh[0];
-    __syncthreads();
-    return r;
 }
 
-__global__ void __launch_bounds__(kRsThreads) k_ransac_frames(const double* __restrict__ src,
-                                                              const double* __restrict__ dst,
-                                                              const uint8_t* __restrict__ valid, int n,
-                                                              Frames* __restrict__ out) {
-    __shared__ double sh[kRsThreads / 32];
-    double c = 0.0, sx = 0.0, sy = 0.0, dx = 0.0, dy = 0.0;
-    for (int i = threadIdx.x; i < n; i += kRsThreads)
+// One cluster of kRsCtas CTAs: the two hypot per point are ~50 FP64
+// instructions (64 clocks each for a warp), which on a single SM took longer
+// than all scoring.  Every CTA takes the means itself; the distances are
+// computed in turns of one point per thread of the cluster and added by CTA 0
+// in the points' order.
+__global__ void __cluster_dims__(kRsCtas, 1, 1) __launch_bounds__(kRsThreads)
+    k_ransac_frames(const double* __restrict__ src, const double* __restrict__ dst,
+                    const uint8_t* __restrict__ valid, int n, Frames* __restrict__ out) {
+    __shared__ double s_part[kRsThreads / 32 * 5], s_tot[5], s_mean[4];
+    __shared__ double s_d[2][2][kRsThreads];  // two turns in flight: source and destination distances
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+    double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int i = tid; i < n; i += kRsThreads)
         if (is_valid(valid, i)) {
-            c += 1.0;
-            sx += src[2 * i];
-            sy += src[2 * i + 1];
-            dx += dst[2 * i];
-            dy += dst[2 * i + 1];
+            a[0] += 1.0;
+            a[1] += src[2 * i];
+            a[2] += src[2 * i + 1];
+            a[3] += dst[2 * i];
+            a[4] += dst[2 * i + 1];
         }
-    const double cnt = block_sum(c, sh);
-    const double mx = cnt > 0 ? block_sum(sx, sh) / cnt : 0.0, my = cnt > 0 ? block_sum(sy, sh) / cnt : 0.0;
-    const double nx = cnt > 0 ? block_sum(dx, sh) / cnt : 0.0, ny = cnt > 0 ? block_sum(dy, sh) / cnt : 0.0;
+    block_sums(a, s_part, s_tot);
+    const double cnt = s_tot[0];
+    if (tid < 4) s_mean[tid] = cnt > 0 ? s_tot[1 + tid] / cnt : 0.0;
+    __syncthreads();
+    const double mx = s_mean[0], my = s_mean[1], nx = s_mean[2], ny = s_mean[3];
     double ds = 0.0, dd = 0.0;
-    for (int i = threadIdx.x; i < n; i += kRsThreads)
-        if (is_valid(valid, i)) {
-            ds += hypot(src[2 * i] - mx, src[2 * i + 1] - my);
-            dd += hypot(dst[2 * i] - nx, dst[2 * i + 1] - ny);
-        }
-    const double ms = cnt > 0 ? block_sum(ds, sh) / cnt : 0.0, md = cnt > 0 ? block_sum(dd, sh) / cnt : 0.0;
-    if (threadIdx.x == 0) {
-        out->s[0] = ms > 0.0 ? sqrt(2.0) / ms : 1.0;
-        out->s[1] = mx;
-        out->s[2] = my;
-        out->d[0] = md > 0.0 ? sqrt(2.0) / md : 1.0;
-        out->d[1] = nx;
-        out->d[2] = ny;
-        out->n_valid = (int)cnt;
+    int turn = 0;
+    for (int i0 = 0; i0 < n; i0 += kRsCtas * kRsThreads, turn ^= 1) {
+        const int i = i0 + rank * kRsThreads + tid;
+        const bool v = i < n && is_valid(valid, i);
+        s_d[turn][0][tid] = v ? hypot(src[2 * i] - mx, src[2 * i + 1] - my) : 0.0;
+        s_d[turn][1][tid] = v ? hypot(dst[2 * i] - nx, dst[2 * i + 1] - ny) : 0.0;
+        // (the next turn's sync orders these reads before this buffer's next use)
+        cl.sync();
+        if (rank == 0)
+            for (int r = 0; r < kRsCtas; ++r) {
+                const int j = i0 + r * kRsThreads + tid;
+                if (j < n && is_valid(valid, j)) {
+                    const double* d = cl.map_shared_rank(&s_d[turn][0][0], r);
+                    ds += d[tid];
+                    dd += d[kRsThreads + tid];
+                }
+            }
     }
+    cl.sync();  // no CTA leaves while CTA 0 reads its distances
+    if (rank != 0) return;
+    double d[2] = {ds, dd};
+    block_sums(d, s_part, s_tot);
+    if (tid < 2) {
+        const double mean = cnt > 0 ? s_tot[tid] / cnt : 0.0;
+        double* f = tid ? out->d : out->s;
+        f[0] = mean > 0.0 ? sqrt(2.0) / mean : 1.0;
+        f[1] = s_mean[2 * tid];
+        f[2] = s_mean[2 * tid + 1];
+    }
+    if (tid == 0) out->n_valid = (int)cnt;
 }
 
 // the two equations of one correspondence (normalised coordinates)
@@ -98,59 +136,84 @@ __device__ __forceinline__ void eq_rows(bool proj, double x, double y, double xp
     r2[6] = proj ? -x * yp : 0.0; r2[7] = proj ? -y * yp : 0.0;
 }
 
-// Gaussian elimination with partial pivoting, n <= 8 (A row-major, b: rhs);
-// false when a pivot falls below 1e-12
-__device__ bool solve_small(double* A, double* b, int n, double* x) {
-    for (int c = 0; c < n; ++c) {
+// Gaussian elimination with partial pivoting of one n x n system (n <= 8) by
+// a group of 8 lanes: lane r holds row r and right side b, so the divisions
+// and updates of a step run side by side (a warp's FP64 instruction takes 64
+// clocks whatever its lanes do, and one thread per system needed ~1100 of
+// them).  Every lane of the warp calls it; the solution comes back in every
+// lane of the group.  False when a pivot falls below 1e-12.
+__device__ bool solve_group(double (&A)[8], double b, int n, double (&x)[8]) {
+    const unsigned full = 0xffffffffu;
+    const int r8 = threadIdx.x & 7;
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        if (c >= n) break;
         int p = c;
-        for (int r = c + 1; r < n; ++r)
-            if (fabs(A[r * 8 + c]) > fabs(A[p * 8 + c])) p = r;
-        if (fabs(A[p * 8 + c]) < 1e-12) return false;
-        if (p != c) {
-            for (int k = 0; k < n; ++k) {
-                const double t = A[c * 8 + k];
-                A[c * 8 + k] = A[p * 8 + k];
-                A[p * 8 + k] = t;
+        double v = fabs(__shfl_sync(full, A[c], c, 8));
+#pragma unroll
+        for (int r = c + 1; r < 8; ++r) {
+            const double u = fabs(__shfl_sync(full, A[c], r, 8));
+            if (r < n && u > v) {
+                v = u;
+                p = r;
             }
-            const double t = b[c];
-            b[c] = b[p];
-            b[p] = t;
         }
-        for (int r = c + 1; r < n; ++r) {
-            const double f = A[r * 8 + c] / A[c * 8 + c];
-            for (int k = c; k < n; ++k) A[r * 8 + k] -= f * A[c * 8 + k];
-            b[r] -= f * b[c];
+        if (v < 1e-12) ok = false;
+        const int from = r8 == c ? p : (r8 == p ? c : r8);
+#pragma unroll
+        for (int k = c; k < 8; ++k) A[k] = __shfl_sync(full, A[k], from, 8);
+        b = __shfl_sync(full, b, from, 8);
+        const double f = A[c] / __shfl_sync(full, A[c], c, 8);
+        const bool below = r8 > c && r8 < n;
+#pragma unroll
+        for (int k = c + 1; k < 8; ++k) {
+            const double pk = __shfl_sync(full, A[k], c, 8);
+            const double up = fma(-f, pk, A[k]);
+            A[k] = below && k < n ? up : A[k];
         }
+        const double pb = __shfl_sync(full, b, c, 8);
+        const double ub = fma(-f, pb, b);
+        b = below ? ub : b;
     }
-    for (int r = n - 1; r >= 0; --r) {
-        double s = b[r];
-        for (int k = r + 1; k < n; ++k) s -= A[r * 8 + k] * x[k];
-        x[r] = s / A[r * 8 + r];
+#pragma unroll
+    for (int r = 7; r >= 0; --r) {
+        x[r] = 0.0;
+        if (r >= n) continue;
+        double s = b;
+#pragma unroll
+        for (int k = r + 1; k < 8; ++k)
+        {
+            const double us = fma(-A[k], x[k], s);
+            s = k < n ? us : s;
+        }
+        x[r] = __shfl_sync(full, s / A[r], r, 8);
     }
-    return true;
+    return ok;
 }
 
-// pixel model from the normalised solution: H = Dinv Hn S, scaled to H[8] = 1
-__device__ bool to_pixels(const double* h, bool proj, const Frames& F, double* H) {
-    const double Hn[9] = {h[0], h[1], h[2], h[3], h[4], h[5], proj ? h[6] : 0.0, proj ? h[7] : 0.0, 1.0};
-    const double S[9] = {F.s[0], 0.0, -F.s[0] * F.s[1], 0.0, F.s[0], -F.s[0] * F.s[2], 0.0, 0.0, 1.0};
-    const double Di[9] = {1.0 / F.d[0], 0.0, F.d[1], 0.0, 1.0 / F.d[0], F.d[2], 0.0, 0.0, 1.0};
-    double M[9], R[9];
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            double s = 0.0;
-            for (int k = 0; k < 3; ++k) s += Hn[i * 3 + k] * S[k * 3 + j];
-            M[i * 3 + j] = s;
-        }
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            double s = 0.0;
-            for (int k = 0; k < 3; ++k) s += Di[i * 3 + k] * M[k * 3 + j];
-            R[i * 3 + j] = s;
-        }
-    if (fabs(R[8]) < 1e-300) return false;
-    for (int i = 0; i < 9; ++i) H[i] = R[i] / R[8];
-    return true;
+// Pixel model from the normalised solution (the same in every lane of a group
+// of 8): H = Dinv Hn S, scaled to H[8] = 1, with the zeros of Dinv and S left
+// out.  *out receives entry (lane mod 8), *last H[8] (1, or NaN where the
+// scale is not finite); false when the scale vanishes.
+__device__ __forceinline__ bool to_pixels(const double (&h)[8], bool proj, const Frames& F, double* out,
+                                          double* last) {
+    const double h6 = proj ? h[6] : 0.0, h7 = proj ? h[7] : 0.0;
+    const double tx = -F.s[0] * F.s[1], ty = -F.s[0] * F.s[2], di = 1.0 / F.d[0];
+    const double M0[3] = {h[0] * F.s[0], h[1] * F.s[0], fma(h[1], ty, h[0] * tx) + h[2]};
+    const double M1[3] = {h[3] * F.s[0], h[4] * F.s[0], fma(h[4], ty, h[3] * tx) + h[5]};
+    const double M2[3] = {h6 * F.s[0], h7 * F.s[0], fma(h7, ty, h6 * tx) + 1.0};
+    const int e = threadIdx.x & 7;
+    double mine = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        if (e == j) mine = fma(F.d[1], M2[j], di * M0[j]);
+        if (e == 3 + j) mine = fma(F.d[2], M2[j], di * M1[j]);
+        if (j < 2 && e == 6 + j) mine = M2[j];
+    }
+    *out = mine / M2[2];
+    *last = isfinite(M2[2]) ? 1.0 : NAN;
+    return !(fabs(M2[2]) < 1e-300);
 }
 
 __device__ __forceinline__ bool inlier(const double* H, const double* src, const double* dst, int i, double t2) {
@@ -162,93 +225,242 @@ __device__ __forceinline__ bool inlier(const double* H, const double* src, const
     return ex * ex + ey * ey <= t2;
 }
 
-// One warp (CTA) per kHpw hypotheses: lane l < kHpw solves hypothesis
-// h0 + l, then the warp counts inliers for each of the models in turn.
-__global__ void __launch_bounds__(32)
-    k_ransac_hyp(const double* __restrict__ src, const double* __restrict__ dst, const uint8_t* __restrict__ valid,
-                 int n, int proj, const int32_t* __restrict__ samples, int n_hyp, double t2,
-                 const Frames* __restrict__ frames, int32_t* __restrict__ scores, double* __restrict__ models) {
-    __shared__ double sH[kHpw][9];
-    __shared__ int sok[kHpw];
-    const int lane = threadIdx.x & 31;
-    const int h0 = blockIdx.x * kHpw;
+// The minimal systems, a group of 8 lanes per hypothesis (lane r: equation r,
+// point r / 2 of the sample).  A singular sample or an index outside [0, n)
+// marks its hypothesis with score -1 and a zero model.
+__global__ void __launch_bounds__(kSolveThreads)
+    k_ransac_solve(const double* __restrict__ src, const double* __restrict__ dst, int n, int proj,
+                   const int32_t* __restrict__ samples, int n_hyp, const Frames* __restrict__ frames,
+                   int32_t* __restrict__ scores, double* __restrict__ models) {
     const bool pj = proj != 0;
-    const int k = pj ? 4 : 3, nu = pj ? 8 : 6;
-    if (lane < kHpw) {
-        const int h = h0 + lane;
-        bool ok = false;
-        if (h < n_hyp) {
-            const Frames F = *frames;
-            double A[64], b[8], x[8], r1[8], r2[8];
-            bool in_range = true;
-            for (int j = 0; j < k; ++j) {
-                const int i0 = samples[(size_t)h * k + j];
-                in_range = in_range && i0 >= 0 && i0 < n;
-                const int i = (i0 >= 0 && i0 < n) ? i0 : 0;  // an index outside [0, n) voids the hypothesis
-                const double sx = F.s[0] * (src[2 * i] - F.s[1]), sy = F.s[0] * (src[2 * i + 1] - F.s[2]);
-                const double dx = F.d[0] * (dst[2 * i] - F.d[1]), dy = F.d[0] * (dst[2 * i + 1] - F.d[2]);
-                eq_rows(pj, sx, sy, dx, dy, r1, r2);
-                for (int c = 0; c < nu; ++c) {
-                    A[(2 * j) * 8 + c] = r1[c];
-                    A[(2 * j + 1) * 8 + c] = r2[c];
-                }
-                b[2 * j] = dx;
-                b[2 * j + 1] = dy;
-            }
-            ok = in_range && solve_small(A, b, nu, x) && to_pixels(x, pj, F, sH[lane]);
-        }
-        sok[lane] = ok ? 1 : 0;
+    const int K = pj ? 4 : 3, nu = pj ? 8 : 6;
+    const int h = blockIdx.x * (kSolveThreads / 8) + (threadIdx.x >> 3), r8 = threadIdx.x & 7;
+    const bool on = h < n_hyp && r8 < nu;
+    const Frames F = *frames;
+    const int i0 = on ? samples[(size_t)h * K + (r8 >> 1)] : 0;
+    const bool in = i0 >= 0 && i0 < n;
+    double sx = 0.0, sy = 0.0, dx = 0.0, dy = 0.0;
+    if (on && in) {  // an index outside [0, n) voids the hypothesis
+        sx = F.s[0] * (src[2 * i0] - F.s[1]);
+        sy = F.s[0] * (src[2 * i0 + 1] - F.s[2]);
+        dx = F.d[0] * (dst[2 * i0] - F.d[1]);
+        dy = F.d[0] * (dst[2 * i0 + 1] - F.d[2]);
     }
-    __syncwarp();
-    const int nh = n_hyp - h0 < kHpw ? n_hyp - h0 : kHpw;
-    for (int q = 0; q < nh; ++q) {
-        int c = 0;
-        if (sok[q]) {
-            double H[9];
+    const bool in_range = (__ballot_sync(0xffffffffu, on && !in) >> (threadIdx.x & 24) & 255u) == 0;
+    double r1[8], r2[8], A[8], x[8], e, e8;
+    eq_rows(pj, sx, sy, dx, dy, r1, r2);
 #pragma unroll
-            for (int r = 0; r < 9; ++r) H[r] = sH[q][r];
-            for (int i = lane; i < n; i += 32) c += (is_valid(valid, i) && inlier(H, src, dst, i, t2)) ? 1 : 0;
+    for (int c = 0; c < 8; ++c) A[c] = on ? ((r8 & 1) ? r2[c] : r1[c]) : 0.0;
+    bool ok = solve_group(A, (r8 & 1) ? dy : dx, nu, x);
+    ok = to_pixels(x, pj, F, &e, &e8) && ok && in_range;
+    if (h < n_hyp) {
+        models[(size_t)h * 9 + r8] = ok ? e : 0.0;
+        if (r8 == 0) {
+            models[(size_t)h * 9 + 8] = ok ? e8 : 0.0;
+            scores[h] = ok ? 0 : -1;
         }
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-        if (lane == 0) scores[h0 + q] = sok[q] ? c : -1;
     }
-    if (lane < nh)
-        for (int r = 0; r < 9; ++r) models[(size_t)(h0 + lane) * 9 + r] = sok[lane] ? sH[lane][r] : 0.0;
+}
+
+// FP32 decision of the inlier test with an error bound.  A model's FP32 copy
+// and the largest |x|, |y|, |x'|, |y'| of the staged points bound the error of
+// the mapped position: with u = 2^-24, the numerators and the denominator w
+// are within en = 6u (|h0| X + |h1| Y + |h2|) and ew of their exact values,
+// so a mapped coordinate is within B = |1/w| (en + m ew) + 8u (m + D) of its
+// own (m the larger mapped coordinate, D the largest destination coordinate)
+// and the distance to the destination within 2B.  Distances outside the
+// threshold -+ 2B are decided; a distance inside, or anything not finite,
+// takes the FP64 test, so every decision is the FP64 one.
+struct ModelF {
+    float h[9];
+    float en, ew;
+};
+struct PointF {
+    float x, y, dx, dy;
+};
+constexpr float kU6 = 6.f * 5.9604645e-8f, kU8 = 8.f * 5.9604645e-8f;
+
+__device__ __forceinline__ ModelF model_f(const double* H, float X, float Y) {
+    ModelF m;
+#pragma unroll
+    for (int r = 0; r < 9; ++r) m.h[r] = (float)H[r];
+    m.en = kU6 * 1.01f * fmaxf(fabsf(m.h[0]) * X + fabsf(m.h[1]) * Y + fabsf(m.h[2]),
+                               fabsf(m.h[3]) * X + fabsf(m.h[4]) * Y + fabsf(m.h[5]));
+    m.ew = kU6 * 1.01f * (fabsf(m.h[6]) * X + fabsf(m.h[7]) * Y + fabsf(m.h[8]));
+    return m;
+}
+
+// 1: inlier, 0: not, -1: undecided.  T: the threshold (at most kMaxFastT).
+constexpr float kMaxFastT = 1e6f;
+__device__ __forceinline__ int inlier_f(const ModelF& m, const PointF& p, float D, float T) {
+    const float w = fmaf(m.h[6], p.x, fmaf(m.h[7], p.y, m.h[8]));
+    const float r = 1.f / w;
+    const float px = fmaf(m.h[0], p.x, fmaf(m.h[1], p.y, m.h[2])) * r;
+    const float py = fmaf(m.h[3], p.x, fmaf(m.h[4], p.y, m.h[5])) * r;
+    const float ex = px - p.dx, ey = py - p.dy;
+    const float d2 = fmaf(ex, ex, ey * ey);
+    const float mm = fmaxf(fabsf(px), fabsf(py));
+    // the error of w may not reach a tenth of it, so that 1/w is good to first order
+    const float B2 = 2.4f * fmaf(fabsf(r), fmaf(mm, m.ew, m.en), kU8 * (mm + D));
+    const float hi = T + B2, lo = T - B2;
+    if (!(m.ew < 0.1f * fabsf(w))) return -1;
+    if (d2 * 0.999999f > hi * hi) return 0;
+    if (lo > 0.f && d2 * 1.000001f < lo * lo) return 1;
+    return -1;
+}
+
+// Inlier counts: one warp per two of the CTA's kScoreHyps models, the points
+// staged as FP32 once per CTA.  4096 hypotheses over 1000 points are 4.1M
+// tests of ~45 FP32 instructions; with FP64 (two divisions a test) they took
+// most of the call.  The undecided tests (within ~0.01 px of the threshold)
+// are listed and taken together: one undecided lane would hold its warp for a
+// whole FP64 test (~3000 clocks).
+__global__ void __launch_bounds__(kRsThreads)
+    k_ransac_score(const double* __restrict__ src, const double* __restrict__ dst, const uint8_t* __restrict__ valid,
+                   int n, int n_hyp, double t2, float T, int32_t* __restrict__ scores,
+                   const double* __restrict__ models) {
+    constexpr int kWarps = kRsThreads / 32, kPer = kScoreHyps / kWarps;
+    __shared__ float4 s_p[kScorePts];  // x, y, x', y'; x' = +inf: not valid (decided as an outlier)
+    __shared__ float s_mx[kWarps][3];
+    __shared__ unsigned s_undec[kScoreList];  // undecided tests: model * kScorePts + point
+    __shared__ int s_nu, s_extra[kScoreHyps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x < kScoreHyps) s_extra[threadIdx.x] = 0;
+    int cnt[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) cnt[q] = 0;
+    for (int i0 = 0; i0 < n; i0 += kScorePts) {
+        const int np = min(kScorePts, n - i0);
+        float X = 0.f, Y = 0.f, D = 0.f;
+        __syncthreads();  // the previous points are done with
+        if (threadIdx.x == 0) s_nu = 0;
+        for (int i = threadIdx.x; i < np; i += kRsThreads) {
+            const bool v = is_valid(valid, i0 + i);
+            const double* a = src + 2 * (size_t)(i0 + i);
+            const double* b = dst + 2 * (size_t)(i0 + i);
+            const float4 p = v ? make_float4((float)a[0], (float)a[1], (float)b[0], (float)b[1])
+                               : make_float4(0.f, 0.f, INFINITY, 0.f);
+            s_p[i] = p;
+            if (v) {
+                X = fmaxf(X, fabsf(p.x));
+                Y = fmaxf(Y, fabsf(p.y));
+                D = fmaxf(D, fmaxf(fabsf(p.z), fabsf(p.w)));
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            X = fmaxf(X, __shfl_xor_sync(0xffffffffu, X, o));
+            Y = fmaxf(Y, __shfl_xor_sync(0xffffffffu, Y, o));
+            D = fmaxf(D, __shfl_xor_sync(0xffffffffu, D, o));
+        }
+        if (lane == 0) {
+            s_mx[w][0] = X;
+            s_mx[w][1] = Y;
+            s_mx[w][2] = D;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kWarps; ++q) {
+            X = fmaxf(X, s_mx[q][0]);
+            Y = fmaxf(Y, s_mx[q][1]);
+            D = fmaxf(D, s_mx[q][2]);
+        }
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int h = blockIdx.x * kScoreHyps + w * kPer + q;
+            if (h >= n_hyp || scores[h] < 0) continue;
+            const double* Hg = models + (size_t)h * 9;
+            const ModelF m = model_f(Hg, X, Y);
+            // four points at a time, so that their divisions overlap
+            for (int i4 = lane; i4 < np; i4 += 4 * 32) {
+                int in[4];
+                bool und = false;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int i = i4 + 32 * u;
+                    const float4 p = s_p[i < np ? i : 0];
+                    in[u] = i < np ? inlier_f(m, PointF{p.x, p.y, p.z, p.w}, D, T) : 0;
+                    und = und || in[u] < 0;
+                    cnt[q] += max(in[u], 0);
+                }
+                if (!und) continue;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (in[u] >= 0) continue;
+                    const int i = i4 + 32 * u, at = atomicAdd(&s_nu, 1);
+                    if (at < kScoreList) s_undec[at] = (unsigned)((w * kPer + q) * kScorePts + i);
+                    else cnt[q] += is_valid(valid, i0 + i) && inlier(Hg, src, dst, i0 + i, t2) ? 1 : 0;
+                }
+            }
+        }
+        __syncthreads();
+        const int nu = min(s_nu, kScoreList);
+        for (int u = threadIdx.x; u < nu; u += kRsThreads) {
+            const int q = (int)(s_undec[u] / kScorePts), i = i0 + (int)(s_undec[u] % kScorePts);
+            if (is_valid(valid, i) && inlier(models + (size_t)(blockIdx.x * kScoreHyps + q) * 9, src, dst, i, t2))
+                atomicAdd(&s_extra[q], 1);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int h = blockIdx.x * kScoreHyps + w * kPer + q;
+        int c = cnt[q];
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
+        if (lane == 0 && h < n_hyp && scores[h] >= 0) scores[h] = c + s_extra[w * kPer + q];
+    }
 }
 
 constexpr int kNE = 44;  // unique entries of the 8 x 8 normal matrix (36) and the right side (8)
 
-__global__ void __launch_bounds__(kRsThreads)
+// One cluster of kRsCtas CTAs, the points strided over them: a single SM's
+// FP64 unit held the recounts and the normal equations for longer than the
+// scoring of every hypothesis takes.  Each thread's 44 sums go through shared
+// memory (a shuffle tree would run its FP64 adds with idle lanes), then over
+// the CTAs in order; warp 0 of every CTA solves the same system.
+struct FinalSmem {
+    double e[kNE][kRsThreads + 1];
+    double tot[kNE];
+};
+
+__global__ void __cluster_dims__(kRsCtas, 1, 1) __launch_bounds__(kRsThreads)
     k_ransac_final(const double* __restrict__ src, const double* __restrict__ dst, const uint8_t* __restrict__ valid,
                    int n, int proj, int n_hyp, double t2, int refits, const Frames* __restrict__ frames,
                    const int32_t* __restrict__ scores, const double* __restrict__ models, double* __restrict__ H_out,
                    uint8_t* __restrict__ mask, int32_t* __restrict__ info) {
-    __shared__ int s_best, s_score[kRsThreads], s_idx[kRsThreads];
+    extern __shared__ __align__(16) char fin_sm[];
+    FinalSmem& S = *reinterpret_cast<FinalSmem*>(fin_sm);
+    __shared__ int s_best, s_score[kRsThreads / 32], s_idx[kRsThreads / 32];
     __shared__ double sH[9];
-    __shared__ double s_part[kRsThreads / 32][kNE];
     __shared__ int s_cnt[kRsThreads / 32];
+    __shared__ int s_total;  // this CTA's inlier count (read by the others)
     __shared__ int s_ok;
+    cg::cluster_group cl = cg::this_cluster();
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int first = (int)cl.block_rank() * kRsThreads + tid, step = kRsCtas * kRsThreads;
     const bool pj = proj != 0;
     const int k = pj ? 4 : 3, nu = pj ? 8 : 6;
-    // argmax: highest score, then lowest index
-    int bs = -2, bi = -1;
-    for (int h = tid; h < n_hyp; h += kRsThreads)
-        if (scores[h] > bs) {
-            bs = scores[h];
-            bi = h;
+    // argmax: highest score, then lowest index (every CTA over all of them)
+    auto take = [](int s, int i, int& bs, int& bi) {
+        if (i >= 0 && (bi < 0 || s > bs || (s == bs && i < bi))) {
+            bs = s;
+            bi = i;
         }
-    s_score[tid] = bs;
-    s_idx[tid] = bi;
+    };
+    int bs = -2, bi = -1;
+    for (int h = tid; h < n_hyp; h += kRsThreads) take(scores[h], h, bs, bi);
+    for (int o = 16; o > 0; o >>= 1) {
+        const int os = __shfl_down_sync(0xffffffffu, bs, o), oi = __shfl_down_sync(0xffffffffu, bi, o);
+        take(os, oi, bs, bi);
+    }
+    if (lane == 0) {
+        s_score[w] = bs;
+        s_idx[w] = bi;
+    }
     __syncthreads();
     if (tid == 0) {
-        int b = -1, v = -1;
-        for (int t = 0; t < kRsThreads; ++t)
-            if (s_idx[t] >= 0 && (s_score[t] > v || (s_score[t] == v && s_idx[t] < b))) {
-                v = s_score[t];
-                b = s_idx[t];
-            }
-        s_best = v >= 0 ? b : -1;  // every hypothesis singular: no winner
+        for (int t = 1; t < kRsThreads / 32; ++t) take(s_score[t], s_idx[t], bs, bi);
+        s_best = bi >= 0 && bs >= 0 ? bi : -1;  // every hypothesis singular: no winner
         for (int q = 0; q < 9; ++q) sH[q] = s_best >= 0 ? models[(size_t)s_best * 9 + q] : ((q % 4 == 0) ? 1.0 : 0.0);
     }
     __syncthreads();
@@ -257,28 +469,35 @@ __global__ void __launch_bounds__(kRsThreads)
         double H[9];
         for (int q = 0; q < 9; ++q) H[q] = sH[q];
         int c = 0;
-        for (int i = tid; i < n; i += kRsThreads) {
+        for (int i = first; i < n; i += step) {
             const bool in = best >= 0 && is_valid(valid, i) && inlier(H, src, dst, i, t2);
             mask[i] = in ? 1 : 0;
             c += in ? 1 : 0;
         }
         for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-        __syncthreads();
         if (lane == 0) s_cnt[w] = c;
         __syncthreads();
+        if (tid == 0) {
+            int t = 0;
+            for (int q = 0; q < kRsThreads / 32; ++q) t += s_cnt[q];
+            s_total = t;
+        }
+        cl.sync();
         int t = 0;
-        for (int q = 0; q < kRsThreads / 32; ++q) t += s_cnt[q];
-        __syncthreads();
+        for (unsigned r = 0; r < cl.num_blocks(); ++r) t += *cl.map_shared_rank(&s_total, r);
+        cl.sync();  // read by every CTA before the next count (or a CTA leaves)
         return t;
     };
     int cnt = recount();
     const Frames F = *frames;
+    const int rows = n - (int)cl.block_rank() * kRsThreads;  // threads of this CTA with a point
+    const int act = rows < 0 ? 0 : (rows < kRsThreads ? rows : kRsThreads);
     for (int it = 0; it < refits && best >= 0 && cnt >= k; ++it) {
         // normal equations over this thread's inliers (the mask it wrote itself)
         double e[kNE];
 #pragma unroll
         for (int q = 0; q < kNE; ++q) e[q] = 0.0;
-        for (int i = tid; i < n; i += kRsThreads) {
+        for (int i = first; i < n; i += step) {
             if (!mask[i]) continue;
             double r1[8], r2[8];
             const double sx = F.s[0] * (src[2 * i] - F.s[1]), sy = F.s[0] * (src[2 * i + 1] - F.s[2]);
@@ -288,42 +507,66 @@ __global__ void __launch_bounds__(kRsThreads)
 #pragma unroll
             for (int a = 0; a < 8; ++a)
 #pragma unroll
-                for (int c = a; c < 8; ++c) e[q++] += r1[a] * r1[c] + r2[a] * r2[c];
-#pragma unroll
-            for (int a = 0; a < 8; ++a) e[q++] += r1[a] * dx + r2[a] * dy;
-        }
-#pragma unroll
-        for (int q = 0; q < kNE; ++q) {
-            double v = e[q];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) s_part[w][q] = v;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double tot[kNE];
-            for (int q = 0; q < kNE; ++q) {
-                double v = 0.0;
-                for (int ww = 0; ww < kRsThreads / 32; ++ww) v += s_part[ww][q];
-                tot[q] = v;
-            }
-            double M[64], v[8], x[8], Hr[9];
-            int q = 0;
-            for (int a = 0; a < 8; ++a)
                 for (int c = a; c < 8; ++c) {
-                    M[a * 8 + c] = tot[q];
-                    M[c * 8 + a] = tot[q];
+                    // the zero entries of the two rows add nothing (columns 0-2 of
+                    // the second, 3-5 of the first)
+                    if (c < 3) e[q] += r1[a] * r1[c];
+                    else if (a < 3 && c < 6) e[q] += 0.0;
+                    else if (a < 3) e[q] += r1[a] * r1[c];
+                    else if (a < 6) e[q] += r2[a] * r2[c];
+                    else e[q] += r1[a] * r1[c] + r2[a] * r2[c];
                     ++q;
                 }
-            for (int a = 0; a < 8; ++a) v[a] = tot[q++];
-            s_ok = solve_small(M, v, nu, x) && to_pixels(x, pj, F, Hr);
-            if (s_ok)
-                for (int r = 0; r < 9; ++r) sH[r] = Hr[r];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) e[q++] += a < 3 ? r1[a] * dx : (a < 6 ? r2[a] * dy : r1[a] * dx + r2[a] * dy);
         }
+#pragma unroll
+        for (int q = 0; q < kNE; ++q) S.e[q][tid] = e[q];
         __syncthreads();
-        if (!s_ok) break;
+        {
+            // four threads per entry, a quarter of the rows each, then in order
+            const int q = tid >> 2, part = tid & 3;
+            double v = 0.0;
+            if (q < kNE)
+                for (int r = part * (kRsThreads / 4); r < min((part + 1) * (kRsThreads / 4), act); ++r) v += S.e[q][r];
+            const double v1 = __shfl_down_sync(0xffffffffu, v, 1), v2 = __shfl_down_sync(0xffffffffu, v, 2),
+                         v3 = __shfl_down_sync(0xffffffffu, v, 3);
+            if (q < kNE && part == 0) S.tot[q] = ((v + v1) + v2) + v3;
+        }
+        cl.sync();
+        if (w == 0) {
+            double tot[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int q = lane + 32 * u;
+                tot[u] = 0.0;
+                if (q < kNE)
+                    for (unsigned r = 0; r < cl.num_blocks(); ++r) tot[u] += cl.map_shared_rank(&S, r)->tot[q];
+            }
+            // lane r takes row r of the symmetric matrix (entry (a, c >= a) at a (17 - a) / 2 + c - a)
+            auto entry = [&](int q) {
+                const double lo = __shfl_sync(0xffffffffu, tot[0], q & 31), hi = __shfl_sync(0xffffffffu, tot[1], q & 31);
+                return q < 32 ? lo : hi;
+            };
+            const int r = lane & 7;
+            double M[8], x[8], mine, last;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int a = min(r, c), b = max(r, c);
+                M[c] = entry(a * (17 - a) / 2 + b - a);
+            }
+            const double rhs = entry(36 + r);
+            bool ok = solve_group(M, rhs, nu, x);
+            ok = to_pixels(x, pj, F, &mine, &last) && ok;
+            if (lane == 0) s_ok = ok;
+            if (ok && lane < 8) sH[lane] = mine;
+            if (ok && lane == 8) sH[8] = last;
+        }
+        cl.sync();  // S.tot read by every CTA; sH written
+        if (!s_ok) break;  // the same in every CTA
         cnt = recount();
     }
-    if (tid == 0) {
+    if (first == 0) {
         for (int q = 0; q < 9; ++q) H_out[q] = sH[q];
         info[0] = best;
         info[1] = best >= 0 ? cnt : 0;
@@ -402,15 +645,23 @@ cudaError_t launch_ransac(const double* src, const double* dst, const uint8_t* v
     p += (sizeof(int32_t) * (size_t)n_hyp + 255) / 256 * 256;
     double* models = reinterpret_cast<double*>(p);
     const double t2 = threshold * threshold;
-    k_ransac_frames<<<1, kRsThreads, 0, st>>>(src, dst, valid, n, frames);
+    // the FP32 decision serves thresholds well inside its range; beyond, T = NaN
+    // leaves every point undecided and the FP64 test decides
+    const float T = threshold <= (double)kMaxFastT ? (float)threshold : NAN;
+    k_ransac_frames<<<kRsCtas, kRsThreads, 0, st>>>(src, dst, valid, n, frames);
     int nl = 1;
     if (n_hyp > 0) {
-        k_ransac_hyp<<<(n_hyp + kHpw - 1) / kHpw, 32, 0, st>>>(src, dst, valid, n, proj, samples, n_hyp, t2, frames,
-                                                                scores, models);
-        ++nl;
+        const int sb = (n_hyp + kSolveThreads / 8 - 1) / (kSolveThreads / 8);
+        k_ransac_solve<<<sb, kSolveThreads, 0, st>>>(src, dst, n, proj, samples, n_hyp, frames, scores, models);
+        k_ransac_score<<<(n_hyp + kScoreHyps - 1) / kScoreHyps, kRsThreads, 0, st>>>(src, dst, valid, n, n_hyp, t2, T,
+                                                                                     scores, models);
+        nl += 2;
     }
-    k_ransac_final<<<1, kRsThreads, 0, st>>>(src, dst, valid, n, proj, n_hyp, t2, refits, frames, scores, models,
-                                             H_out, mask, info);
+    const int smem = (int)sizeof(FinalSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_ransac_final, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_ransac_final<<<kRsCtas, kRsThreads, smem, st>>>(src, dst, valid, n, proj, n_hyp, t2, refits, frames, scores,
+                                                      models, H_out, mask, info);
     ++nl;
     if (launches) *launches = nl;
     return cudaGetLastError();
