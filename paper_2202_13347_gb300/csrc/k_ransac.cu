@@ -574,45 +574,197 @@ __global__ void __cluster_dims__(kRsCtas, 1, 1) __launch_bounds__(kRsThreads)
 }
 
 // Rectification (Sec. 3.2.3): out(x, y) = bilinear sample of the sensed
-// image at H^-1 (x, y); outside [0, W-1] x [0, H-1] the fill value.  The
-// mapping is FP64 (coordinates of 10^4 px keep their sub-pixel part), the
-// blend FP32.  Each CTA inverts H (the adjugate scaled by its last entry);
-// a singular model gives an all-fill image.
-__global__ void k_rectify(const float* __restrict__ img, int H, int W, size_t pitch, const double* __restrict__ Hm,
-                          float fill, int out_h, int out_w, float* __restrict__ out) {
+// image at H^-1 (x, y); outside [0, W-1] x [0, H-1] the fill value.  Each CTA
+// inverts H (the adjugate scaled by its last entry); a singular model gives
+// an all-fill image.  The mapping is as good as FP64 (coordinates of 10^4 px
+// keep their sub-pixel part), the blend FP32.
+//
+// FP64 runs at two lanes per clock and SM, so the mapping of every pixel in
+// FP64 (~50 instructions) set the time: 2048 x 2048 took 349 us against 5 us
+// of HBM time.  Here a warp maps one pixel of its kRectW x kRectH tile in
+// FP64, (u0, t0) at (x0, y0), and steps from it exactly:
+//   u(x0 + i, y0 + k) = u0 + d / (1 + e),  d = i sx + k sy,  e = i qx + k qy,
+//   sx = (a - g u0) / w0, sy = (b - h u0) / w0, qx = g / w0, qy = h / w0
+// (a, b, g, h the model's x row and its last row).  The steps are kept as a
+// float whose product with i or k is exact plus a float remainder, and the
+// integer parts are split off before the fractions are added, so a position
+// is within ~2^-23 px of the FP64 one wherever it lies (FP32 rounds the
+// fraction to 2^-25 in either form).  Tiles with a strong perspective or
+// scale, and pixels mapped within 2^-10 px of the image's border lines (where
+// a rounding could decide inside or outside), take the FP64 mapping itself.  2048 x 2048: 29 us.
+// The CTA's first warp prepares up to 32 tiles, one per lane (inverse, tile
+// maps: a chain of ~1500 clocks whose length does not depend on their
+// number), so large images give a warp four tiles (kRectTiles) and small ones
+// one, which keeps more CTAs.
+constexpr int kRectW = 32, kRectH = 8, kRectTiles = 4, kRectB = 4;
+struct RectTile {
+    int nu, nt;                 // integer parts of u0, t0
+    float fu, ft;               // fractions
+    float sx[2], sxl[2], sy[2], syl[2];  // per axis (u, t): steps, high part and remainder
+    float qx, qy;
+    int ok;                     // the steps serve the whole tile
+};
+
+// one pixel by the FP64 mapping
+__device__ __noinline__ float rect_fp64(const float* __restrict__ img, int H, int W, size_t pitch, const double* inv,
+                                        int ok, int x, int y, float fill) {
+    const double w = inv[6] * x + inv[7] * y + inv[8];
+    if (!ok || w == 0.0) return fill;
+    const double rw = 1.0 / w;
+    const double u = (inv[0] * x + inv[1] * y + inv[2]) * rw;
+    const double t = (inv[3] * x + inv[4] * y + inv[5]) * rw;
+    if (!(u >= 0.0 && t >= 0.0 && u <= W - 1 && t <= H - 1)) return fill;
+    const int u0 = min((int)floor(u), max(W - 2, 0)), t0 = min((int)floor(t), max(H - 2, 0));
+    const int u1 = min(u0 + 1, W - 1), t1 = min(t0 + 1, H - 1);
+    const float fu = (float)(u - u0), ft = (float)(t - t0);
+    const float p00 = img[(size_t)t0 * pitch + u0], p01 = img[(size_t)t0 * pitch + u1];
+    const float p10 = img[(size_t)t1 * pitch + u0], p11 = img[(size_t)t1 * pitch + u1];
+    const float r0 = fmaf(fu, p01 - p00, p00), r1 = fmaf(fu, p11 - p10, p10);
+    return fmaf(ft, r1 - r0, r0);
+}
+
+__global__ void __launch_bounds__(kRsThreads, 4)
+    k_rectify(const float* __restrict__ img, int H, int W, size_t pitch, const double* __restrict__ Hm, float fill,
+              int out_h, int out_w, float* __restrict__ out, int per_warp) {
+    constexpr int kWarps = kRsThreads / 32;
     __shared__ double s_inv[9];
     __shared__ int s_ok;
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        const double a = Hm[0], b = Hm[1], c = Hm[2], d = Hm[3], e = Hm[4], f = Hm[5], g = Hm[6], h = Hm[7],
-                     i = Hm[8];
-        double inv[9] = {e * i - f * h, c * h - b * i, b * f - c * e, f * g - d * i, a * i - c * g,
-                         c * d - a * f, d * h - e * g, b * g - a * h, a * e - b * d};
-        const double det = a * inv[0] + b * inv[3] + c * inv[6];
-        s_ok = det != 0.0 && inv[8] != 0.0;
-        for (int k = 0; k < 9; ++k) s_inv[k] = s_ok ? inv[k] / inv[8] : 0.0;
-    }
-    __syncthreads();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= out_w || y >= out_h) return;
-    float v = fill;
-    const double w = s_inv[6] * x + s_inv[7] * y + s_inv[8];
-    if (s_ok && w != 0.0) {
-        const double rw = 1.0 / w;  // one division per pixel (FP64 is slow on this part)
-        const double u = (s_inv[0] * x + s_inv[1] * y + s_inv[2]) * rw;
-        const double t = (s_inv[3] * x + s_inv[4] * y + s_inv[5]) * rw;
-        if (u >= 0.0 && t >= 0.0 && u <= W - 1 && t <= H - 1) {
-            int u0 = (int)floor(u), t0 = (int)floor(t);
-            u0 = min(u0, max(W - 2, 0));
-            t0 = min(t0, max(H - 2, 0));
-            const int u1 = min(u0 + 1, W - 1), t1 = min(t0 + 1, H - 1);
-            const float fu = (float)(u - u0), ft = (float)(t - t0);
-            const float p00 = img[(size_t)t0 * pitch + u0], p01 = img[(size_t)t0 * pitch + u1];
-            const float p10 = img[(size_t)t1 * pitch + u0], p11 = img[(size_t)t1 * pitch + u1];
-            const float r0 = fmaf(fu, p01 - p00, p00), r1 = fmaf(fu, p11 - p10, p10);
-            v = fmaf(ft, r1 - r0, r0);
+    __shared__ RectTile s_tile[kWarps * kRectTiles];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // tile t of the CTA (t < kWarps * per_warp): column block t / kWarps, row block t % kWarps
+    const int xb = blockIdx.x * kRectW * per_warp, yb = blockIdx.y * (kRectH * kWarps);
+    // a warp's FP64 instruction holds its sub-partition's FP64 unit for 64
+    // clocks: neighbouring CTAs use different warps for this
+    if (warp == (int)((blockIdx.x + blockIdx.y) & (kWarps - 1))) {
+        {
+            const double a = Hm[0], b = Hm[1], c = Hm[2], d = Hm[3], e = Hm[4], f = Hm[5], g = Hm[6], h = Hm[7],
+                         i = Hm[8];
+            const double inv[9] = {e * i - f * h, c * h - b * i, b * f - c * e, f * g - d * i, a * i - c * g,
+                                   c * d - a * f, d * h - e * g, b * g - a * h, a * e - b * d};
+            const double det = a * inv[0] + b * inv[3] + c * inv[6];
+            const bool ok = det != 0.0 && inv[8] != 0.0;
+            double mine = inv[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (lane == k) mine = inv[k];
+            if (lane < 9) s_inv[lane] = ok ? mine / inv[8] : 0.0;
+            if (lane == 0) s_ok = ok;
+        }
+        __syncwarp();
+        if (lane < kWarps * per_warp) {  // lane t: tile t
+            RectTile T;
+            const double x = xb + (lane / kWarps) * kRectW, y = yb + (lane % kWarps) * kRectH;
+            const double w = s_inv[6] * x + s_inv[7] * y + s_inv[8];
+            const double rw = 1.0 / w;
+            const double p[2] = {(s_inv[0] * x + s_inv[1] * y + s_inv[2]) * rw,
+                                 (s_inv[3] * x + s_inv[4] * y + s_inv[5]) * rw};
+            const double qx = s_inv[6] * rw, qy = s_inv[7] * rw;
+            bool ok = s_ok && fabs(p[0]) < 1e8 && fabs(p[1]) < 1e8 &&
+                      fabs(qx) * kRectW + fabs(qy) * kRectH < 1.0 / 1024;
+            const double n0 = floor(p[0]), n1 = floor(p[1]);
+            T.fu = (float)(p[0] - n0);
+            T.ft = (float)(p[1] - n1);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const double sx = (s_inv[3 * q] - s_inv[6] * p[q]) * rw, sy = (s_inv[3 * q + 1] - s_inv[7] * p[q]) * rw;
+                ok = ok && fabs(sx) < 4.0 && fabs(sy) < 4.0;
+                // 19 (21) significant bits: the product with i < 32 (k < 8) is exact
+                T.sx[q] = __uint_as_float(__float_as_uint((float)sx) & 0xffffffe0u);
+                T.sy[q] = __uint_as_float(__float_as_uint((float)sy) & 0xfffffff8u);
+                T.sxl[q] = (float)(sx - (double)T.sx[q]);
+                T.syl[q] = (float)(sy - (double)T.sy[q]);
+            }
+            T.qx = (float)qx;
+            T.qy = (float)qy;
+            T.ok = ok;
+            T.nu = ok ? (int)n0 : 0;
+            T.nt = ok ? (int)n1 : 0;
+            s_tile[lane] = T;
         }
     }
-    out[(size_t)y * out_w + x] = v;
+    __syncthreads();
+    for (int xt = 0; xt < per_warp; ++xt) {
+    const int x = xb + xt * kRectW + lane, y0 = yb + warp * kRectH;
+    if (x >= out_w) break;
+    const RectTile T = s_tile[xt * kWarps + warp];
+    const float fi = (float)lane;
+    // the column part of the steps: d = i sx split into integer and fraction
+    float ipx[2], fpx[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const float p = fi * T.sx[q];
+        ipx[q] = floorf(p);
+        fpx[q] = p - ipx[q];
+    }
+    // kRectB rows at a time: their positions, then all their samples in flight,
+    // then the blends (with one row after the other the kernel waited for every
+    // row's samples: 60 us)
+#pragma unroll 1
+    for (int kb = 0; kb < kRectH; kb += kRectB) {
+        size_t at[kRectB];
+        float fu[kRectB], ft[kRectB];
+        bool ld[kRectB], fp64[kRectB];
+        bool any64 = false;
+#pragma unroll
+        for (int b = 0; b < kRectB; ++b) {
+            const float fk = (float)(kb + b);
+            const float e0 = fmaf(fi, T.qx, fk * T.qy);
+            const float e = e0 * (1.f - e0 * (1.f - e0));  // e0 / (1 + e0), e0 < 2^-10
+            int ci[2];
+            float fr[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float p = fk * T.sy[q];
+                const float ip = floorf(p), fp = p - ip;
+                // remainders of the steps, and the perspective term
+                const float corr = fmaf(-e, fmaf(fi, T.sx[q], p), fmaf(fi, T.sxl[q], fk * T.syl[q]));
+                const float f = (q ? T.ft : T.fu) + ((fpx[q] + fp) + corr);
+                const float c = floorf(f);
+                fr[q] = f - c;
+                ci[q] = (q ? T.nt : T.nu) + (int)(ipx[q] + ip + c);
+            }
+            // inside, outside, or within 2^-10 px of the image's border lines, where
+            // the FP64 mapping decides
+            ld[b] = T.ok;
+            fp64[b] = !T.ok;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int last = (q ? H : W) - 1;
+                constexpr float eps = 1.f / 1024;
+                fp64[b] = fp64[b] || (fr[q] < eps && (ci[q] == 0 || ci[q] == last)) ||
+                          (fr[q] > 1.f - eps && (ci[q] == -1 || ci[q] == last - 1));
+                ld[b] = ld[b] && ci[q] >= 0 && ci[q] < last;
+            }
+            any64 = any64 || fp64[b];
+            at[b] = ld[b] ? (size_t)ci[1] * pitch + ci[0] : 0;
+            fu[b] = fr[0];
+            ft[b] = fr[1];
+        }
+        float p00[kRectB], p01[kRectB], p10[kRectB], p11[kRectB];
+#pragma unroll
+        for (int b = 0; b < kRectB; ++b) {
+            p00[b] = ld[b] ? img[at[b]] : 0.f;
+            p01[b] = ld[b] ? img[at[b] + 1] : 0.f;
+            p10[b] = ld[b] ? img[at[b] + pitch] : 0.f;
+            p11[b] = ld[b] ? img[at[b] + pitch + 1] : 0.f;
+        }
+#pragma unroll
+        for (int b = 0; b < kRectB; ++b) {
+            const int y = y0 + kb + b;
+            const float r0 = fmaf(fu[b], p01[b] - p00[b], p00[b]), r1 = fmaf(fu[b], p11[b] - p10[b], p10[b]);
+            if (y < out_h) out[(size_t)y * out_w + x] = ld[b] ? fmaf(ft[b], r1 - r0, r0) : fill;
+        }
+        if (any64) {
+            for (int b = 0; b < kRectB; ++b) {
+                const int y = y0 + kb + b;
+                bool mine = false;
+#pragma unroll
+                for (int u = 0; u < kRectB; ++u) mine = mine || (u == b && fp64[u]);
+                if (mine && y < out_h) out[(size_t)y * out_w + x] = rect_fp64(img, H, W, pitch, s_inv, s_ok, x, y, fill);
+            }
+        }
+    }
+    }
 }
 
 __global__ void k_results_to_points(const int32_t* __restrict__ pts, const fastncc_result* __restrict__ res, int n,
@@ -669,8 +821,12 @@ cudaError_t launch_ransac(const double* src, const double* dst, const uint8_t* v
 
 cudaError_t launch_rectify(const float* img, int H, int W, size_t pitch, const double* Hm, float fill, int out_h,
                            int out_w, float* out, cudaStream_t st) {
-    dim3 blk(32, 8), grid((unsigned)((out_w + 31) / 32), (unsigned)((out_h + 7) / 8));
-    k_rectify<<<grid, blk, 0, st>>>(img, H, W, pitch, Hm, fill, out_h, out_w, out);
+    constexpr int rows = kRectH * (kRsThreads / 32);
+    const unsigned gy = (unsigned)((out_h + rows - 1) / rows);
+    // four tiles a warp once that still leaves two CTAs per SM
+    const int per = (size_t)gy * ((out_w + kRectTiles * kRectW - 1) / (kRectTiles * kRectW)) >= 2 * 152 ? kRectTiles : 1;
+    dim3 grid((unsigned)((out_w + per * kRectW - 1) / (per * kRectW)), gy);
+    k_rectify<<<grid, kRsThreads, 0, st>>>(img, H, W, pitch, Hm, fill, out_h, out_w, out, per);
     return cudaGetLastError();
 }
 
