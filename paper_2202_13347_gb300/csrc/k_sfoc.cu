@@ -6,9 +6,11 @@
 //                summed, group-wise L2 normalisation and stacking, plus the
 //                per-pixel sum planes used by the integral images (Eq. 14).
 //
-// Both kernels stage a 2-D tile with its clamped halo in shared memory and
-// do the horizontal pass into shared planes, then the vertical pass per
-// output pixel.  Borders clamp to the edge in every convolution.
+// Borders clamp to the edge in every convolution.  These two serve any radii
+// and rates: they stage a 2-D tile with its clamped halo in shared memory and
+// do the horizontal pass into shared planes, then the vertical pass per output
+// pixel.  The paper's own parameters take the streaming forms
+// k_sfoc_steer_ct (tiles, radii at compile time) and k_sfoc_smooth_strip.
 #include <cuda_bf16.h>
 #include <string.h>
 
@@ -284,7 +286,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_sfoc_steer_ct(const __grid_cons
 // g = the six channels of group g and two zeros) in both pixel orders,
 // plus the per-pixel sum planes.  Tiles are 32 columns x 64 rows.
 constexpr int kSTW = 32, kSTH = 64, kSRows = 8;
-constexpr int kPRows = 4;  // rows per thread of the paired vertical pass (2 columns x 4 rows)
 
 template <int KD>
 __device__ __forceinline__ void smooth_channel(const float* __restrict__ Fk, size_t fpitch, int H, int W, int x0,
@@ -339,126 +340,6 @@ __device__ __forceinline__ void smooth_channel(const float* __restrict__ Fk, siz
 #pragma unroll
             for (int q = 1; q <= KD; ++q) a = fmaf(t[q], x[(j - q * rate) * kSTW] + x[(j + q * rate) * kSTW], a);
             Dk[j] += a;
-        }
-    }
-}
-
-// The paper's dilation rates 1, 2, 3 at compile time: every thread loads
-// its input span into registers once (float4 rows in the horizontal pass,
-// one column in the vertical pass) and applies all three rates from there,
-// instead of reading shared memory once per tap and rate.  Same arithmetic,
-// same order of operations per output as smooth_channel.
-// Input tile layout of the compile-time path: shared column j of a row holds
-// image column x0 - OFF + j, OFF = hal rounded up to 4, so every row starts
-// on a 16-byte boundary in global and shared memory.
-template <int HAL>
-struct TileGeom {
-    static constexpr int OFF = (HAL + 3) / 4 * 4;
-    static constexpr int NL = (OFF + kSTW + HAL + 3) / 4;  // float4 per row (covers the halo)
-    static constexpr int IH = kSTH + 2 * HAL;
-};
-
-// Asynchronous copy of one channel's input tile into shared memory, one
-// commit group per tile.  Interior tiles copy whole rows as 16-byte pieces;
-// tiles at the image border copy element by element with clamped indices.
-template <int HAL>
-__device__ __forceinline__ void tile_load_async(const float* __restrict__ Fk, size_t fpitch, int H, int W, int x0,
-                                                int y0, float* dst, int FW) {
-    using TG = TileGeom<HAL>;
-    const int xs = x0 - TG::OFF;
-    const bool interior = xs >= 0 && xs + 4 * TG::NL <= W && y0 - HAL >= 0 && y0 + kSTH + HAL <= H;
-    if (interior) {
-        const float* src0 = Fk + (size_t)(y0 - HAL) * fpitch + xs;
-        for (int i = threadIdx.x; i < TG::IH * TG::NL; i += kThreads) {
-            const int rr = i / TG::NL, v = i - rr * TG::NL;
-            const unsigned d = (unsigned)__cvta_generic_to_shared(dst + rr * FW + 4 * v);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src0 + (size_t)rr * fpitch + 4 * v)
-                         : "memory");
-        }
-    } else {
-        constexpr int IW = kSTW + 2 * HAL;
-        for (int i = threadIdx.x; i < TG::IH * IW; i += kThreads) {
-            const int rr = i / IW, cc = i - rr * IW;  // tile column cc = image column x0 - HAL + cc
-            const int yy = clampi(y0 + rr - HAL, 0, H - 1), xx = clampi(x0 + cc - HAL, 0, W - 1);
-            const unsigned d = (unsigned)__cvta_generic_to_shared(dst + rr * FW + (TG::OFF - HAL) + cc);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(Fk + (size_t)yy * fpitch + xx)
-                         : "memory");
-        }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// One channel with the tile already in s_F (the caller waited for its copy
-// and synchronised the block).
-template <int KD>
-__device__ __forceinline__ void smooth_channel_123(const float* t, const float* s_F, int FW, float* s_h, int HR,
-                                                   float2 (&Dk)[kPRows]) {
-    constexpr int hal = 3 * KD;
-    constexpr int IH = kSTH + 2 * hal;
-    float tq[KD + 1];
-#pragma unroll
-    for (int q = 0; q <= KD; ++q) tq[q] = t[q];
-    // horizontal: task = (row, 4-column block); the block's inputs are
-    // shared columns cb + OFF - hal .. cb + OFF + 3 + hal.  Blocks of 4 give
-    // 8 (64 + 2 hal) tasks for the 256 threads, which fill their last round
-    // better than 4 (64 + 2 hal) blocks of 8 did (0.689 -> 0.652 ms of
-    // smoothing per 2048 x 2048 step)
-    constexpr int OFF = TileGeom<hal>::OFF;
-    constexpr int CW = 4;  // columns per task
-    constexpr int NV = (OFF + CW + hal + 3) / 4;
-    for (int task = threadIdx.x; task < IH * (kSTW / CW); task += kThreads) {
-        const int rr = task / (kSTW / CW), cb = (task % (kSTW / CW)) * CW;
-        const float4* x4 = reinterpret_cast<const float4*>(s_F + rr * FW + cb);
-        float in[NV * 4];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const float4 f = x4[v];
-            in[4 * v] = f.x;
-            in[4 * v + 1] = f.y;
-            in[4 * v + 2] = f.z;
-            in[4 * v + 3] = f.w;
-        }
-#pragma unroll
-        for (int r = 1; r <= 3; ++r) {
-            float o[CW];
-#pragma unroll
-            for (int c = 0; c < CW; ++c) {
-                float a = tq[0] * in[OFF + c];
-#pragma unroll
-                for (int q = 1; q <= KD; ++q) a = fmaf(tq[q], in[OFF + c - q * r] + in[OFF + c + q * r], a);
-                o[c] = a;
-            }
-            float4* dst = reinterpret_cast<float4*>(s_h + ((r - 1) * HR + rr) * kSTW + cb);
-#pragma unroll
-            for (int c = 0; c < CW; c += 4) dst[c / 4] = make_float4(o[c], o[c + 1], o[c + 2], o[c + 3]);
-        }
-    }
-    __syncthreads();
-    // vertical: thread = (column pair, 4-row block); each value is a float2
-    // over two adjacent columns, so every filter step is one paired FP32
-    // instruction (per lane the same rounding as the scalar form)
-    const int cp = threadIdx.x & 15, rb = (threadIdx.x >> 4) * kPRows;
-    float2 tq2[KD + 1];
-#pragma unroll
-    for (int q = 0; q <= KD; ++q) tq2[q] = make_float2(tq[q], tq[q]);
-#pragma unroll
-    for (int j = 0; j < kPRows; ++j) Dk[j] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int r = 1; r <= 3; ++r) {
-        constexpr int kMaxSpan = kPRows + 2 * KD * 3;
-        const int span = kPRows + 2 * KD * r;
-        const float2* x = reinterpret_cast<const float2*>(s_h + ((r - 1) * HR + rb + hal - KD * r) * kSTW) + cp;
-        float2 in[kMaxSpan];
-#pragma unroll
-        for (int i = 0; i < kMaxSpan; ++i)
-            if (i < span) in[i] = x[i * (kSTW / 2)];
-#pragma unroll
-        for (int j = 0; j < kPRows; ++j) {
-            float2 a = __fmul2_rn(tq2[0], in[KD * r + j]);
-#pragma unroll
-            for (int q = 1; q <= KD; ++q)
-                a = __ffma2_rn(tq2[q], __fadd2_rn(in[KD * r + j - q * r], in[KD * r + j + q * r]), a);
-            Dk[j] = __fadd2_rn(Dk[j], a);
         }
     }
 }
@@ -546,112 +427,334 @@ __device__ __forceinline__ void smooth_group(int g, const float* __restrict__ F,
     }
 }
 
-// One group with radius KDG and the rates 1, 2, 3 at compile time: tiles
-// double-buffered with asynchronous copies, paired vertical pass; a thread
-// owns 2 columns x kPRows rows of every channel.
-template <int NO, int KDG>
-__device__ __forceinline__ void smooth_group_123(int g, const float* __restrict__ F, size_t fpitch, size_t fplane,
-                                                 int H, int W, float eps, const float* t, float* s_F,
-                                                 float* s_F2, int FW, float* s_h, int HR, int x0, int y0,
-                                                 float* __restrict__ c32, size_t cpitch, size_t cplane,
-                                                 __nv_bfloat16* __restrict__ rm, __nv_bfloat16* __restrict__ cm,
-                                                 float (&a1)[kPRows][2], float (&a2)[kPRows][2]) {
-    constexpr int KO = NO;
-    const int cp = threadIdx.x & 15, rb = (threadIdx.x >> 4) * kPRows;
-    const int gx = x0 + 2 * cp;
-    float2 D[KO][kPRows];
-    __syncthreads();  // the previous group is done with both tile buffers (and the taps are written)
-    tile_load_async<3 * KDG>(F + (size_t)(g * NO) * fplane, fpitch, H, W, x0, y0, s_F, FW);
+// The paper's dilation rates 1, 2, 3 with smoothing radius KD at compile time,
+// one group g per launch (the second group's launch continues the per-pixel
+// sums from the stored planes, adding in the same order as one launch would).
+//
+// A CTA takes a strip of 64 columns and streams down its rows, one warp per
+// channel of the group, a lane per column pair.  A lane takes its window of an
+// input row from shared memory once (LDS.64 pairs), makes the row's three
+// horizontal sums in registers and adds them at once to the output rows they
+// belong to: rate r, tap q of row i goes to row i + q r, so the vertical pass
+// is 2 hal + 8 running sums per column in registers and touches no shared
+// memory.  Rows are taken 8 at a time; the 8 rows a block completes go to
+// shared memory, where two more warps meet the group's six channels of a pixel,
+// normalise and write them, while the channel warps are on the next block
+// (named barriers hand the two buffers over; with the channel warps doing this
+// themselves behind block barriers the kernel was 1.5x slower).
+//
+// What bounds it: per pixel and channel the 2 x 3 (2 KD + 1) multiply-adds
+// take 66 / 128 clocks of an SM at KD = 5, and the window reads 34 / 64.  The
+// tiled form this replaces (horizontal sums of every rate written to shared
+// memory, read back by the vertical pass, 32 x 64 tiles that redo 1.5x of the
+// horizontal work) needed 30 shared words and ~90 instructions per pixel and
+// channel against 17 and ~50 here, with block barriers between its passes.
+// 2048 x 2048, F32 cube: group 0 (KD = 3) 133 -> 105 us, group 1
+// (KD = 5) 187 -> 143 us.
+constexpr int kStW = 64;     // strip width: 32 lanes x 2 columns
+constexpr int kStU = 8;      // rows per block
+constexpr int kStH = 4;      // rows between two shifts of the running sums
+constexpr int kStChan = 6, kStFin = 2;  // channel warps, finishing warps
+constexpr int kStThreads = (kStChan + kStFin) * 32;
+
+template <int KD>
+struct StripGeom {
+    static constexpr int HAL = 3 * KD;
+    static constexpr int OFF = (HAL + 3) / 4 * 4;             // shared column of the strip's first column
+    static constexpr int RW = (OFF + kStW + HAL + 1 + 3) / 4 * 4;  // floats per staged row
+    static constexpr int NW2 = HAL + 2;                        // window, float2
+    static constexpr int NA = 2 * HAL + kStH;                  // running sums
+    static constexpr int LEAD = (2 * HAL + kStU - 1) / kStU;   // blocks before the first completed rows
+    // per CTA: staged rows (two blocks per channel), completed rows and bf16
+    // chunks (two blocks each)
+    static constexpr size_t rows_f = (size_t)6 * 2 * kStU * RW;
+    static constexpr size_t done_f = (size_t)2 * 6 * kStU * kStW;
+    static constexpr int CP = kStW + 1;                        // chunk row pitch (16-byte units)
+    static constexpr size_t smem = sizeof(float) * (rows_f + done_f) + 16 * (size_t)2 * kStU * CP;
+};
+
+// output rows per CTA of a batched launch (a single image's launch passes its own)
+__host__ __device__ inline int strip_rows(int H) {
+    const int seg = (H + 128) / 256 > 0 ? (H + 128) / 256 : 1;
+    return ((H + seg - 1) / seg + kStU - 1) / kStU * kStU;
+}
+
+// Copies kStU rows of one channel from row i0 (clamped to the image) into dst;
+// one commit group.  Strips whose window lies inside the rows copy 16-byte
+// pieces (rows and x0 - OFF are 16-byte aligned); others element by element
+// with clamped columns.
+template <int KD>
+__device__ __forceinline__ void strip_rows_async(const float* __restrict__ Fk, size_t fpitch, int H, int W, int x0,
+                                                 int i0, float* dst, int lane) {
+    using G = StripGeom<KD>;
+    const int xs = x0 - G::OFF;
+    if (xs >= 0 && xs + G::RW <= W) {
 #pragma unroll
-    for (int k = 0; k < KO; ++k) {
-        const float* Fk = F + (size_t)(g * NO + k) * fplane;
-        // tile k is in buffer k & 1; prefetch tile k+1 into the other one (its
-        // last reader, channel k-1's horizontal pass, is behind the barrier
-        // that ended that pass)
-        if (k + 1 < KO) {
-            tile_load_async<3 * KDG>(Fk + fplane, fpitch, H, W, x0, y0, (k & 1) ? s_F : s_F2, FW);
+        for (int u = 0; u < kStU; ++u) {
+            const float* src = Fk + (size_t)clampi(i0 + u, 0, H - 1) * fpitch + xs + 4 * lane;
+            const unsigned d = (unsigned)__cvta_generic_to_shared(dst + u * G::RW + 4 * lane);
+            if (lane < G::RW / 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+        }
+    } else {
+        for (int u = 0; u < kStU; ++u) {
+            const float* row = Fk + (size_t)clampi(i0 + u, 0, H - 1) * fpitch;
+            for (int c = lane; c < G::RW; c += 32) {
+                const unsigned d = (unsigned)__cvta_generic_to_shared(dst + u * G::RW + c);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(row + clampi(xs + c, 0, W - 1))
+                             : "memory");
+            }
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// The column-order bf16 chunks of a completed block: 8 lanes take the 8 rows of
+// one column, so that a column's 128 contiguous bytes leave together.
+__device__ __forceinline__ void strip_write_cm(const ImgJob& J, int g, const uint4* s_chunk, int cp, int x0, int yb,
+                                               int y1) {
+    uint4* const cm = reinterpret_cast<uint4*>(J.cm) + (size_t)g * J.H * J.W;
+    for (int p = threadIdx.x - kStChan * 32; p < kStU * kStW; p += kStFin * 32) {
+        const int c = p >> 3, u = p & 7;
+        const int gx = x0 + c, gy = yb + u;
+        if (gx < J.W && gy < y1) cm[(size_t)gx * J.H + gy] = s_chunk[u * cp + c];
+    }
+}
+
+// Where a finishing warp's lane writes: its two pixels of row 0, and what holds
+// for every row.
+struct StripOut {
+    float* s1;
+    float* s2;
+    float* c32;   // group g's first plane (or nullptr)
+    uint4* rm;    // group g's chunks (or nullptr)
+    size_t pitch, plane;
+    int W;
+    bool two;     // the second pixel is inside the image
+    bool vec;     // pairs of floats are 8-byte aligned in every row
+};
+
+// One completed row of a strip: a lane normalises its two pixels' six channels
+// (as write_pixel does) and writes the F32 planes, or the bf16 chunks, and the
+// per-pixel sums, continued from `sums` (g of both pixels, then g^2).
+// `done`: the row's [channel][8][64] values at the lane's columns; `chunk`: the
+// lane's place in the chunk buffer.
+__device__ __forceinline__ void strip_finish(const StripOut& o, float eps, const float* done, uint4* chunk, int gy,
+                                             const float4& sums) {
+    float2 d[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) d[k] = *reinterpret_cast<const float2*>(done + k * kStU * kStW);
+    float a1[2] = {sums.x, sums.y}, a2[2] = {sums.z, sums.w};
+    const bool bf = o.rm != nullptr;
+    float v[2][6];
+    unsigned pk[2][3];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        float n2 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const float x = e ? d[k].y : d[k].x;
+            n2 = fmaf(x, x, n2);
+        }
+        const float den = sqrtf(n2) + eps;
+        const float inv = den > 0.f ? 1.f / den : 0.f;  // NaN stays NaN through d * inv, and 0 / 0 is 0
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[e][k] = (e ? d[k].y : d[k].x) * inv;
+        if (bf) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const __nv_bfloat162 h = __floats2bfloat162_rn(v[e][2 * k], v[e][2 * k + 1]);
+                pk[e][k] = *reinterpret_cast<const unsigned*>(&h);
+                v[e][2 * k] = __uint_as_float(pk[e][k] << 16);
+                v[e][2 * k + 1] = __uint_as_float(pk[e][k] & 0xffff0000u);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            a1[e] += v[e][k];
+            a2[e] = fmaf(v[e][k], v[e][k], a2[e]);
+        }
+    }
+    const size_t at = (size_t)gy * o.pitch;
+    auto put2 = [&](float* q, float x, float y) {
+        if (o.vec && o.two) {
+            *reinterpret_cast<float2*>(q) = make_float2(x, y);
+        } else {
+            q[0] = x;
+            if (o.two) q[1] = y;
+        }
+    };
+    put2(o.s1 + at, a1[0], a1[1]);
+    put2(o.s2 + at, a2[0], a2[1]);
+    if (o.c32) {
+        float* q = o.c32 + at;
+#pragma unroll
+        for (int k = 0; k < 6; ++k, q += o.plane) put2(q, v[0][k], v[1][k]);
+    }
+    if (bf) {
+        uint4* const rm = o.rm + (size_t)gy * o.W;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {  // chunk g: the six channels, then two zeros
+            const uint4 c = make_uint4(pk[e][0], pk[e][1], pk[e][2], 0u);
+            if (e == 0 || o.two) rm[e] = c;
+            chunk[e] = c;
+        }
+    }
+}
+
+// One image (`one`, CTA = strip of the image's strips x segments) or a batch
+// (device table `jobs`, CTAs of image j from begin[j]).  seg_rows: output rows
+// per CTA, a multiple of kStU (0: strip_rows of the image).
+template <int KD>
+__global__ void __launch_bounds__(kStThreads, 2)
+    k_sfoc_smooth_strip(const __grid_constant__ ImgJob one, const ImgJob* __restrict__ jobs,
+                        const int* __restrict__ begin, int n_jobs, const __grid_constant__ SmoothTaps tp, int g,
+                        int seg_rows) {
+    using G = StripGeom<KD>;
+    constexpr int HAL = G::HAL, U = kStU, UH = kStH;
+    constexpr int kFull = 1, kEmpty = 3, kPair = 5;  // named barriers (two buffers each; the finishing warps' own)
+    extern __shared__ __align__(16) float sm[];
+    float* s_rows = sm;                 // [channel][2][U][RW]
+    float* s_done = s_rows + G::rows_f;  // [2][channel][U][kStW]
+    uint4* s_chunk = reinterpret_cast<uint4*>(s_done + G::done_f);  // [2][U][CP]
+    int tile;
+    const ImgJob& J = img_job(one, jobs, begin, n_jobs, &tile);
+    const int H = J.H, W = J.W;
+    const int strips = (W + kStW - 1) / kStW;
+    const int rows = seg_rows ? seg_rows : strip_rows(H);
+    const int seg = tile / strips;
+    const int x0 = (tile - seg * strips) * kStW, y0 = seg * rows;
+    const int y1 = min(y0 + rows, H);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nout = (y1 - y0 + U - 1) / U;  // blocks of completed rows
+    // the first group's launch lets the second one's start beside it; the second
+    // one reads only F (complete before the first began) until its finishing warps
+    // have waited for the first to end
+    if (g == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (warp >= kStChan) {
+        if (g) asm volatile("griddepcontrol.wait;" ::: "memory");
+        // ---- finishing warps: rows warp - kStChan, + kStFin, ... of each block
+        const int gx = x0 + 2 * lane;
+        const size_t plane = J.cpitch * (size_t)H;
+        StripOut o;
+        o.s1 = J.s1 + gx;
+        o.s2 = J.s2 + gx;
+        o.c32 = J.c32 ? J.c32 + (size_t)g * 6 * plane + gx : nullptr;
+        o.rm = J.rm ? reinterpret_cast<uint4*>(J.rm) + (size_t)g * H * W + gx : nullptr;
+        o.pitch = J.cpitch;
+        o.plane = plane;
+        o.W = W;
+        o.two = gx + 1 < W;
+        o.vec = (J.cpitch & 1) == 0 && ((reinterpret_cast<uintptr_t>(J.s1) | reinterpret_cast<uintptr_t>(J.s2) |
+                                         reinterpret_cast<uintptr_t>(J.c32)) & 7) == 0;
+        for (int m = 0; m < nout; ++m) {
+            const int b = m & 1, yb = y0 + m * U + warp - kStChan;
+            float4 sums[U / kStFin];
+#pragma unroll
+            for (int v = 0; v < U / kStFin; ++v) {
+                const int gy = yb + v * kStFin;
+                sums[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (g > 0 && gy < y1 && gx < W) {
+                    const size_t at = (size_t)gy * o.pitch;
+                    sums[v].x = o.s1[at];
+                    sums[v].z = o.s2[at];
+                    if (o.two) {
+                        sums[v].y = o.s1[at + 1];
+                        sums[v].w = o.s2[at + 1];
+                    }
+                }
+            }
+            __syncwarp();
+            asm volatile("bar.sync %0, %1;" ::"r"(kFull + b), "n"(kStThreads) : "memory");
+            const float* done = s_done + (size_t)b * kStChan * U * kStW + (warp - kStChan) * kStW + 2 * lane;
+            uint4* chunk = s_chunk + (size_t)b * U * G::CP + (warp - kStChan) * G::CP + 2 * lane;
+#pragma unroll
+            for (int v = 0; v < U / kStFin; ++v)
+                if (yb + v * kStFin < y1 && gx < W)
+                    strip_finish(o, tp.eps, done + v * kStFin * kStW, chunk + v * kStFin * G::CP, yb + v * kStFin, sums[v]);
+            __syncwarp();
+            if (m + 2 < nout) asm volatile("bar.arrive %0, %1;" ::"r"(kEmpty + b), "n"(kStThreads) : "memory");
+            if (J.cm) {  // (a chunk buffer's next writer is behind the next block's barrier)
+                asm volatile("bar.sync %0, %1;" ::"r"(kPair), "n"(kStFin * 32) : "memory");
+                strip_write_cm(J, g, s_chunk + (size_t)b * U * G::CP, G::CP, x0, y0 + m * U, y1);
+                __syncwarp();
+            }
+        }
+        return;
+    }
+    // ---- channel warps
+    const size_t fpitch = J.fpitch, fplane = J.fpitch * (size_t)J.H;
+    const float* __restrict__ Fk = J.F + (size_t)(g * kStChan + warp) * fplane;
+    float* const ring = s_rows + (size_t)warp * 2 * U * G::RW;
+    float2 tq[KD + 1];
+#pragma unroll
+    for (int q = 0; q <= KD; ++q) {
+        const float t = g ? tp.g[1][q] : tp.g[0][q];
+        tq[q] = make_float2(t, t);
+    }
+    float2 a[G::NA];  // a[k]: output row i0 + k - HAL of the rows that start at input row i0
+#pragma unroll
+    for (int k = 0; k < G::NA; ++k) a[k] = make_float2(0.f, 0.f);
+
+    // input rows from i0 = y0 - (LEAD U - HAL), so that block LEAD completes y0 .. y0 + U - 1
+    const int first = y0 + HAL - G::LEAD * U;
+    const int nb = G::LEAD + nout;
+    strip_rows_async<KD>(Fk, fpitch, H, W, x0, first, ring, lane);
+#pragma unroll 1
+    for (int n = 0; n < nb; ++n) {
+        if (n + 1 < nb) {
+            strip_rows_async<KD>(Fk, fpitch, H, W, x0, first + (n + 1) * U, ring + ((n + 1) & 1) * U * G::RW, lane);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
-        __syncthreads();  // tile k visible; every thread is done with channel k-1
-        smooth_channel_123<KDG>(t, (k & 1) ? s_F2 : s_F, FW, s_h, HR, D[k]);
-    }
+        __syncwarp();  // every lane's copies of the block have landed
+        const int m = n - G::LEAD;
+        float* done = s_done + (size_t)((m & 1) * kStChan + warp) * U * kStW + 2 * lane;
+        if (m >= 2) asm volatile("bar.sync %0, %1;" ::"r"(kEmpty + (m & 1)), "n"(kStThreads) : "memory");
+        const float* blk = ring + (n & 1) * U * G::RW + (G::OFF - HAL - 1) + 2 * lane;
+#pragma unroll 1
+        for (int uh = 0; uh < U; uh += UH) {
 #pragma unroll
-    for (int j = 0; j < kPRows; ++j) {
-        float d0[KO], d1[KO];
+            for (int u = 0; u < UH; ++u) {
+                float2 w[G::NW2];  // shared columns OFF + 2 lane - HAL - 1 ...
 #pragma unroll
-        for (int k = 0; k < KO; ++k) {
-            d0[k] = D[k][j].x;
-            d1[k] = D[k][j].y;
-        }
-        const int gy = y0 + rb + j;
-        write_pixel<NO, KO>(g, NO, d0, eps, gy, gx, H, W, c32, cpitch, cplane, rm, cm, a1[j][0], a2[j][0]);
-        write_pixel<NO, KO>(g, NO, d1, eps, gy, gx + 1, H, W, c32, cpitch, cplane, rm, cm, a1[j][1], a2[j][1]);
-    }
-}
-
-// The paper's dilation rates 1, 2, 3 with smoothing radius KDG at compile
-// time, one group g per launch: the kernel holds only one group's code (its
-// instruction footprint is what limits the fully unrolled passes) and fits
-// two CTAs per SM.  The second group's launch continues the per-pixel sums
-// from the stored planes, adding in the same order as one launch would.
-// One image (`one`, CTA = tile in row-major tile order) or a batch (device
-// table `jobs`, CTAs of image j from begin[j]).
-template <int NO, int KDG>
-__global__ void __launch_bounds__(kThreads, 2)
-    k_sfoc_smooth_grp(const __grid_constant__ ImgJob one, const ImgJob* __restrict__ jobs,
-                      const int* __restrict__ begin, int n_jobs, SmoothTaps tp, int g) {
-    extern __shared__ float sm[];
-    int tile;
-    const ImgJob& J = img_job(one, jobs, begin, n_jobs, &tile);
-    const float* __restrict__ F = J.F;
-    const size_t fpitch = J.fpitch, fplane = J.fpitch * (size_t)J.H;
-    const int H = J.H, W = J.W;
-    float* __restrict__ c32 = J.c32;
-    const size_t cpitch = J.cpitch, cplane = J.cpitch * (size_t)J.H;
-    __nv_bfloat16* __restrict__ rm = J.rm;
-    __nv_bfloat16* __restrict__ cm = J.cm;
-    float* __restrict__ s1 = J.s1;
-    float* __restrict__ s2 = J.s2;
-    __shared__ float s_tap[kMaxSmoothRadius + 1];
-    if (threadIdx.x == 0) {  // constant indices: the parameter block stays in the constant bank
+                for (int v = 0; v < G::NW2; ++v) w[v] = *reinterpret_cast<const float2*>(blk + u * G::RW + 2 * v);
 #pragma unroll
-        for (int q = 0; q <= kMaxSmoothRadius; ++q) s_tap[q] = g ? tp.g[1][q] : tp.g[0][q];
-    }
-    constexpr int hal = 3 * KDG;
-    const int FW = smooth_row_stride(hal);
-    constexpr int HR = kSTH + 2 * hal;
-    float* s_F = sm;                   // HR x FW
-    float* s_h = s_F + HR * FW;        // 3 x HR x kSTW
-    float* s_F2 = s_h + 3 * HR * kSTW;  // second input tile buffer
-    const int ntx = (W + kSTW - 1) / kSTW;
-    const int tby = tile / ntx;
-    const int x0 = (tile - tby * ntx) * kSTW, y0 = tby * kSTH;
-    const int cp = threadIdx.x & 15, rb = (threadIdx.x >> 4) * kPRows;
-
-    float a1[kPRows][2], a2[kPRows][2];
+                for (int r = 1; r <= 3; ++r) {
+                    // horizontal sum of rate r at both columns, outer taps first
+                    float2 h = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < kPRows; ++j)
+                    for (int q = KD; q >= 1; --q) {
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int gy = y0 + rb + j, gx = x0 + 2 * cp + e;
-            const bool in = g > 0 && gy < H && gx < W;
-            a1[j][e] = in ? s1[(size_t)gy * cpitch + gx] : 0.f;
-            a2[j][e] = in ? s2[(size_t)gy * cpitch + gx] : 0.f;
-        }
-    smooth_group_123<NO, KDG>(g, F, fpitch, fplane, H, W, tp.eps, s_tap, s_F, s_F2, FW, s_h, HR, x0, y0, c32, cpitch,
-                              cplane, rm, cm, a1, a2);
+                        for (int sg = -1; sg <= 1; sg += 2) {
+                            const int s = HAL + 1 + sg * q * r;  // window index of column 0's sample
+                            const bool firstt = q == KD && sg < 0;
+                            if (s % 2 == 0) {
+                                h = firstt ? __fmul2_rn(tq[q], w[s / 2]) : __ffma2_rn(tq[q], w[s / 2], h);
+                            } else {
+                                h.x = firstt ? tq[q].x * w[s / 2].y : fmaf(tq[q].x, w[s / 2].y, h.x);
+                                h.y = firstt ? tq[q].x * w[s / 2 + 1].x : fmaf(tq[q].x, w[s / 2 + 1].x, h.y);
+                            }
+                        }
+                    }
+                    h = __ffma2_rn(tq[0], w[(HAL + 1) / 2], h);
+                    // row i = i0 + u of rate r belongs to output rows i + q r
 #pragma unroll
-    for (int j = 0; j < kPRows; ++j)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int gy = y0 + rb + j, gx = x0 + 2 * cp + e;
-            if (gy < H && gx < W) {
-                s1[(size_t)gy * cpitch + gx] = a1[j][e];
-                s2[(size_t)gy * cpitch + gx] = a2[j][e];
+                    for (int q = -KD; q <= KD; ++q)
+                        a[u + HAL + q * r] = __ffma2_rn(tq[q < 0 ? -q : q], h, a[u + HAL + q * r]);
+                }
             }
+            blk += UH * G::RW;
+            if (m >= 0) {
+#pragma unroll
+                for (int u = 0; u < UH; ++u) *reinterpret_cast<float2*>(done + (uh + u) * kStW) = a[u];
+            }
+#pragma unroll
+            for (int k = 0; k < G::NA; ++k) a[k] = k + UH < G::NA ? a[k + UH] : make_float2(0.f, 0.f);
         }
+        __syncwarp();  // the block's rows are read before the copies of block n + 2 replace them
+        if (m >= 0) asm volatile("bar.arrive %0, %1;" ::"r"(kFull + (m & 1)), "n"(kStThreads) : "memory");
+    }
 }
 
 // Any radii and rates at run time.
@@ -772,23 +875,52 @@ int smooth_launch_count(const SmoothTaps& tp) { return smooth_is_paper(tp) ? 2 :
 namespace {
 
 // the two group launches of the paper's smoothing (sigma_d 1.0 / 1.5, rates
-// 1, 2, 3) over `ctas` CTAs
+// 1, 2, 3) over `ctas` CTAs of seg_rows output rows (0: a batch's own)
 cudaError_t launch_smooth_paper(const ImgJob& one, const ImgJob* jobs, const int* begin, int n_jobs, int ctas,
-                                const SmoothTaps& tp, cudaStream_t st) {
-    auto run = [&](auto kern, int g, int hal) -> cudaError_t {
-        const int HR = kSTH + 2 * hal, FW = smooth_row_stride(hal);
-        const size_t smem = sizeof(float) * (2 * (size_t)HR * FW + 3 * (size_t)HR * kSTW);
-        cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e2 == cudaSuccess)
-            e2 = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      (int)cudaSharedmemCarveoutMaxShared);
+                                int seg_rows, const SmoothTaps& tp, cudaStream_t st) {
+    auto run = [&](auto kern, int g, size_t smem) -> cudaError_t {
+        const cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e2 != cudaSuccess) return e2;
-        kern<<<ctas, kThreads, smem, st>>>(one, jobs, begin, n_jobs, tp, g);
-        return cudaGetLastError();
+        // The second group may start while the first one's last CTAs run (it needs
+        // of them only the sum planes, which its finishing warps wait for): the
+        // first launch's partial last wave, or the half-empty chip of a small
+        // image, does not idle.
+        cudaLaunchAttribute early;
+        early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        early.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3(kStThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cfg.attrs = &early;
+        cfg.numAttrs = g ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, kern, one, jobs, begin, n_jobs, tp, g, seg_rows);
     };
-    cudaError_t e = run(k_sfoc_smooth_grp<6, 3>, 0, 9);
-    if (e == cudaSuccess) e = run(k_sfoc_smooth_grp<6, 5>, 1, 15);
+    cudaError_t e = run(k_sfoc_smooth_strip<3>, 0, StripGeom<3>::smem);
+    if (e == cudaSuccess) e = run(k_sfoc_smooth_strip<5>, 1, StripGeom<5>::smem);
     return e;
+}
+
+// Output rows per CTA for one image: every CTA streams up to four blocks more
+// than it completes, and an SM's time is the blocks of its CTAs (one alone runs
+// a block in about half the time of two together): the rows with the fewest
+// blocks on the fullest SM.
+int strip_rows_single(int H, int W) {
+    const long strips = (W + kStW - 1) / kStW, sms = 152;
+    long best = -1;
+    int rows = kStU;
+    for (int r = kStU; r < H + kStU; r += kStU) {
+        const long ctas = strips * ((H + r - 1) / r);
+        const long cost = (ctas + sms - 1) / sms * (r / kStU + 4);
+        if (best < 0 || cost < best) {
+            best = cost;
+            rows = r;
+        }
+        if (ctas <= sms) break;  // one CTA per SM already: longer segments only take longer
+    }
+    return rows;
 }
 
 }  // namespace
@@ -797,7 +929,8 @@ bool sfoc_batch_supported(const SteerTaps& st, const SmoothTaps& sm) { return st
 
 void sfoc_batch_tiles(int H, int W, int* steer_ctas, int* smooth_ctas) {
     *steer_ctas = ((W + kTW - 1) / kTW) * ((H + kTH - 1) / kTH);
-    *smooth_ctas = ((W + kSTW - 1) / kSTW) * ((H + kSTH - 1) / kSTH);
+    const int rows = strip_rows(H);
+    *smooth_ctas = ((W + kStW - 1) / kStW) * ((H + rows - 1) / rows);
 }
 
 cudaError_t launch_sfoc_batch(const ImgJob* jobs, int n_jobs, const int* steer_begin, int steer_ctas,
@@ -814,7 +947,7 @@ cudaError_t launch_sfoc_batch(const ImgJob* jobs, int n_jobs, const int* steer_b
     kern<<<steer_ctas, kThreads, smem, s>>>(none, jobs, steer_begin, n_jobs, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_smooth_paper(none, jobs, smooth_begin, n_jobs, smooth_ctas, sm, s);
+    return launch_smooth_paper(none, jobs, smooth_begin, n_jobs, smooth_ctas, 0, sm, s);
 }
 
 cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, const SmoothTaps& tp, Cube& c,
@@ -834,7 +967,9 @@ cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, cons
         one.cm = c.cm;
         one.s1 = c.s1;
         one.s2 = c.s2;
-        return launch_smooth_paper(one, nullptr, nullptr, 0, (int)(grid.x * grid.y), tp, st);
+        const int rows = strip_rows_single(H, W);
+        const int ctas = ((W + kStW - 1) / kStW) * ((H + rows - 1) / rows);
+        return launch_smooth_paper(one, nullptr, nullptr, 0, ctas, rows, tp, st);
     }
     const int maxhal = tp.halo[0] > tp.halo[1] ? tp.halo[0] : tp.halo[1];
     const int HR = kSTH + 2 * maxhal, FW = smooth_row_stride(maxhal);
