@@ -10,7 +10,7 @@
 // and rates: they stage a 2-D tile with its clamped halo in shared memory and
 // do the horizontal pass into shared planes, then the vertical pass per output
 // pixel.  The paper's own parameters take the streaming forms
-// k_sfoc_steer_ct (tiles, radii at compile time) and k_sfoc_smooth_strip.
+// k_sfoc_steer_strip and k_sfoc_smooth_strip.
 #include <cuda_bf16.h>
 #include <string.h>
 
@@ -130,148 +130,177 @@ __global__ void __launch_bounds__(kThreads) k_sfoc_steer(const T* __restrict__ i
     }
 }
 
-// Steering with the radii at compile time (three first-order scales of
-// radii KA, KB, KC and the second-order radius KS; the paper's scales give
-// 2, 3, 3 and 5).  Same arithmetic per output as k_sfoc_steer, register
-// blocked: a thread of the horizontal pass loads one row span once (float4)
-// and produces all nine basis planes for 8 columns; a thread of the
-// vertical pass loads each plane's column span once and produces 4 rows.
-template <int K>
-__device__ __forceinline__ float ceven(const float* x, const float* t) {
-    float acc = t[0] * x[0];
-#pragma unroll
-    for (int q = 1; q <= K; ++q) acc = fmaf(t[q], x[-q] + x[q], acc);
-    return acc;
-}
-template <int K>
-__device__ __forceinline__ float codd(const float* x, const float* t) {
-    float acc = 0.f;
-#pragma unroll
-    for (int q = 1; q <= K; ++q) acc = fmaf(t[q], x[-q] - x[q], acc);
-    return acc;
+// Steering at the paper's radii (three first-order scales of radii 2, 3, 3 and
+// the second-order radius 5; six orientations).
+//
+// A warp takes a strip of 32 columns, a lane per column, and streams down its
+// rows: from a row's window of 11 samples a lane makes the nine horizontal
+// sums (sums and differences x[-q] +- x[q] shared by all nine) and adds each at
+// once to the rows of its vertical pass, which are running sums in registers.
+// Nothing but the image row passes through shared memory.  Rows are taken 4 at
+// a time; first-order rows complete 3 rows behind the input, second-order rows
+// 5, and are steered and written as they complete.
+//
+// What bounds it: writing the twelve planes (48 B per pixel), then ~180 FP32
+// operations per pixel.  The tiled form this replaces (image tile with clamped
+// element-wise loads, nine planes written to shared memory and read back)
+// spent most of its time waiting for the tile.  2048 x 2048: 90 -> 53 us
+// (the planes alone take 30).
+constexpr int kSrW = 32, kSrU = 4, kSrThreads = 128, kSrPitch = 44;  // staged columns x0 - 5 .. x0 + 36
+
+// output rows per warp of a batched launch (a single image's launch passes its own)
+__host__ __device__ inline int steer_rows(int H) {
+    const int seg = (H + 64) / 128 > 0 ? (H + 64) / 128 : 1;
+    return ((H + seg - 1) / seg + kSrU - 1) / kSrU * kSrU;
 }
 
-// Three CTAs per SM: the 80-register cap (a few spilled values) hides the
-// tile loads better than two CTAs at 127 registers did (0.207 -> 0.179 ms
-// per step for the two 2048 x 2048 images).
-// One image (`one`, CTA = tile in row-major tile order) or a batch (device
-// table `jobs`, CTAs of image j from begin[j]).
-template <typename T, int KA, int KB, int KC, int KS>
-__global__ void __launch_bounds__(kThreads, 3) k_sfoc_steer_ct(const __grid_constant__ ImgJob one,
-                                                             const ImgJob* __restrict__ jobs,
-                                                             const int* __restrict__ begin, int n_jobs,
-                                                             SteerTaps tp) {
-    constexpr int HAL = KS > KA ? (KS > KB ? (KS > KC ? KS : KC) : (KB > KC ? KB : KC))
-                                : (KA > KB ? (KA > KC ? KA : KC) : (KB > KC ? KB : KC));
-    constexpr int IH = kTH + 2 * HAL, IW = kTW + 2 * HAL;
-    constexpr int NV = (8 + 2 * HAL + 3) / 4;            // float4 per horizontal span
-    constexpr int IWP = ((24 + 4 * NV + 3) / 4 % 2) ? (24 + 4 * NV + 3) / 4 * 4 : (24 + 4 * NV + 3) / 4 * 4 + 4;
-    constexpr int NP = 9;                                 // basis planes
-    __shared__ __align__(16) float s_img[IH * IWP];
-    extern __shared__ float4 sm4[];
-    float* s_h = reinterpret_cast<float*>(sm4);          // NP x IH x kTW
-    __shared__ float s_t[NP][kMaxDerivRadius + 1];        // taps of the nine 1-D factors
+// One image (`one`, warps = strips x segments in row-major order) or a batch
+// (device table `jobs`, CTAs of image j from begin[j]).  seg_rows: output rows
+// per warp (0: steer_rows of the image).
+template <typename T>
+__global__ void __launch_bounds__(kSrThreads, 3)
+    k_sfoc_steer_strip(const __grid_constant__ ImgJob one, const ImgJob* __restrict__ jobs,
+                       const int* __restrict__ begin, int n_jobs, const __grid_constant__ SteerTaps tp, int seg_rows) {
+    constexpr int U = kSrU, N1 = U + 6, N2 = U + 10;
+    __shared__ float s_rows[kSrThreads / 32][2][U][kSrPitch];
     int tile;
     const ImgJob& J = img_job(one, jobs, begin, n_jobs, &tile);
     const T* __restrict__ img = static_cast<const T*>(J.img);
     const int H = J.H, W = J.W;
     const size_t pitch = J.pitch, fpitch = J.fpitch, fplane = J.fpitch * (size_t)J.H;
     float* __restrict__ F = J.F;
-    const int ntx = (W + kTW - 1) / kTW;
-    const int tby = tile / ntx;
-    const int x0 = (tile - tby * ntx) * kTW, y0 = tby * kTH;
-    if (threadIdx.x < NP * (kMaxDerivRadius + 1)) {
-        const int pl = threadIdx.x / (kMaxDerivRadius + 1), q = threadIdx.x % (kMaxDerivRadius + 1);
-        const float* src = pl < 6 ? ((pl & 1) ? tp.g1[pl >> 1] : tp.a1[pl >> 1])
-                                  : (pl == 6 ? tp.a2 : (pl == 7 ? tp.g2 : tp.c2x));
-        s_t[pl][q] = src[q];
-    }
-    for (int i = threadIdx.x; i < IH * IW; i += kThreads) {
-        const int r = i / IW, c = i - r * IW;
-        const int gy = clampi(y0 + r - HAL, 0, H - 1), gx = clampi(x0 + c - HAL, 0, W - 1);
-        s_img[r * IWP + c] = to_unit(__ldg(img + (size_t)gy * pitch + gx));
-    }
-    __syncthreads();
-    // horizontal: task = (row, 8-column block); planes 2s = a1_s (odd),
-    // 2s+1 = g1_s (even), 6 = a2 (even), 7 = g2 (even), 8 = c2x (odd)
-    for (int task = threadIdx.x; task < IH * 4; task += kThreads) {
-        const int rr = task >> 2, cb = (task & 3) * 8;
-        const float4* x4 = reinterpret_cast<const float4*>(s_img + rr * IWP + cb);
-        float in[NV * 4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int strips = (W + kSrW - 1) / kSrW;
+    const int rows = seg_rows ? seg_rows : steer_rows(H);
+    const int task = tile * (kSrThreads / 32) + warp;
+    const int seg = task / strips;
+    const int x0 = (task - seg * strips) * kSrW, y0 = seg * rows;
+    if (y0 >= H) return;  // (no block barrier below)
+    const int y1 = min(y0 + rows, H);
+    const int gx = x0 + lane;
+    const int xa = clampi(gx - 5, 0, W - 1), xb = clampi(gx + 27, 0, W - 1);  // this lane's staged columns
+
+    float ix[3][N1], iy[3][N1], dxx[N2], dyy[N2], dxy[N2];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const float4 f = x4[v];
-            in[4 * v] = f.x;
-            in[4 * v + 1] = f.y;
-            in[4 * v + 2] = f.z;
-            in[4 * v + 3] = f.w;
+    for (int k = 0; k < N1; ++k)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) ix[q][k] = iy[q][k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < N2; ++k) dxx[k] = dyy[k] = dxy[k] = 0.f;
+
+    float pa[U], pb[U];  // the next block's samples
+    auto fetch = [&](int i0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const T* row = img + (size_t)clampi(i0 + u, 0, H - 1) * pitch;
+            pa[u] = to_unit(__ldg(row + xa));
+            pb[u] = lane < 10 ? to_unit(__ldg(row + xb)) : 0.f;
         }
-        float o[NP][8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const float* x = in + HAL + c;
-            o[0][c] = codd<KA>(x, s_t[0]);
-            o[1][c] = ceven<KA>(x, s_t[1]);
-            o[2][c] = codd<KB>(x, s_t[2]);
-            o[3][c] = ceven<KB>(x, s_t[3]);
-            o[4][c] = codd<KC>(x, s_t[4]);
-            o[5][c] = ceven<KC>(x, s_t[5]);
-            o[6][c] = ceven<KS>(x, s_t[6]);
-            o[7][c] = ceven<KS>(x, s_t[7]);
-            o[8][c] = codd<KS>(x, s_t[8]);
-        }
-#pragma unroll
-        for (int pl = 0; pl < NP; ++pl) {
-            float4* dst = reinterpret_cast<float4*>(s_h + (pl * IH + rr) * kTW + cb);
-            dst[0] = make_float4(o[pl][0], o[pl][1], o[pl][2], o[pl][3]);
-            dst[1] = make_float4(o[pl][4], o[pl][5], o[pl][6], o[pl][7]);
-        }
-    }
-    __syncthreads();
-    // vertical: thread = (column, 4-row block)
-    const int col = threadIdx.x & 31, rb = (threadIdx.x >> 5) * 4;
-    float Ix[3][4], Iy[3][4], Ixx[4], Iyy[4], Ixy[4];
-    auto vpass = [&](int pl, auto kr, auto odd, const float* t, float (&out)[4]) {
-        constexpr int K = decltype(kr)::value;
-        float in[4 + 2 * K];
-        const float* x = s_h + (pl * IH + rb + HAL - K) * kTW + col;
-#pragma unroll
-        for (int i = 0; i < 4 + 2 * K; ++i) in[i] = x[i * kTW];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[j] = decltype(odd)::value ? codd<K>(in + K + j, t) : ceven<K>(in + K + j, t);
     };
-    using F0 = std::integral_constant<bool, false>;
-    using T1 = std::integral_constant<bool, true>;
-    vpass(0, std::integral_constant<int, KA>(), F0(), tp.g1[0], Ix[0]);  // a1(x) g(y)
-    vpass(1, std::integral_constant<int, KA>(), T1(), tp.a1[0], Iy[0]);  // g(x) a1(y)
-    vpass(2, std::integral_constant<int, KB>(), F0(), tp.g1[1], Ix[1]);
-    vpass(3, std::integral_constant<int, KB>(), T1(), tp.a1[1], Iy[1]);
-    vpass(4, std::integral_constant<int, KC>(), F0(), tp.g1[2], Ix[2]);
-    vpass(5, std::integral_constant<int, KC>(), T1(), tp.a1[2], Iy[2]);
-    vpass(6, std::integral_constant<int, KS>(), F0(), tp.g2, Ixx);       // a2(x) g2(y)
-    vpass(7, std::integral_constant<int, KS>(), F0(), tp.a2, Iyy);       // g2(x) a2(y)
-    vpass(8, std::integral_constant<int, KS>(), T1(), tp.c2y, Ixy);      // c(x) c(y)
-    const int gx = x0 + col;
+    fetch(y0 - 5);
+    int buf = 0;
+    for (int i0 = y0 - 5; i0 < y1 + 5; i0 += U, buf ^= 1) {
+        float (*st)[kSrPitch] = s_rows[warp][buf];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int gy = y0 + rb + j;
-        if (gy >= H || gx >= W) continue;
-        float* out = F + (size_t)gy * fpitch + gx;
+        for (int u = 0; u < U; ++u) {
+            st[u][lane] = pa[u];
+            if (lane < 10) st[u][32 + lane] = pb[u];
+        }
+        // one warp barrier a block: a buffer's readers are behind the next block's
+        __syncwarp();
+        if (i0 + U < y1 + 5) fetch(i0 + U);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            float f = 0.f;
+        for (int u = 0; u < U; ++u) {
+            const float* x = &st[u][lane + 5];
+            const float c = x[0];
+            float e[6], o[6];
 #pragma unroll
-            for (int sc = 0; sc < 3; ++sc) {
-                float v = fmaf(tp.ct[k], Ix[sc][j], tp.st[k] * Iy[sc][j]);
-                f += tp.rectify ? fabsf(v) : v;
+            for (int q = 1; q <= 5; ++q) {
+                const float l = x[-q], r = x[q];
+                e[q] = l + r;
+                o[q] = l - r;
             }
-            out[(size_t)k * fplane] = f;
+            auto even = [&](const float* t, int K) {
+                float v = t[0] * c;
+#pragma unroll
+                for (int q = 1; q <= 5; ++q)
+                    if (q <= K) v = fmaf(t[q], e[q], v);
+                return v;
+            };
+            auto odd = [&](const float* t, int K) {
+                float v = t[1] * o[1];
+#pragma unroll
+                for (int q = 2; q <= 5; ++q)
+                    if (q <= K) v = fmaf(t[q], o[q], v);
+                return v;
+            };
+            // vertical: row i0 + u goes to rows i0 + u +- q; entry k of the first
+            // order is row i0 + k - 3, of the second order row i0 + k - 5
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int K = q == 0 ? 2 : 3;
+                const float ha = odd(tp.a1[q], K), hg = even(tp.g1[q], K);
+                ix[q][u + 3] = fmaf(tp.g1[q][0], ha, ix[q][u + 3]);
+#pragma unroll
+                for (int d = 1; d <= 3; ++d)
+                    if (d <= K) {
+                        ix[q][u + 3 - d] = fmaf(tp.g1[q][d], ha, ix[q][u + 3 - d]);
+                        ix[q][u + 3 + d] = fmaf(tp.g1[q][d], ha, ix[q][u + 3 + d]);
+                        iy[q][u + 3 + d] = fmaf(tp.a1[q][d], hg, iy[q][u + 3 + d]);
+                        iy[q][u + 3 - d] = fmaf(-tp.a1[q][d], hg, iy[q][u + 3 - d]);
+                    }
+            }
+            const float hx = even(tp.a2, 5), hy = even(tp.g2, 5), hc = odd(tp.c2x, 5);
+            dxx[u + 5] = fmaf(tp.g2[0], hx, dxx[u + 5]);
+            dyy[u + 5] = fmaf(tp.a2[0], hy, dyy[u + 5]);
+#pragma unroll
+            for (int d = 1; d <= 5; ++d) {
+                dxx[u + 5 - d] = fmaf(tp.g2[d], hx, dxx[u + 5 - d]);
+                dxx[u + 5 + d] = fmaf(tp.g2[d], hx, dxx[u + 5 + d]);
+                dyy[u + 5 - d] = fmaf(tp.a2[d], hy, dyy[u + 5 - d]);
+                dyy[u + 5 + d] = fmaf(tp.a2[d], hy, dyy[u + 5 + d]);
+                dxy[u + 5 + d] = fmaf(tp.c2y[d], hc, dxy[u + 5 + d]);
+                dxy[u + 5 - d] = fmaf(-tp.c2y[d], hc, dxy[u + 5 - d]);
+            }
         }
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            float c2 = tp.ct[k] * tp.ct[k], s2 = tp.st[k] * tp.st[k], cs = 2.f * tp.st[k] * tp.ct[k];
-            float v = fmaf(c2, Ixx[j], fmaf(s2, Iyy[j], -cs * Ixy[j]));
-            out[(size_t)(6 + k) * fplane] = tp.rectify ? fabsf(v) : v;
+        for (int u = 0; u < U; ++u) {
+            const int ya = i0 + u - 3, yb = i0 + u - 5;
+            if (gx < W && ya >= y0 && ya < y1) {
+                float* out = F + (size_t)ya * fpitch + gx;
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    float f = 0.f;
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        const float v = fmaf(tp.ct[k], ix[q][u], tp.st[k] * iy[q][u]);
+                        f += tp.rectify ? fabsf(v) : v;
+                    }
+                    out[(size_t)k * fplane] = f;
+                }
+            }
+            if (gx < W && yb >= y0 && yb < y1) {
+                float* out = F + (size_t)yb * fpitch + gx;
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    const float c2 = tp.ct[k] * tp.ct[k], s2 = tp.st[k] * tp.st[k], cs = 2.f * tp.st[k] * tp.ct[k];
+                    const float v = fmaf(c2, dxx[u], fmaf(s2, dyy[u], -cs * dxy[u]));
+                    out[(size_t)(6 + k) * fplane] = tp.rectify ? fabsf(v) : v;
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < N1; ++k)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                ix[q][k] = k + U < N1 ? ix[q][k + U] : 0.f;
+                iy[q][k] = k + U < N1 ? iy[q][k + U] : 0.f;
+            }
+#pragma unroll
+        for (int k = 0; k < N2; ++k) {
+            dxx[k] = k + U < N2 ? dxx[k + U] : 0.f;
+            dyy[k] = k + U < N2 ? dyy[k + U] : 0.f;
+            dxy[k] = k + U < N2 ? dxy[k + U] : 0.f;
         }
     }
 }
@@ -827,16 +856,35 @@ bool steer_is_paper(const SteerTaps& tp) {
     return tp.ns == 3 && tp.K1[0] == 2 && tp.K1[1] == 3 && tp.K1[2] == 3 && tp.second && tp.K2 == 5 && tp.no == 6;
 }
 
+int steer_ctas(int H, int W, int rows) {
+    const int tasks = ((W + kSrW - 1) / kSrW) * ((H + rows - 1) / rows);
+    return (tasks + kSrThreads / 32 - 1) / (kSrThreads / 32);
+}
+
+// Output rows per warp for one image: the rows with the least waves (three CTAs
+// of four warps per SM) x rows streamed (10 more than the output rows).
+int steer_rows_single(int H, int W) {
+    const int slots = 3 * 152;
+    long best = -1;
+    int rows = kSrU;
+    for (int r = 4 * kSrU; r < H + kSrU; r += kSrU) {
+        const long ctas = steer_ctas(H, W, r);
+        const long cost = (ctas + slots - 1) / slots * (r + 14);
+        if (best < 0 || cost <= best) {
+            best = cost;
+            rows = r;
+        }
+        if (ctas <= slots / 2) break;  // one partial wave already: longer segments only take longer
+    }
+    return rows;
+}
+
 template <typename T>
 cudaError_t launch_steer_any(const T* img, int H, int W, size_t pitch, float* F, size_t fpitch, const SteerTaps& tp,
                              cudaStream_t st) {
     dim3 grid((W + kTW - 1) / kTW, (H + kTH - 1) / kTH);
     // the paper's scales (0.6, 0.8, 1.0 and 1.5 at 3 sigma: radii 2, 3, 3, 5), six orientations
     if (steer_is_paper(tp)) {
-        auto kern = k_sfoc_steer_ct<T, 2, 3, 3, 5>;
-        const size_t smem = sizeof(float) * 9 * (size_t)(kTH + 10) * kTW;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
         ImgJob one;
         memset(&one, 0, sizeof(one));
         one.img = img;
@@ -845,7 +893,8 @@ cudaError_t launch_steer_any(const T* img, int H, int W, size_t pitch, float* F,
         one.W = W;
         one.F = F;
         one.fpitch = fpitch;
-        kern<<<grid.x * grid.y, kThreads, smem, st>>>(one, nullptr, nullptr, 0, tp);
+        const int rows = steer_rows_single(H, W);
+        k_sfoc_steer_strip<T><<<steer_ctas(H, W, rows), kSrThreads, 0, st>>>(one, nullptr, nullptr, 0, tp, rows);
         return cudaGetLastError();
     }
     const int hal = tp.halo;
@@ -927,8 +976,8 @@ int strip_rows_single(int H, int W) {
 
 bool sfoc_batch_supported(const SteerTaps& st, const SmoothTaps& sm) { return steer_is_paper(st) && smooth_is_paper(sm); }
 
-void sfoc_batch_tiles(int H, int W, int* steer_ctas, int* smooth_ctas) {
-    *steer_ctas = ((W + kTW - 1) / kTW) * ((H + kTH - 1) / kTH);
+void sfoc_batch_tiles(int H, int W, int* n_steer, int* smooth_ctas) {
+    *n_steer = steer_ctas(H, W, steer_rows(H));
     const int rows = strip_rows(H);
     *smooth_ctas = ((W + kStW - 1) / kStW) * ((H + rows - 1) / rows);
 }
@@ -940,12 +989,8 @@ cudaError_t launch_sfoc_batch(const ImgJob* jobs, int n_jobs, const int* steer_b
     if (!sfoc_batch_supported(st, sm)) return cudaErrorNotSupported;
     ImgJob none;
     memset(&none, 0, sizeof(none));
-    auto kern = k_sfoc_steer_ct<float, 2, 3, 3, 5>;
-    const size_t smem = sizeof(float) * 9 * (size_t)(kTH + 10) * kTW;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<steer_ctas, kThreads, smem, s>>>(none, jobs, steer_begin, n_jobs, st);
-    e = cudaGetLastError();
+    k_sfoc_steer_strip<float><<<steer_ctas, kSrThreads, 0, s>>>(none, jobs, steer_begin, n_jobs, st, 0);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_smooth_paper(none, jobs, smooth_begin, n_jobs, smooth_ctas, 0, sm, s);
 }
