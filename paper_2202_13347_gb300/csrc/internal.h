@@ -148,10 +148,13 @@ constexpr long long kIntNonFinite = 1ll << 46;
 constexpr long long kIntNonFiniteMin = 1ll << 45;
 __host__ __device__ inline double int_units_to_double(long long v) { return (double)v * (1.0 / 268435456.0); }
 // one pixel value in those units (the integral images and the template sums
-// round every pixel with this one function)
+// round every pixel with this one function).  The units of a valid value (below
+// 5.7) fit 32 bits, and the 32-bit conversion gives the same integer as the
+// 64-bit one, which runs on the FP64 pipe (64 clocks a warp) and held the
+// kernels that round every pixel.
 __device__ __forceinline__ unsigned long long int_quant(float v) {
     if (!isfinite(v)) return (unsigned long long)kIntNonFinite;
-    return (unsigned long long)__float2ll_rn(v * kIntScale);
+    return (unsigned long long)(long long)__float2int_rn(v * kIntScale);
 }
 
 size_t integral_scratch_bytes(int H, int W);

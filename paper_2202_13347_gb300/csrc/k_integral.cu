@@ -12,12 +12,21 @@
 // sums of valid values stay below 2^45 (see internal.h), so a window sum at
 // or above 2^45 marks a window with a non-finite value.
 //
-// Three steps over 64 x 64 tiles:
+// Steps over tiles of 128 columns x 64 rows:
 //   k_int_tilesums  per tile: column sums and row sums (reads s1, s2 once)
-//   k_int_lines     P on the tile grid lines: running sums over the tiles
-//                   above (left), then a scan along the line
+//   k_int_carry     running sums of those over the tiles above (left)
+//   k_int_lines     P on the tile grid lines: a scan along each line
 //   k_int_final     per tile: local 2-D prefix + the grid-line values
-// HBM traffic is ~8 B/px read twice + 16 B/px written.
+// HBM traffic is ~8 B/px read twice + 16 B/px written: 15 us of HBM time for a
+// 2048 x 2048 cube.  A CTA takes one tile of one plane, a warp eight of its
+// rows with four columns per lane: all eight rows' loads are in flight at once,
+// a row's prefix is a lane's own three adds and one warp scan, and the eight
+// warps meet once, at a table of their column sums.  (64 x 64 tiles in shared
+// memory, where one thread per row and then per column adds 64 dependent
+// entries, took twice the time; a single warp per tile, eight or four rows of
+// loads in flight at a time, lost to them: the latency of 64 rows in a row.)
+// 2048 x 2048, tilesums + carry + lines + final: 40 + 7 + 10 + 54 -> 15 + 6 + 9 + 30
+// us; 512 x 512: 6 + 3 + 4 + 8 us.
 #include <math.h>
 #include <string.h>
 
@@ -27,7 +36,9 @@ namespace sfoc {
 
 namespace {
 
-constexpr int kT = 64;
+constexpr int kTR = 64, kTC = 128;  // tile rows and columns
+constexpr int kIR = 8;              // rows per warp of the tile kernels
+constexpr int kIntWarps = kTR / kIR;
 typedef unsigned long long u64;
 
 __device__ __forceinline__ u64 quant(float v) { return int_quant(v); }
@@ -44,8 +55,8 @@ IntLayout layout(int H, int W, void* scratch) {
     IntLayout L;
     L.H = H;
     L.W = W;
-    L.nty = (H + kT - 1) / kT;
-    L.ntx = (W + kT - 1) / kT;
+    L.nty = (H + kTR - 1) / kTR;
+    L.ntx = (W + kTC - 1) / kTC;
     u64* p = static_cast<u64*>(scratch);
     L.colsum = p;
     p += 2 * (size_t)L.nty * W;
@@ -73,12 +84,12 @@ struct IntCtas {
 };
 
 IntCtas int_ctas(int H, int W) {
-    const int nty = (H + kT - 1) / kT, ntx = (W + kT - 1) / kT;
+    const int nty = (H + kTR - 1) / kTR, ntx = (W + kTC - 1) / kTC;
     IntCtas c;
-    c.tiles = ntx * nty;
+    c.tiles = 2 * ntx * nty;
     c.carry = (2 * W + 2 * H + 255) / 256;
     c.lines = 2 * nty + 2 * ntx;
-    c.fin = 2 * ntx * nty;
+    c.fin = c.tiles;
     return c;
 }
 
@@ -101,36 +112,80 @@ __device__ __forceinline__ const IntJob& int_job(const IntJob& one, const IntJob
     return jobs[lo];
 }
 
-__global__ void __launch_bounds__(256) k_int_tilesums(const __grid_constant__ IntJob one, const IntJob* __restrict__ jobs,
-                                                       const int* __restrict__ begin, int n_jobs) {
-    __shared__ u64 t[kT][kT + 1];
-    int local;
+// this warp's rows y .. y + kIR - 1 at the lane's columns x .. x + 3 (x a multiple
+// of 4), zero past the image: rows are pitch (a multiple of 32) floats, so the
+// load stays inside the row
+__device__ __forceinline__ void int_rows(const float* __restrict__ s, size_t pitch, int y, int x, int H, int W,
+                                         float4 (&f)[kIR]) {
+#pragma unroll
+    for (int r = 0; r < kIR; ++r) {
+        f[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (x < W && y + r < H) f[r] = *reinterpret_cast<const float4*>(s + (size_t)(y + r) * pitch + x);
+    }
+}
+
+// four columns' values rounded; zero past the image, whatever the row's padding holds
+__device__ __forceinline__ void int_quant4(const float4& f, int x, int W, u64 (&q)[4]) {
+    q[0] = x < W ? quant(f.x) : 0ull;
+    q[1] = x + 1 < W ? quant(f.y) : 0ull;
+    q[2] = x + 2 < W ? quant(f.z) : 0ull;
+    q[3] = x + 3 < W ? quant(f.w) : 0ull;
+}
+
+// the tile of this CTA: plane *p, tile row *ty and column *tx
+__device__ __forceinline__ void int_tile(const IntLayout& L, int local, int* p, int* ty, int* tx) {
+    const int n = L.ntx * L.nty;
+    *p = local >= n ? 1 : 0;
+    local -= *p * n;
+    *ty = local / L.ntx;
+    *tx = local - *ty * L.ntx;
+}
+
+__global__ void __launch_bounds__(32 * kIntWarps)
+    k_int_tilesums(const __grid_constant__ IntJob one, const IntJob* __restrict__ jobs, const int* __restrict__ begin,
+                   int n_jobs) {
+    __shared__ __align__(16) u64 s_col[kIntWarps][kTC];
+    int local, p, ty, tx;
     const IntJob& J = int_job(one, jobs, begin, n_jobs, &local);
     const IntLayout& L = J.L;
-    const float* __restrict__ s1 = J.s1;
-    const float* __restrict__ s2 = J.s2;
-    const size_t pitch = J.pitch;
-    const int ty = local / L.ntx, tx = local - (local / L.ntx) * L.ntx;
-    const int y0 = ty * kT, x0 = tx * kT;
-    for (int p = 0; p < 2; ++p) {
-        const float* s = p ? s2 : s1;
-        __syncthreads();
-        for (int i = threadIdx.x; i < kT * kT; i += 256) {
-            int r = i / kT, c = i % kT;
-            int y = y0 + r, x = x0 + c;
-            t[r][c] = (y < L.H && x < L.W) ? quant(s[(size_t)y * pitch + x]) : 0ull;
-        }
-        __syncthreads();
-        const int role = threadIdx.x / kT, j = threadIdx.x % kT;  // roles 0,1: columns; 2,3: rows (half each)
-        if (role == 0) {
-            u64 acc = 0;
-            for (int r = 0; r < kT; ++r) acc += t[r][j];
-            if (x0 + j < L.W) L.colsum[((size_t)p * L.nty + ty) * L.W + x0 + j] = acc;
-        } else if (role == 1) {
-            u64 acc = 0;
-            for (int c = 0; c < kT; ++c) acc += t[j][c];
-            if (y0 + j < L.H) L.rowsum[((size_t)p * L.ntx + tx) * L.H + y0 + j] = acc;
-        }
+    int_tile(L, local, &p, &ty, &tx);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, H = L.H, W = L.W;
+    const int x0 = tx * kTC, x = x0 + 4 * lane, y0 = ty * kTR + w * kIR;
+    float4 f[kIR];
+    int_rows(p ? J.s2 : J.s1, J.pitch, y0, x, H, W, f);
+    u64 col[4] = {0ull, 0ull, 0ull, 0ull}, rs[kIR];  // rs: this lane's part of each row's sum
+#pragma unroll
+    for (int r = 0; r < kIR; ++r) {
+        u64 q[4];
+        int_quant4(f[r], x, W, q);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) col[c] += q[c];
+        rs[r] = (q[0] + q[1]) + (q[2] + q[3]);
+    }
+    *reinterpret_cast<ulonglong2*>(&s_col[w][4 * lane]) = make_ulonglong2(col[0], col[1]);
+    *reinterpret_cast<ulonglong2*>(&s_col[w][4 * lane + 2]) = make_ulonglong2(col[2], col[3]);
+    // lanes exchange halves of the rows: lane l of each eight ends with its eight's
+    // sum of row l, then the four eights are added
+#pragma unroll
+    for (int o = kIR / 2; o >= 1; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < kIR / 2; ++i)
+            if (i < o) {
+                const u64 give = up ? rs[i] : rs[i + o], keep = up ? rs[i + o] : rs[i];
+                rs[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+    }
+#pragma unroll
+    for (int o = kIR; o < 32; o <<= 1) rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], o);
+    if (lane < kIR && y0 + lane < H) L.rowsum[((size_t)p * L.ntx + tx) * H + y0 + lane] = rs[0];
+    __syncthreads();
+    const int t = threadIdx.x;
+    if (t < kTC && x0 + t < W) {
+        u64 a = 0;
+#pragma unroll
+        for (int k = 0; k < kIntWarps; ++k) a += s_col[k][t];
+        L.colsum[((size_t)p * L.nty + ty) * W + x0 + t] = a;
     }
 }
 
@@ -220,55 +275,93 @@ __global__ void __launch_bounds__(256) k_int_lines(const __grid_constant__ IntJo
     }
 }
 
-__global__ void __launch_bounds__(256) k_int_final(const __grid_constant__ IntJob one, const IntJob* __restrict__ jobs,
-                                                    const int* __restrict__ begin, int n_jobs) {
-    __shared__ u64 t[kT][kT + 1];
-    int local;
+__global__ void __launch_bounds__(32 * kIntWarps, 2)
+    k_int_final(const __grid_constant__ IntJob one, const IntJob* __restrict__ jobs, const int* __restrict__ begin,
+                int n_jobs) {
+    __shared__ __align__(16) u64 s_col[kIntWarps][kTC];
+    __shared__ __align__(16) u64 s_row[kIntWarps][2][kTC];
+    int local, p, ty, tx;
     const IntJob& J = int_job(one, jobs, begin, n_jobs, &local);
     const IntLayout& L = J.L;
-    const float* __restrict__ s1 = J.s1;
-    const float* __restrict__ s2 = J.s2;
-    const size_t pitch = J.pitch, ipitch = J.ipitch;
-    u64* __restrict__ P = J.P;
-    const int ntiles = L.ntx * L.nty;
-    const int p = local >= ntiles ? 1 : 0;
-    const int tl = local - p * ntiles;
-    const int ty = tl / L.ntx, tx = tl - (tl / L.ntx) * L.ntx;
-    const int y0 = ty * kT, x0 = tx * kT;
-    const float* s = p ? s2 : s1;
-    u64* Pp = P + (size_t)p * (L.H + 1) * ipitch;
-    for (int i = threadIdx.x; i < kT * kT; i += 256) {
-        int r = i / kT, c = i % kT;
-        int y = y0 + r, x = x0 + c;
-        t[r][c] = (y < L.H && x < L.W) ? quant(s[(size_t)y * pitch + x]) : 0ull;
-    }
-    __syncthreads();
-    // row prefix, then column prefix (one thread per row / column: 64 integer adds)
-    if (threadIdx.x < kT) {
-        u64 a = 0;
-        for (int c = 0; c < kT; ++c) { a += t[threadIdx.x][c]; t[threadIdx.x][c] = a; }
-    }
-    __syncthreads();
-    if (threadIdx.x < kT) {
-        u64 a = 0;
-        for (int r = 0; r < kT; ++r) { a += t[r][threadIdx.x]; t[r][threadIdx.x] = a; }
-    }
-    __syncthreads();
-    const u64* top = &L.top[((size_t)p * L.nty + ty) * (L.W + 1)];
-    const u64* left = &L.left[((size_t)p * L.ntx + tx) * (L.H + 1)];
+    int_tile(L, local, &p, &ty, &tx);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, H = L.H, W = L.W;
+    const size_t ipitch = J.ipitch;
+    u64* const Pp = J.P + (size_t)p * (H + 1) * ipitch;
+    const u64* const top = &L.top[((size_t)p * L.nty + ty) * (W + 1)];
+    const u64* const left = &L.left[((size_t)p * L.ntx + tx) * (H + 1)];
+    const int x0 = tx * kTC, x = x0 + 4 * lane, y0 = ty * kTR + w * kIR;
+    float4 f[kIR];
+    int_rows(p ? J.s2 : J.s1, J.pitch, y0, x, H, W, f);
+    // run[c]: P at column x + c down to the current row, less the line left of the
+    // tile; it starts with the line above the tile
     const u64 corner = top[x0];
-    for (int i = threadIdx.x; i < kT * kT; i += 256) {
-        int r = i / kT, c = i % kT;
-        int y = y0 + r, x = x0 + c;
-        if (y < L.H && x < L.W) Pp[(size_t)(y + 1) * ipitch + (x + 1)] = top[x + 1] + (left[y + 1] - corner) + t[r][c];
+    u64 run[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) run[c] = (x + c < W ? top[x + c + 1] : 0ull) - corner;
+    const u64 lft = lane < kIR && y0 + lane < H ? left[y0 + lane + 1] : 0ull;
+    u64 pre[kIR][4], ex[kIR];  // the tile rows' prefixes
+#pragma unroll
+    for (int r = 0; r < kIR; ++r) {
+        int_quant4(f[r], x, W, pre[r]);
+        pre[r][1] += pre[r][0];
+        pre[r][2] += pre[r][1];
+        pre[r][3] += pre[r][2];
+        ex[r] = pre[r][3];
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int r = 0; r < kIR; ++r) {
+            const u64 v = __shfl_up_sync(0xffffffffu, ex[r], o);
+            ex[r] += lane >= o ? v : 0ull;
+        }
+    u64 col[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+    for (int r = 0; r < kIR; ++r) {
+        const u64 before = ex[r] - pre[r][3];  // the lanes to the left
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            pre[r][c] += before;
+            col[c] += pre[r][c];
+        }
+    }
+    *reinterpret_cast<ulonglong2*>(&s_col[w][4 * lane]) = make_ulonglong2(col[0], col[1]);
+    *reinterpret_cast<ulonglong2*>(&s_col[w][4 * lane + 2]) = make_ulonglong2(col[2], col[3]);
+    __syncthreads();
+    for (int k = 0; k < w; ++k) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&s_col[k][4 * lane]);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&s_col[k][4 * lane + 2]);
+        run[0] += a.x;
+        run[1] += a.y;
+        run[2] += b.x;
+        run[3] += b.y;
+    }
+    u64 (*row)[kTC] = s_row[w];
+#pragma unroll
+    for (int r = 0; r < kIR; ++r) {
+        const int y = y0 + r;
+        const u64 l = __shfl_sync(0xffffffffu, lft, r);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) run[c] += pre[r][c];
+        // through shared memory, so that a store instruction writes 32 adjacent
+        // entries (rows of W + 1 entries keep no wider alignment); two rows
+        // alternate, so one warp barrier orders each
+        u64* const buf = row[r & 1];
+        *reinterpret_cast<ulonglong2*>(buf + 4 * lane) = make_ulonglong2(run[0] + l, run[1] + l);
+        *reinterpret_cast<ulonglong2*>(buf + 4 * lane + 2) = make_ulonglong2(run[2] + l, run[3] + l);
+        __syncwarp();
+        u64* const out = Pp + (size_t)(y + 1) * ipitch + x0 + 1;
+        if (y < H)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (x0 + 32 * c + lane < W) out[32 * c + lane] = buf[32 * c + lane];
     }
     // zero first row / column
-    if (ty == 0)
-        for (int c = threadIdx.x; c < kT; c += 256)
-            if (x0 + c < L.W) Pp[x0 + c + 1] = 0;
-    if (tx == 0)
-        for (int r = threadIdx.x; r < kT; r += 256)
-            if (y0 + r < L.H) Pp[(size_t)(y0 + r + 1) * ipitch] = 0;
+    if (ty == 0 && w == 0)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (x0 + 32 * c + lane < W) Pp[x0 + 32 * c + lane + 1] = 0;
+    if (tx == 0 && lane < kIR && y0 + lane < H) Pp[(size_t)(y0 + lane + 1) * ipitch] = 0;
     if (tx == 0 && ty == 0 && threadIdx.x == 0) Pp[0] = 0;
 }
 
@@ -326,7 +419,7 @@ cudaError_t launch_integral_export(const Cube& c, void* scratch, double* out, cu
 }
 
 size_t integral_scratch_bytes(int H, int W) {
-    size_t nty = (H + kT - 1) / kT, ntx = (W + kT - 1) / kT;
+    size_t nty = (H + kTR - 1) / kTR, ntx = (W + kTC - 1) / kTC;
     return sizeof(u64) * (2 * nty * W + 2 * ntx * H + 2 * nty * (W + 1) + 2 * ntx * (H + 1));
 }
 
@@ -348,10 +441,10 @@ IntJob int_job_of(const Cube& c, void* scratch) {
 cudaError_t launch_integral(const Cube& c, void* scratch, cudaStream_t st, int* launches) {
     const IntJob one = int_job_of(c, scratch);
     const IntCtas n = int_ctas(c.H, c.W);
-    k_int_tilesums<<<n.tiles, 256, 0, st>>>(one, nullptr, nullptr, 0);
+    k_int_tilesums<<<n.tiles, 32 * kIntWarps, 0, st>>>(one, nullptr, nullptr, 0);
     k_int_carry<<<n.carry, 256, 0, st>>>(one, nullptr, nullptr, 0);
     k_int_lines<<<n.lines, 256, 0, st>>>(one, nullptr, nullptr, 0);
-    k_int_final<<<n.fin, 256, 0, st>>>(one, nullptr, nullptr, 0);
+    k_int_final<<<n.fin, 32 * kIntWarps, 0, st>>>(one, nullptr, nullptr, 0);
     if (launches) *launches += 4;
     return cudaGetLastError();
 }
@@ -396,10 +489,10 @@ cudaError_t launch_integral_batch(const void* d_blob, int n, const int* ctas4, c
         reinterpret_cast<const int*>(static_cast<const char*>(d_blob) + ((sizeof(IntJob) * (size_t)n + 15) / 16) * 16);
     IntJob none;
     memset(&none, 0, sizeof(none));
-    k_int_tilesums<<<ctas4[0], 256, 0, st>>>(none, jobs, pre, n);
+    k_int_tilesums<<<ctas4[0], 32 * kIntWarps, 0, st>>>(none, jobs, pre, n);
     k_int_carry<<<ctas4[1], 256, 0, st>>>(none, jobs, pre + (n + 1), n);
     k_int_lines<<<ctas4[2], 256, 0, st>>>(none, jobs, pre + 2 * (n + 1), n);
-    k_int_final<<<ctas4[3], 256, 0, st>>>(none, jobs, pre + 3 * (n + 1), n);
+    k_int_final<<<ctas4[3], 32 * kIntWarps, 0, st>>>(none, jobs, pre + 3 * (n + 1), n);
     return cudaGetLastError();
 }
 
