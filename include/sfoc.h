@@ -443,19 +443,24 @@ SFOC_API sfoc_status sfoc_ctx_plan_info(const sfoc_ctx* ctx, char* buf, size_t c
  * With SFOC_CORR_AUTO (family 0) and SFOC_CORR_IGEMM_TC (family 1) the
  * correlation form of a (cube dtype, m, R) is measured, not ruled: on the
  * first match of that key (outside a stream capture) every form of the
- * family that runs for it is launched on the first min(n, 2 x SMs) points
+ * family that runs for it is launched on the first min(n, 4 x SMs) points
  * of that call (one warm-up launch, then the better of two timed with CUDA
  * events), and the fastest is kept in the context and used from then on.
- *   family 0, F32 cubes:  the Fourier correlation (where m + 2R <= 64 also
- *                         with its 128-point transform) and the direct kernel;
+ *   family 0, F32 cubes:  the Fourier correlation (sides 64 and 128; where
+ *                         m + 2R is in (64, 96] also 96, in (128, 224] also
+ *                         160, 192 or 224, the least that holds it; where
+ *                         m + 2R <= 64 also 128) and the direct kernel;
  *   family 0, BF16 cubes: the band, column and Toeplitz tensor-core forms and
- *                         the Fourier correlation (reading the bf16 cube);
+ *                         the Fourier correlation of the same sides (reading
+ *                         the bf16 cube);
  *   family 1 (BF16):      the tensor-core forms only.
  * The paper weighs its FFT against spatial correlation by operation counts
  * (Eq. 17-19); on this device the choice is made by measurement.  Without
  * an entry (autotuning off, or inside a capture) the fixed rule: F32 cubes
- * the Fourier form when m + 2R <= 128, else the direct kernel; BF16 cubes
- * the tensor-core form with the fewest MMAs.
+ * the Fourier form when m + 2R <= 224, else the direct kernel; BF16 cubes
+ * the tensor-core form with the fewest MMAs.  (m, R) that neither side 128 nor
+ * one of the other kernels serves are refused, and an explicit SFOC_CORR_FFT
+ * stays with sides 64 and 128.
  */
 SFOC_API sfoc_status sfoc_ctx_set_autotune(sfoc_ctx* ctx, int enable);
 /* The entry of (dtype, m, R): *corr_path = the chosen sfoc_corr_path (-1 when

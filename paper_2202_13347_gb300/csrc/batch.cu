@@ -141,6 +141,7 @@ int tc_form(int path) {
 int class_of(int path, int option, int m, int R) {
     switch (path) {
         case SFOC_CORR_FFT:
+            if (option == corr_fft2_side(m, R) && option) return option;
             if (!corr_fft_supported(m, R)) return 0;
             return option ? option : corr_fft_side(m, R);
         case SFOC_CORR_DIRECT_F32: return corr_f32_supported(m, R) ? corr_f32_class(R) : 0;
@@ -220,7 +221,9 @@ cudaError_t enqueue_match_tail(sfoc_ctx* ctx, BatchPlan* p, cudaStream_t s) {
             continue;
         }
         StageScope sc(ctx, ST_CORR, 1);
-        if (c.path == SFOC_CORR_FFT) e = launch_corr_fft(none, is, c.cls, p->dtype == SFOC_DTYPE_BF16, s);
+        if (c.path == SFOC_CORR_FFT && c.cls != 64 && c.cls != 128)
+            e = launch_corr_fft2(none, is, c.cls, p->dtype == SFOC_DTYPE_BF16, s);
+        else if (c.path == SFOC_CORR_FFT) e = launch_corr_fft(none, is, c.cls, p->dtype == SFOC_DTYPE_BF16, s);
         else if (c.path == SFOC_CORR_DIRECT_F32) e = launch_corr_f32(none, is, c.cls, s);
         else e = launch_corr_tc(tc_form(c.path), c.cls, none, is, c.ms.data(), c.Rs.data(), (int)c.ms.size(),
                                 ctx->d_err, s);
@@ -349,6 +352,7 @@ sfoc_status plan_build(sfoc_ctx* ctx, BatchPlan* p, const BuildIn& in, const sfo
         j.cpitch = c.pitch;
         j.rm = c.rm;
         j.cm = c.cm;
+        j.pl = c.pl;
         j.s1 = c.s1;
         j.s2 = c.s2;
         used += fb;

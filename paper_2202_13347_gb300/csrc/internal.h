@@ -63,12 +63,17 @@ struct SmoothTaps {
 //   cm: [2][W][H][8] (pixels column-major)  - templates; column-form windows
 // Both buffers carry 256 bytes of padding past the end (copies in 128-byte
 // runs of pixels may read up to 7 pixels past the last column).
+// A third copy, pl: planar [12][H][pitch] as the F32 cube, serves the Fourier
+// correlation, which takes one channel at a time: from rm a channel's pixels
+// are 2 bytes in every 16, and the L2 traffic of a point would be eight times
+// its values.
 struct Cube {
     int H = 0, W = 0, z = 0, dtype = SFOC_DTYPE_F32;
     size_t pitch = 0;          // elements per row of f32 planes / sum planes
     float* f32 = nullptr;      // [z][H][pitch]
     __nv_bfloat16* rm = nullptr;
     __nv_bfloat16* cm = nullptr;
+    __nv_bfloat16* pl = nullptr;
     float* s1 = nullptr;       // [H][pitch] sum over channels of g
     float* s2 = nullptr;       // [H][pitch] sum over channels of g^2
     unsigned long long* integ = nullptr;  // [2][H+1][ipitch] exclusive prefix of s1, s2 in units of 2^-28
@@ -94,6 +99,7 @@ struct ImgJob {
     size_t cpitch;
     __nv_bfloat16* rm; // BF16 cube layouts or nullptr
     __nv_bfloat16* cm;
+    __nv_bfloat16* pl;
     float* s1;         // per-pixel sums [H][cpitch]
     float* s2;
 };
@@ -190,8 +196,9 @@ struct MatchJob {  // aligned as its tensor maps (128 bytes)
     const float* rf32;
     const __nv_bfloat16* rrm;
     const __nv_bfloat16* rcm;
+    const __nv_bfloat16* rpl;
     const unsigned long long* rint;
-    size_t rpitch, rplane, ripitch;
+    size_t rpitch, rplane, ripitch;  // of the planar values (F32 or pl) and the integral images
     int Hr, Wr;
     // sensed (template) cube
     const float* sf32;
@@ -199,6 +206,7 @@ struct MatchJob {  // aligned as its tensor maps (128 bytes)
     const float* ss2;
     const __nv_bfloat16* srm;
     const __nv_bfloat16* scm;
+    const __nv_bfloat16* spl;
     size_t spitch, splane;
     int Hs, Ws;
     int z, m, R, n;
@@ -244,6 +252,13 @@ bool corr_f32_supported(int m, int R);
 cudaError_t launch_corr_f32(const MatchJob& one, const ItemSet& is, int tpt, cudaStream_t st);
 bool corr_fft_supported(int m, int R);
 int corr_fft_side(int m, int R);  // smallest transform side that serves (m, R): 64 or 128
+// The Fourier form by halves of the spectrum (k_corr_fft2.cu): the side that
+// serves (m, R), 96 for m + 2R in (64, 96] and 160, 192 or 224 above 128; 0
+// elsewhere.  AUTO takes it (the option of a measured entry is its side);
+// SFOC_CORR_FFT itself stays with sides 64 and 128.  bf16: the jobs' cubes are
+// BF16 (read from the planes pl).  Every item of a launch has side L.
+int corr_fft2_side(int m, int R);
+cudaError_t launch_corr_fft2(const MatchJob& one, const ItemSet& is, int L, bool bf16, cudaStream_t st);
 // bf16: the jobs' cubes are BF16 (read from the row-major chunk layout rm)
 cudaError_t launch_corr_fft(const MatchJob& one, const ItemSet& is, int L, bool bf16, cudaStream_t st);
 // tensor-core forms: 1 Toeplitz, 2 column, 3 band.  corr_tc_class: the

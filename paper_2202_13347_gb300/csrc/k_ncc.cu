@@ -290,6 +290,7 @@ MatchJob make_job(const Cube& ref, const Cube& sen, const int32_t* pts, int n, i
     j.rf32 = ref.f32;
     j.rrm = ref.rm;
     j.rcm = ref.cm;
+    j.rpl = ref.pl;
     j.rint = ref.integ;
     j.rpitch = ref.pitch;
     j.rplane = ref.pitch * (size_t)ref.H;
@@ -301,6 +302,7 @@ MatchJob make_job(const Cube& ref, const Cube& sen, const int32_t* pts, int n, i
     j.ss2 = sen.s2;
     j.srm = sen.rm;
     j.scm = sen.cm;
+    j.spl = sen.pl;
     j.spitch = sen.pitch;
     j.splane = sen.pitch * (size_t)sen.H;
     j.Hs = sen.H;

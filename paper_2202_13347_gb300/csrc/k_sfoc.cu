@@ -374,13 +374,14 @@ __device__ __forceinline__ void smooth_channel(const float* __restrict__ Fk, siz
 }
 
 // Normalises one pixel's group of `no` smoothed values d[k] (Sec. 2.1) and
-// writes it out: F32 planes, or the bf16 chunk in both pixel orders; adds
+// writes it out: F32 planes, or the bf16 chunk in both pixel orders and the
+// bf16 planes; adds
 // the stored values to the per-pixel sums a1 (g) and a2 (g^2).
 template <int NO, int KO>
 __device__ __forceinline__ void write_pixel(int g, int no, const float* d, float eps, int gy, int gx, int H, int W,
                                             float* __restrict__ c32, size_t cpitch, size_t cplane,
                                             __nv_bfloat16* __restrict__ rm, __nv_bfloat16* __restrict__ cm,
-                                            float& a1, float& a2) {
+                                            __nv_bfloat16* __restrict__ pl, float& a1, float& a2) {
     const bool bf = rm != nullptr;
     float n2 = 0.f;
 #pragma unroll
@@ -399,6 +400,7 @@ __device__ __forceinline__ void write_pixel(int g, int no, const float* d, float
         a1 += v;
         a2 = fmaf(v, v, a2);
         if (c32 && in) c32[(size_t)(g * no + k) * cplane + (size_t)gy * cpitch + gx] = v;
+        if (pl && in) pl[(size_t)(g * no + k) * cplane + (size_t)gy * cpitch + gx] = __float2bfloat16_rn(v);
     }
     if constexpr (NO == 6) {
         if (bf && in) {  // chunk g: the six channels, then two zeros
@@ -423,6 +425,7 @@ __device__ __forceinline__ void smooth_group(int g, const float* __restrict__ F,
                                              float* s_F, int FW, float* s_h, int HR, int x0,
                                              int y0, float* __restrict__ c32, size_t cpitch, size_t cplane,
                                              __nv_bfloat16* __restrict__ rm, __nv_bfloat16* __restrict__ cm,
+                                             __nv_bfloat16* __restrict__ pl,
                                              float (&a1)[kSRows], float (&a2)[kSRows]) {
     constexpr int KO = NO > 0 ? NO : kMaxOrient;
     const int no = NO > 0 ? NO : tp.no;
@@ -452,7 +455,7 @@ __device__ __forceinline__ void smooth_group(int g, const float* __restrict__ F,
         float d[KO];
 #pragma unroll
         for (int k = 0; k < KO; ++k) d[k] = D[k][j];
-        write_pixel<NO, KO>(g, no, d, tp.eps, y0 + rb + j, gx, H, W, c32, cpitch, cplane, rm, cm, a1[j], a2[j]);
+        write_pixel<NO, KO>(g, no, d, tp.eps, y0 + rb + j, gx, H, W, c32, cpitch, cplane, rm, cm, pl, a1[j], a2[j]);
     }
 }
 
@@ -556,6 +559,7 @@ struct StripOut {
     float* s2;
     float* c32;   // group g's first plane (or nullptr)
     uint4* rm;    // group g's chunks (or nullptr)
+    __nv_bfloat16* pl;  // group g's first bf16 plane (with rm)
     size_t pitch, plane;
     int W;
     bool two;     // the second pixel is inside the image
@@ -620,6 +624,12 @@ __device__ __forceinline__ void strip_finish(const StripOut& o, float eps, const
         for (int k = 0; k < 6; ++k, q += o.plane) put2(q, v[0][k], v[1][k]);
     }
     if (bf) {
+        // the planes: both columns in one store (gx is even and the pitch a multiple
+        // of 32, so the second one is inside the row's padding at worst)
+        __nv_bfloat16* q = o.pl + at;
+#pragma unroll
+        for (int k = 0; k < 6; ++k, q += o.plane)
+            *reinterpret_cast<unsigned*>(q) = __byte_perm(pk[0][k >> 1], pk[1][k >> 1], (k & 1) ? 0x7632 : 0x5410);
         uint4* const rm = o.rm + (size_t)gy * o.W;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {  // chunk g: the six channels, then two zeros
@@ -669,6 +679,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
         o.s2 = J.s2 + gx;
         o.c32 = J.c32 ? J.c32 + (size_t)g * 6 * plane + gx : nullptr;
         o.rm = J.rm ? reinterpret_cast<uint4*>(J.rm) + (size_t)g * H * W + gx : nullptr;
+        o.pl = J.pl ? J.pl + (size_t)g * 6 * plane + gx : nullptr;
         o.pitch = J.cpitch;
         o.plane = plane;
         o.W = W;
@@ -791,7 +802,8 @@ template <int NO>
 __global__ void __launch_bounds__(kThreads, 1)
     k_sfoc_smooth(const float* __restrict__ F, size_t fpitch, size_t fplane, int H, int W, SmoothTaps tp,
                   float* __restrict__ c32, size_t cpitch, size_t cplane, __nv_bfloat16* __restrict__ rm,
-                  __nv_bfloat16* __restrict__ cm, float* __restrict__ s1, float* __restrict__ s2) {
+                  __nv_bfloat16* __restrict__ cm, __nv_bfloat16* __restrict__ pl, float* __restrict__ s1,
+                  float* __restrict__ s2) {
     extern __shared__ float sm[];
     __shared__ float s_tap[2][kMaxSmoothRadius + 1];  // taps in shared memory: no local copy of the params
     __shared__ int s_dil[kMaxDil];
@@ -816,7 +828,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int j = 0; j < kSRows; ++j) a1[j] = a2[j] = 0.f;
     for (int g = 0; g < ng; ++g)
         smooth_group<NO>(g, F, fpitch, fplane, H, W, tp, s_dil, s_tap[g], s_F, FW, s_h, HR, x0, y0, c32, cpitch,
-                         cplane, rm, cm, a1, a2);
+                         cplane, rm, cm, pl, a1, a2);
 #pragma unroll
     for (int j = 0; j < kSRows; ++j) {
         const int gy = y0 + rb + j;
@@ -1010,6 +1022,7 @@ cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, cons
         one.cpitch = c.pitch;
         one.rm = c.rm;
         one.cm = c.cm;
+        one.pl = c.pl;
         one.s1 = c.s1;
         one.s2 = c.s2;
         const int rows = strip_rows_single(H, W);
@@ -1023,13 +1036,13 @@ cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, cons
         e = cudaFuncSetAttribute(k_sfoc_smooth<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_sfoc_smooth<6><<<grid, kThreads, smem, st>>>(F, fpitch, fpitch * (size_t)H, H, W, tp, c.f32, c.pitch,
-                                                       c.pitch * (size_t)H, c.rm, c.cm, c.s1, c.s2);
+                                                       c.pitch * (size_t)H, c.rm, c.cm, c.pl, c.s1, c.s2);
     } else {
         if (c.rm) return cudaErrorNotSupported;  // bf16 layouts need 12 channels
         e = cudaFuncSetAttribute(k_sfoc_smooth<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_sfoc_smooth<0><<<grid, kThreads, smem, st>>>(F, fpitch, fpitch * (size_t)H, H, W, tp, c.f32, c.pitch,
-                                                       c.pitch * (size_t)H, c.rm, c.cm, c.s1, c.s2);
+                                                       c.pitch * (size_t)H, c.rm, c.cm, c.pl, c.s1, c.s2);
     }
     return cudaGetLastError();
 }

@@ -213,11 +213,12 @@ void free_cube_mem(Cube& c) {
     cudaFree(c.f32);
     cudaFree(c.rm);
     cudaFree(c.cm);
+    cudaFree(c.pl);
     cudaFree(c.s1);
     cudaFree(c.s2);
     cudaFree(c.integ);
     c.f32 = nullptr;
-    c.rm = c.cm = nullptr;
+    c.rm = c.cm = c.pl = nullptr;
     c.s1 = c.s2 = nullptr;
     c.integ = nullptr;
 }
@@ -239,6 +240,7 @@ sfoc_status alloc_cube(sfoc_ctx* ctx, Cube& c, int H, int W, int z, int dtype) {
         // bytes past the last column
         e = cudaMalloc(&c.rm, sizeof(__nv_bfloat16) * 16 * (size_t)H * W + 256);
         if (e == cudaSuccess) e = cudaMalloc(&c.cm, sizeof(__nv_bfloat16) * 16 * (size_t)H * W + 256);
+        if (e == cudaSuccess) e = cudaMalloc(&c.pl, sizeof(__nv_bfloat16) * plane * z);
     }
     if (e == cudaSuccess) e = cudaMalloc(&c.s1, sizeof(float) * plane);
     if (e == cudaSuccess) e = cudaMalloc(&c.s2, sizeof(float) * plane);
@@ -279,6 +281,8 @@ cudaError_t launch_corr_path(sfoc_ctx* ctx, int path, int option, MatchJob& one)
             return launch_corr_f32(one, none, c, ctx->stream);
         }
         case SFOC_CORR_FFT: {
+            if (option && option == corr_fft2_side(m, R))
+                return launch_corr_fft2(one, none, option, one.rf32 == nullptr, ctx->stream);
             if (!corr_fft_supported(m, R)) return cudaErrorNotSupported;
             return launch_corr_fft(one, none, option ? option : corr_fft_side(m, R), one.rf32 == nullptr,
                                    ctx->stream);
@@ -307,7 +311,11 @@ int auto_rule(int dtype, int m, int R, int family) {
     }
     if (family != 0) return -1;
     if (corr_fft_supported(m, R)) return SFOC_CORR_FFT;
-    return corr_f32_supported(m, R) ? SFOC_CORR_DIRECT_F32 : -1;
+    // beyond, whatever the direct kernel serves (nothing else was ever accepted),
+    // by the Fourier form where that has a side: 4 us a point against 120 at
+    // m = 80, R = 60, 1.6 against 40 at m = 81, R = 36
+    if (!corr_f32_supported(m, R)) return -1;
+    return corr_fft2_side(m, R) ? SFOC_CORR_FFT : SFOC_CORR_DIRECT_F32;
 }
 
 const TuneEntry* autotune_pair(sfoc_ctx* ctx, int dtype, int family, MatchJob one) {
@@ -328,12 +336,17 @@ const TuneEntry* autotune_pair(sfoc_ctx* ctx, int dtype, int family, MatchJob on
         add(SFOC_CORR_FFT, side);
         if (side == 64) add(SFOC_CORR_FFT, 128);  // the larger transform as a tile option
     }
+    // (m, R) that no other form serves stay refused, so beyond m + 2R = 128 this
+    // side is a candidate only beside one
+    const int side2 = corr_fft2_side(m, R);
+    if (family == 0 && side2 && auto_rule(dtype, m, R, 0) >= 0) add(SFOC_CORR_FFT, side2);
     if (family == 0 && dtype == SFOC_DTYPE_F32 && corr_f32_supported(m, R)) add(SFOC_CORR_DIRECT_F32, 0);
     if (t.n_cand == 0) return nullptr;
-    // a sample of up to two waves of points, timed per candidate: one
+    // a sample of up to four points per SM (the Fourier form of side 96 runs four
+    // CTAs on one), timed per candidate: one
     // warm-up launch, then the better of two
     const int sms = sm_count(ctx->device);
-    one.n = one.n < 2 * sms ? one.n : 2 * sms;
+    one.n = one.n < 4 * sms ? one.n : 4 * sms;
     t.sample = one.n;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     for (auto& e : ev)
@@ -382,7 +395,9 @@ int resolve_path(sfoc_ctx* ctx, int path, int dtype, const MatchJob* one, bool m
         *option = te->option;
         return te->path;
     }
-    return auto_rule(dtype, m, R, family);
+    const int rule = auto_rule(dtype, m, R, family);
+    if (rule == SFOC_CORR_FFT && !corr_fft_supported(m, R)) *option = corr_fft2_side(m, R);
+    return rule;
 }
 
 }  // namespace sfoc
@@ -1064,9 +1079,12 @@ sfoc_status sfoc_ctx_autotune_import(sfoc_ctx* ctx, const char* text) {
             m < 1 || m > kMaxTemplate || R < 0 || R > kMaxRadius)
             return fail(ctx, SFOC_ERR_INVALID_ARG, "autotune entry out of range");
         const int opt = t.path == SFOC_CORR_FFT ? t.option : 0;
-        if (t.path == SFOC_CORR_FFT && (opt != 64 && opt != 128)) return fail(ctx, SFOC_ERR_INVALID_ARG, "bad FFT side");
+        const bool half = t.path == SFOC_CORR_FFT && opt && opt == corr_fft2_side(m, R);
+        if (t.path == SFOC_CORR_FFT && !half && opt != 64 && opt != 128)
+            return fail(ctx, SFOC_ERR_INVALID_ARG, "bad FFT side");
         // the entry must name a form that runs for (m, R)
-        if (t.path == SFOC_CORR_FFT ? (!corr_fft_supported(m, R) || m + 2 * R > opt)
+        if (half ? auto_rule(dtype, m, R, 0) < 0
+            : t.path == SFOC_CORR_FFT ? (!corr_fft_supported(m, R) || m + 2 * R > opt)
             : t.path == SFOC_CORR_DIRECT_F32 ? !corr_f32_supported(m, R)
                                              : corr_tc_class(t.path == SFOC_CORR_TC_TOEPLITZ ? 1
                                                              : t.path == SFOC_CORR_TC_COLUMN ? 2 : 3, m, R) == 0)
