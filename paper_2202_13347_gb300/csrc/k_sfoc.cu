@@ -512,31 +512,42 @@ __host__ __device__ inline int strip_rows(int H) {
 }
 
 // Copies kStU rows of one channel from row i0 (clamped to the image) into dst;
-// one commit group.  Strips whose window lies inside the rows copy 16-byte
-// pieces (rows and x0 - OFF are 16-byte aligned); others element by element
-// with clamped columns.
+// one commit group.  Pieces of 16 bytes inside the rows (rows and x0 - OFF are
+// 16-byte aligned), and on the image's left and right strips the clamped columns
+// one by one, 16 of a row at a time.  (Copying such a strip's rows element by
+// element made its CTAs issue 1.4 times the instructions of the others, and a
+// launch of one wave waited for them: 512 x 512 19.4 and 25.9 us for groups 0 and
+// 1, with this 17.5 and 23.6; 2048 x 2048, two of 32 strips, 146 -> 141.5 for
+// group 1.)
 template <int KD>
 __device__ __forceinline__ void strip_rows_async(const float* __restrict__ Fk, size_t fpitch, int H, int W, int x0,
                                                  int i0, float* dst, int lane) {
     using G = StripGeom<KD>;
+    static_assert(G::OFF <= 16 && G::RW / 4 <= 32, "a lane per piece, one step left of the image");
     const int xs = x0 - G::OFF;
-    if (xs >= 0 && xs + G::RW <= W) {
+    const int xl = xs + 4 * lane;
+    const bool whole = lane < G::RW / 4 && xl >= 0 && xl + 4 <= W;
 #pragma unroll
-        for (int u = 0; u < kStU; ++u) {
-            const float* src = Fk + (size_t)clampi(i0 + u, 0, H - 1) * fpitch + xs + 4 * lane;
-            const unsigned d = (unsigned)__cvta_generic_to_shared(dst + u * G::RW + 4 * lane);
-            if (lane < G::RW / 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-        }
-    } else {
-        for (int u = 0; u < kStU; ++u) {
-            const float* row = Fk + (size_t)clampi(i0 + u, 0, H - 1) * fpitch;
-            for (int c = lane; c < G::RW; c += 32) {
+    for (int u = 0; u < kStU; ++u) {
+        const float* src = Fk + (size_t)clampi(i0 + u, 0, H - 1) * fpitch + xl;
+        const unsigned d = (unsigned)__cvta_generic_to_shared(dst + u * G::RW + 4 * lane);
+        if (whole) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    }
+    auto clamped = [&](int c0, int c1) {  // columns [c0, min(c0 + 16, c1)) of the staged rows
+        const int c = c0 + (lane & 15);
+        const float* col = Fk + clampi(xs + c, 0, W - 1);
+        if (c < c1)
+#pragma unroll
+            for (int u = lane >> 4; u < kStU; u += 2) {
                 const unsigned d = (unsigned)__cvta_generic_to_shared(dst + u * G::RW + c);
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(row + clampi(xs + c, 0, W - 1))
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d),
+                             "l"(col + (size_t)clampi(i0 + u, 0, H - 1) * fpitch)
                              : "memory");
             }
-        }
-    }
+    };
+    if (xs < 0) clamped(0, -xs);
+    // (W > x0, so the first piece that is not whole is right of those)
+    for (int c0 = (W & ~3) - xs; c0 < G::RW; c0 += 16) clamped(c0, G::RW);
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
