@@ -40,6 +40,11 @@ struct FftShape {
     static constexpr int G = L / 2;                     // groups of 8 threads
     static constexpr int T = 8 * G;                     // threads
     static constexpr int ZP = L + 2;                    // row pitch of the L x L array (float2)
+    // CTAs per SM.  At L = 64 a CTA is 8 warps that wait for each other at every
+    // pass; two fill one another's gaps: 2000 points of m = 41, R = 10 take 388 us
+    // instead of 634 (F32 cubes; BF16 395 instead of 540), 100 points 38 as before.
+    // At 128 the L x L array leaves room for one.
+    static constexpr int MINB = L == 64 ? 2 : 1;
     // scratch per group (float2): 8 rows per array, both arrays of the dual
     // transform (16 rows), or E rows of one; consecutive groups 64 B apart mod 128
     static constexpr int SG = (E < 16 ? 16 : E) * kScP + 8;
@@ -193,44 +198,35 @@ __device__ __forceinline__ float2 cross_spectrum(float2 a, float2 b) {
 
 // Rows of one item's window (or template) in a cube: `p` points at channel
 // 0, row 0, column 0 of the region; row(c, y) is channel c, region row y.
-// F32 cubes: planar, `pitch` elements per row, `plane` per channel.  BF16
-// cubes: the row-major chunks (chunk c / 6, lane c % 6 of a pixel's 8),
-// widened to FP32 as read; `pitch` = 8 W elements per row, `plane` = 8 H W
-// per chunk.
-struct CubeF32 {
-    const float* p;
+// Planes of F32 cubes, or the planes pl of BF16 cubes widened to FP32 as read:
+// `pitch` elements per row, `plane` per channel.  (From the row-major
+// chunks, 2 bytes in every 16, a BF16 point of m = 81, R = 20 took 1.01 us, from
+// the planes 0.85: F32 cubes take 0.83.)
+template <typename T>
+struct CubePlanes {
+    const T* p;
     size_t plane;
     unsigned pitch;
-    __device__ __forceinline__ const float* row(int c, int y) const {
+    __device__ __forceinline__ const T* row(int c, int y) const {
         return p + (size_t)c * plane + (size_t)y * pitch;
     }
-    __device__ __forceinline__ static float at(const float* r, int x) { return r[x]; }
-};
-struct CubeBF16 {
-    const __nv_bfloat16* p;
-    size_t plane;
-    unsigned pitch;
-    __device__ __forceinline__ const __nv_bfloat16* row(int c, int y) const {
-        const int g = c / 6;
-        return p + (size_t)g * plane + (size_t)y * pitch + (c - 6 * g);
-    }
-    __device__ __forceinline__ static float at(const __nv_bfloat16* r, int x) { return __bfloat162float(r[8 * x]); }
+    __device__ __forceinline__ static float at(const T* r, int x) { return (float)r[x]; }
 };
 
 // Items: the points of `one` (items == nullptr) or (job, point) pairs of a
 // batch; with a queue the CTAs take items from an atomic counter (points of
 // uneven cost balance across the SMs), else item k goes to CTA k mod grid.
-// BF: the jobs' cubes are BF16 (12 channels), read from the row-major layout.
+// BF: the jobs' cubes are BF16 (12 channels), read from their planes.
 template <int L, bool BF>
-__global__ void __launch_bounds__(FftShape<L>::T, 1)
+__global__ void __launch_bounds__(FftShape<L>::T, FftShape<L>::MINB)
     k_corr_fft(const __grid_constant__ MatchJob one, const MatchJob* __restrict__ jobs,
                const int2* __restrict__ items, int n_items, int* __restrict__ queue) {
     using Sh = FftShape<L>;
     constexpr int E = Sh::E, ZP = Sh::ZP, kFftGroups = Sh::G, kFftThreads = Sh::T;
     extern __shared__ __align__(16) float2 fsm[];
     __shared__ int s_item;
-    typedef typename std::conditional<BF, CubeBF16, CubeF32>::type SrcT;
-    __shared__ SrcT s_src[2];  // the item's window and template rows
+    typedef CubePlanes<typename std::conditional<BF, __nv_bfloat16, float>::type> Src;
+    __shared__ Src s_src[2];  // the item's window and template rows
     __shared__ float* s_out;
     __shared__ int s_par[4];   // the item's m, m + 2R, 2R + 1, channels
     __shared__ float s_tmean;  // the item's template mean
@@ -280,7 +276,6 @@ __global__ void __launch_bounds__(FftShape<L>::T, 1)
         const MatchJob& J = item_job(one, jobs, items, kk, &k);
         const PointStat st = J.stats[k];
         if (st.status != SFOC_PT_OK) continue;  // uniform across the CTA
-        typedef typename std::conditional<BF, CubeBF16, CubeF32>::type Src;
         const int m = J.m, R = J.R, z = J.z;
         const int P1 = 2 * R + 1, Lw = m + 2 * R;
         const int h = template_half(m);
@@ -296,11 +291,11 @@ __global__ void __launch_bounds__(FftShape<L>::T, 1)
             const int ty0 = J.pts[2 * k + 1] - h, tx0 = J.pts[2 * k] - h;
             const int wy0 = ty0 - R, wx0 = tx0 - R;
             if constexpr (BF) {
-                s_src[0] = CubeBF16{J.rrm + ((size_t)wy0 * J.Wr + wx0) * 8, (size_t)8 * J.Hr * J.Wr, 8u * (unsigned)J.Wr};
-                s_src[1] = CubeBF16{J.srm + ((size_t)ty0 * J.Ws + tx0) * 8, (size_t)8 * J.Hs * J.Ws, 8u * (unsigned)J.Ws};
+                s_src[0] = Src{J.rpl + (size_t)wy0 * J.rpitch + wx0, J.rplane, (unsigned)J.rpitch};
+                s_src[1] = Src{J.spl + (size_t)ty0 * J.spitch + tx0, J.splane, (unsigned)J.spitch};
             } else {
-                s_src[0] = CubeF32{J.rf32 + (size_t)wy0 * J.rpitch + wx0, J.rplane, (unsigned)J.rpitch};
-                s_src[1] = CubeF32{J.sf32 + (size_t)ty0 * J.spitch + tx0, J.splane, (unsigned)J.spitch};
+                s_src[0] = Src{J.rf32 + (size_t)wy0 * J.rpitch + wx0, J.rplane, (unsigned)J.rpitch};
+                s_src[1] = Src{J.sf32 + (size_t)ty0 * J.spitch + tx0, J.splane, (unsigned)J.spitch};
             }
             s_out = J.maps + (size_t)k * P1 * P1;
             s_par[0] = m;
@@ -436,7 +431,7 @@ cudaError_t launch_corr_fft(const MatchJob& one, const ItemSet& is, int L, bool 
     if (n <= 0) return cudaSuccess;
     const int lw = is.items ? is.max_lw : one.m + 2 * one.R;
     if ((L != 64 && L != 128) || lw > L) return cudaErrorNotSupported;
-    if (!is.items && (bf16 ? (one.rrm == nullptr || one.srm == nullptr || one.z != 12)
+    if (!is.items && (bf16 ? (one.rpl == nullptr || one.spl == nullptr || one.z != 12)
                            : (one.rf32 == nullptr || one.sf32 == nullptr)))
         return cudaErrorNotSupported;
     int dev = 0, sms = 148;
@@ -448,7 +443,7 @@ cudaError_t launch_corr_fft(const MatchJob& one, const ItemSet& is, int L, bool 
         const int smem = (int)FftShape<LV>::smem;                                                                 \
         e = cudaFuncSetAttribute(k_corr_fft<LV, BV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);         \
         if (e != cudaSuccess) return e;                                                                           \
-        const int grid = n < sms ? n : sms;                                                                       \
+        const int slots = sms * FftShape<LV>::MINB, grid = n < slots ? n : slots;                                                                       \
         k_corr_fft<LV, BV><<<grid, FftShape<LV>::T, smem, st>>>(one, is.jobs, is.items, n, is.queue);             \
     }
     if (L == 64) {
