@@ -177,7 +177,8 @@ size_t integral_export_scratch_bytes(int H, int W);
 cudaError_t launch_integral_export(const Cube& c, void* scratch, double* out, cudaStream_t st);
 
 struct PointStat {
-    double RT, RTT;       // template sums (Eq. 12) from the sensed integral images
+    long long rt;         // R_T (Eq. 12) in 2^-28 units, exact
+    float vT;             // R_TT - R_T^2 / mnz
     float tmean;          // R_T / mnz (for the zero-mean template)
     int status;           // SFOC_PT_*
 };
@@ -215,6 +216,8 @@ struct MatchJob {  // aligned as its tensor maps (128 bytes)
     PointStat* stats;       // n
     float* maps;            // n x (2R+1)^2 correlation maps (scratch)
     float* out_maps;        // optional n x (2R+1)^2 NCC maps
+    float flat, sc;         // 1e-6 mnz, the variance of a flat window; 2^-56 / mnz, a product of two window
+                            // sums in 2^-28 units divided by mnz
     fastncc_result* out;    // n
 };
 

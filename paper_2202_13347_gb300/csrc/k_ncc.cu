@@ -11,15 +11,15 @@
 // k_ncc_argmax      per point (one CTA): for every offset, R_S and R_SS from
 //                   the reference integral images (4 lookups each, exact
 //                   64-bit fixed point); the two steps that cancel are taken
-//                   in exact 128-bit integers: mnz R_SS - R_S^2 (the
+//                   in exact 96-bit integers: mnz R_SS - R_S^2 (the
 //                   variance times mnz) and, for the uncentred correlation
 //                   forms, R_S R_T (the mean correction of the numerator);
 //                   each is rounded to FP32 once, then NCC = num / sqrt(vS vT)
 //                   in FP32; a warp-shuffle argmax with the (NCC desc, dy
 //                   asc, dx asc) order and a 3-point parabola per axis.  No
 //                   FP64 per offset: GB300 runs it at a small fraction of its
-//                   FP32 rate, and 64 x 64-bit integer products cost a few
-//                   integer multiply-adds.
+//                   FP32 rate, and the integer products cost a few 32-bit
+//                   multiply-adds.
 #include <math.h>
 #include <string.h>
 
@@ -31,17 +31,29 @@ namespace {
 
 typedef unsigned long long u64;
 
-// a non-negative 128-bit integer to FP32 (two roundings: relative error
-// below 2^-23)
-__device__ __forceinline__ float u128_to_float(unsigned __int128 v) {
-    const u64 hi = (u64)(v >> 64), lo = (u64)v;
-    return fmaf(__ull2float_rn(hi), 18446744073709551616.f, __ull2float_rn(lo));
+// A non-negative integer below 2^96 in 32-bit words.  Window sums in 2^-28 units
+// stay below 2^45 in size and mnz below 2^19, so the exact products of the NCC fit
+// it and take a handful of 32 x 32-bit multiply-adds (as 128-bit integers they
+// took twice the instructions).
+struct U96 {
+    unsigned w0, w1, w2;
+};
+
+// a b, both below 2^45
+__device__ __forceinline__ U96 mul96(u64 a, u64 b) {
+    const unsigned al = (unsigned)a, ah = (unsigned)(a >> 32), bl = (unsigned)b, bh = (unsigned)(b >> 32);
+    const u64 t0 = (u64)al * bl;
+    const u64 t1 = (u64)al * bh + (u64)ah * bl + (t0 >> 32);  // below 2^47
+    return {(unsigned)t0, (unsigned)t1, ah * bh + (unsigned)(t1 >> 32)};
 }
 
-// window sum (Eq. 16) in 2^-28 units; exact (the planes wrap modulo 2^64)
-__device__ __forceinline__ long long rect(const u64* P, size_t ip, int y0, int x0, int y1, int x1) {
-    return (long long)(P[(size_t)y1 * ip + x1] - P[(size_t)y0 * ip + x1] - P[(size_t)y1 * ip + x0] +
-                       P[(size_t)y0 * ip + x0]);
+// to FP32 from its first two words that count (two roundings, relative error below
+// 2^-23; what a third word adds is below 2^-32 of it).  32-bit conversions: the
+// 64-bit ones run on the FP64 pipe, 64 clocks a warp each.
+__device__ __forceinline__ float u96_to_float(const U96& v) {
+    const unsigned hi = v.w2 ? v.w2 : v.w1, lo = v.w2 ? v.w1 : v.w0;
+    const float f = fmaf(__uint2float_rn(hi), 4294967296.f, __uint2float_rn(lo));
+    return v.w2 ? f * 4294967296.f : f;
 }
 
 // Threads per point and loads in flight per thread: the two planes come from L2
@@ -106,8 +118,8 @@ __global__ void __launch_bounds__(kStatThreads)
     __syncthreads();
     if (threadIdx.x != 0) return;
     PointStat s;
-    s.RT = s.RTT = 0.0;
-    s.tmean = 0.f;
+    s.rt = 0;
+    s.tmean = s.vT = 0.f;
     if (!ok) {
         s.status = SFOC_PT_OUT_OF_BOUNDS;
     } else {
@@ -119,13 +131,13 @@ __global__ void __launch_bounds__(kStatThreads)
         const long long rt = (long long)t1, rtt = (long long)t2;
         const double N = (double)m * m * z;
         if (rt >= kIntNonFiniteMin || rtt >= kIntNonFiniteMin) {
-            s.RT = s.RTT = NAN;
             s.status = SFOC_PT_NAN;
         } else {
-            s.RT = int_units_to_double(rt);
-            s.RTT = int_units_to_double(rtt);
-            s.tmean = (float)(s.RT / N);
-            const double vT = s.RTT - s.RT * s.RT / N;
+            const double RT = int_units_to_double(rt), RTT = int_units_to_double(rtt);
+            const double vT = RTT - RT * RT / N;
+            s.rt = rt;
+            s.vT = (float)vT;
+            s.tmean = (float)(RT / N);
             s.status = vT <= 1e-6 * N ? SFOC_PT_FLAT_TEMPLATE : SFOC_PT_OK;
         }
     }
@@ -137,22 +149,29 @@ __device__ __forceinline__ bool better(float v, int i, float bv, int bi) {
     return v > bv || (v == bv && i < bi);
 }
 
+// What bounds the kernel: the lookups (64 B an offset from L2, little locality in
+// L1) and ~80 instructions an offset.  Nothing of it may touch the FP64 pipe, which
+// a warp's instruction holds for 64 clocks: what a point's warps all need in FP64
+// is in its PointStat, or in the job.  Five CTAs per SM: more spill, fewer hide less
+// of the lookups' latency (R = 40: 102 us, with four 126, with six 115; several
+// offsets' lookups in flight per thread were slower too, 147 and 155).  With FP64
+// in every warp, 128-bit products and the map in shared memory: 41 -> 31 us for
+// 1000 points of R = 20, 146 -> 102 for 2000 of R = 40, 80 -> 65 for 400 of R = 60,
+// 41 -> 25 for 2000 of R = 10.
 constexpr int kNccThreads = 256;
 
-__global__ void __launch_bounds__(kNccThreads) k_ncc_argmax(const __grid_constant__ MatchJob one,
-                                                            const MatchJob* __restrict__ jobs,
-                                                            const int2* __restrict__ items) {
-    extern __shared__ float s_map[];  // P1 * P1
+__global__ void __launch_bounds__(kNccThreads, 5)
+    k_ncc_argmax(const __grid_constant__ MatchJob one, const MatchJob* __restrict__ jobs,
+                 const int2* __restrict__ items) {
     __shared__ float s_bv[kNccThreads / 32];
     __shared__ int s_bi[kNccThreads / 32];
     __shared__ int s_nan;
     int k;
     const MatchJob& J = item_job(one, jobs, items, blockIdx.x, &k);
     const u64* __restrict__ Pr = J.rint;
-    const int Hr = J.Hr, m = J.m, R = J.R, z = J.z, centered = J.centered;
+    const int Hr = J.Hr, m = J.m, R = J.R, centered = J.centered;
     const size_t ipr = J.ripitch;
     const int32_t* __restrict__ pts = J.pts;
-    const float* __restrict__ num = J.maps;
     float* __restrict__ out_maps = J.out_maps;
     fastncc_result* __restrict__ out = J.out;
     const int P1 = 2 * R + 1, P = P1 * P1;
@@ -170,26 +189,31 @@ __global__ void __launch_bounds__(kNccThreads) k_ncc_argmax(const __grid_constan
         return;
     }
     __syncthreads();
-    const long long Ni = (long long)m * m * z;
-    const double N = (double)Ni;
-    const float flat = (float)(1e-6 * N);
-    const float vTf = (float)(st.RTT - st.RT * st.RT / N);
-    // 2^-56 / mnz: a product of two window sums in 2^-28 units, divided by mnz
-    const float sc = (float)(1.0 / (72057594037927936.0 * N));
-    const long long rt = (long long)(st.RT * 268435456.0);  // R_T in 2^-28 units (exact)
+    const unsigned Ni = (unsigned)(m * m * J.z);
+    const float flat = J.flat, sc = J.sc, vTf = st.vT;
+    const long long rt = st.rt;
+    const u64 rta = (u64)(rt < 0 ? -rt : rt);
     const int h = template_half(m);
     const int ty0 = pts[2 * k + 1] - h, tx0 = pts[2 * k] - h;
     const u64* P1p = Pr;
-    const u64* P2p = Pr + (size_t)(Hr + 1) * ipr;
-    const float* nk = num + (size_t)k * P;
+    const size_t plane = (size_t)(Hr + 1) * ipr;
+    // each numerator is replaced by its NCC: the peak's neighbours are read back
+    // from there (a copy in shared memory kept CTAs out at large R)
+    float* const nk = J.maps + (size_t)k * P;
     float bv = -INFINITY;
     int bi = 0x7fffffff;
     int has_nan = 0;
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const int iy = i / P1, ix = i - iy * P1;
-        const int wy = ty0 + iy - R, wx = tx0 + ix - R;
-        const long long rs = rect(P1p, ipr, wy, wx, wy + m, wx + m);
-        const long long rss = rect(P2p, ipr, wy, wx, wy + m, wx + m);
+    // (i + 1/2) / P1 is at least 1 / (2 P1) from an integer, P1 <= 127: far more
+    // than its two roundings
+    const float inv = 1.f / (float)P1;
+    const size_t dn = (size_t)m * ipr;
+    for (int i = threadIdx.x; i < P; i += kNccThreads) {
+        const int iy = (int)(((float)i + 0.5f) * inv), ix = i - iy * P1;
+        const u64* a = P1p + (size_t)(ty0 + iy - R) * ipr + (tx0 + ix - R);
+        const u64* b = a + plane;
+        // window sums (Eq. 16) in 2^-28 units; exact (the planes wrap modulo 2^64)
+        const long long rs = (long long)(a[dn + m] - a[m] - a[dn] + a[0]);
+        const long long rss = (long long)(b[dn + m] - b[m] - b[dn] + b[0]);
         const float n32 = nk[i];
         float v;
         if (rs >= kIntNonFiniteMin || rss >= kIntNonFiniteMin || n32 != n32) {
@@ -197,17 +221,20 @@ __global__ void __launch_bounds__(kNccThreads) k_ncc_argmax(const __grid_constan
         } else {
             // mnz R_SS - R_S^2, exact (units 2^-56); negative only through the
             // per-pixel rounding of a flat window
-            const __int128 d = ((__int128)(Ni * rss) << 28) - (__int128)rs * rs;
-            const float vS = d > 0 ? u128_to_float((unsigned __int128)d) * sc : 0.f;
+            const u64 rsa = (u64)(rs < 0 ? -rs : rs);
+            const u64 x = (u64)Ni * (unsigned)rss + ((u64)(Ni * (unsigned)((u64)rss >> 32)) << 32);
+            const U96 q = mul96(rsa, rsa);
+            const u64 xl = x << 28, ql = (u64)q.w1 << 32 | q.w0, dl = xl - ql;
+            const int d2 = (int)((unsigned)(x >> 36) - q.w2 - (xl < ql ? 1u : 0u));
+            const float vS = d2 >= 0 ? u96_to_float({(unsigned)dl, (unsigned)(dl >> 32), (unsigned)d2}) * sc : 0.f;
             float nm = n32;
             if (!centered) {
-                const __int128 p = (__int128)rs * rt;  // R_S R_T, exact
-                const float pf = p >= 0 ? u128_to_float((unsigned __int128)p) : -u128_to_float((unsigned __int128)(-p));
-                nm = fmaf(-pf, sc, n32);
+                const float pf = u96_to_float(mul96(rsa, rta));  // |R_S R_T|, exact
+                nm = fmaf((rs < 0) != (rt < 0) ? pf : -pf, sc, n32);
             }
             v = vS <= flat ? 0.f : nm / sqrtf(vS * vTf);
         }
-        s_map[i] = v;
+        nk[i] = v;
         if (out_maps) out_maps[(size_t)k * P + i] = v;
         if (v != v) { has_nan = 1; continue; }
         if (better(v, i, bv, bi)) { bv = v; bi = i; }
@@ -248,9 +275,9 @@ __global__ void __launch_bounds__(kNccThreads) k_ncc_argmax(const __grid_constan
                 double d = (cm - cp) / (2.0 * den);
                 return d > 0.5 ? 0.5 : (d < -0.5 ? -0.5 : d);
             };
-            if (ix > 0 && ix < P1 - 1) ddx = parab(s_map[bi - 1], bv, s_map[bi + 1]);
+            if (ix > 0 && ix < P1 - 1) ddx = parab(nk[bi - 1], bv, nk[bi + 1]);
             else edge = true;
-            if (iy > 0 && iy < P1 - 1) ddy = parab(s_map[bi - P1], bv, s_map[bi + P1]);
+            if (iy > 0 && iy < P1 - 1) ddy = parab(nk[bi - P1], bv, nk[bi + P1]);
             else edge = true;
             if (ddx != ddx) ddx = 0.0;
             if (ddy != ddy) ddy = 0.0;
@@ -274,12 +301,7 @@ cudaError_t launch_template_stats(const MatchJob& one, const ItemSet& is, cudaSt
 cudaError_t launch_ncc_argmax(const MatchJob& one, const ItemSet& is, cudaStream_t st) {
     const int n = is.items ? is.n : one.n;
     if (n <= 0) return cudaSuccess;
-    const int R = is.items ? is.max_R : one.R;
-    const int P1 = 2 * R + 1;
-    size_t smem = sizeof(float) * (size_t)P1 * P1;
-    cudaError_t e = cudaFuncSetAttribute(k_ncc_argmax, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_ncc_argmax<<<n, kNccThreads, smem, st>>>(one, is.jobs, is.items);
+    k_ncc_argmax<<<n, kNccThreads, 0, st>>>(one, is.jobs, is.items);
     return cudaGetLastError();
 }
 
@@ -315,6 +337,9 @@ MatchJob make_job(const Cube& ref, const Cube& sen, const int32_t* pts, int n, i
     j.stats = stats;
     j.maps = maps;
     j.out_maps = out_maps;
+    const double N = (double)m * m * ref.z;
+    j.flat = (float)(1e-6 * N);
+    j.sc = (float)(1.0 / (72057594037927936.0 * N));
     j.out = out;
     return j;
 }
