@@ -104,13 +104,20 @@ struct ImgJob {
     float* s2;
 };
 
+// One or two images passed by value: CTAs from `split` on are the second's.
+struct ImgPair {
+    ImgJob j[2];
+    int split;
+};
+
 // The image of this CTA and its tile index within it.
-__device__ __forceinline__ const ImgJob& img_job(const ImgJob& one, const ImgJob* jobs, const int* begin, int n_jobs,
+__device__ __forceinline__ const ImgJob& img_job(const ImgPair& one, const ImgJob* jobs, const int* begin, int n_jobs,
                                                  int* tile) {
     const int bid = blockIdx.x;
     if (!jobs) {
-        *tile = bid;
-        return one;
+        const bool second = bid >= one.split;
+        *tile = second ? bid - one.split : bid;
+        return one.j[second ? 1 : 0];
     }
     int lo = 0, hi = n_jobs - 1;  // the last image whose first CTA is at or before this one
     while (lo < hi) {
@@ -136,6 +143,9 @@ cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, cons
 // image (sfoc_batch_tiles gives the counts).
 bool sfoc_batch_supported(const SteerTaps& st, const SmoothTaps& sm);
 void sfoc_batch_tiles(int H, int W, int* steer_ctas, int* smooth_ctas);
+// Two float images in one launch per kernel (both within the batched forms'
+// parameters): small images leave most of the chip idle one after the other.
+cudaError_t launch_sfoc_two(const ImgJob* two, const SteerTaps& st, const SmoothTaps& sm, cudaStream_t s);
 cudaError_t launch_sfoc_batch(const ImgJob* jobs, int n_jobs, const int* steer_begin, int steer_ctas,
                               const int* smooth_begin, int smooth_ctas, const SteerTaps& st, const SmoothTaps& sm,
                               cudaStream_t s);

@@ -154,12 +154,12 @@ __host__ __device__ inline int steer_rows(int H) {
     return ((H + seg - 1) / seg + kSrU - 1) / kSrU * kSrU;
 }
 
-// One image (`one`, warps = strips x segments in row-major order) or a batch
+// One or two images (`one`, warps = strips x segments in row-major order) or a batch
 // (device table `jobs`, CTAs of image j from begin[j]).  seg_rows: output rows
 // per warp (0: steer_rows of the image).
 template <typename T>
 __global__ void __launch_bounds__(kSrThreads, 3)
-    k_sfoc_steer_strip(const __grid_constant__ ImgJob one, const ImgJob* __restrict__ jobs,
+    k_sfoc_steer_strip(const __grid_constant__ ImgPair one, const ImgJob* __restrict__ jobs,
                        const int* __restrict__ begin, int n_jobs, const __grid_constant__ SteerTaps tp, int seg_rows) {
     constexpr int U = kSrU, N1 = U + 6, N2 = U + 10;
     __shared__ float s_rows[kSrThreads / 32][2][U][kSrPitch];
@@ -651,12 +651,12 @@ __device__ __forceinline__ void strip_finish(const StripOut& o, float eps, const
     }
 }
 
-// One image (`one`, CTA = strip of the image's strips x segments) or a batch
+// One or two images (`one`, CTA = strip of the image's strips x segments) or a batch
 // (device table `jobs`, CTAs of image j from begin[j]).  seg_rows: output rows
 // per CTA, a multiple of kStU (0: strip_rows of the image).
 template <int KD>
 __global__ void __launch_bounds__(kStThreads, 2)
-    k_sfoc_smooth_strip(const __grid_constant__ ImgJob one, const ImgJob* __restrict__ jobs,
+    k_sfoc_smooth_strip(const __grid_constant__ ImgPair one, const ImgJob* __restrict__ jobs,
                         const int* __restrict__ begin, int n_jobs, const __grid_constant__ SmoothTaps tp, int g,
                         int seg_rows) {
     using G = StripGeom<KD>;
@@ -884,14 +884,25 @@ int steer_ctas(int H, int W, int rows) {
     return (tasks + kSrThreads / 32 - 1) / (kSrThreads / 32);
 }
 
-// Output rows per warp for one image: the rows with the least waves (three CTAs
-// of four warps per SM) x rows streamed (10 more than the output rows).
-int steer_rows_single(int H, int W) {
+ImgPair img_none() {
+    ImgPair p;
+    memset(&p, 0, sizeof(p));
+    p.split = 0x7fffffff;
+    return p;
+}
+
+// Output rows per warp for one or two images: the rows with the least waves
+// (three CTAs of four warps per SM) x rows streamed (10 more than the output
+// rows).
+int steer_rows_for(const ImgJob* j, int n) {
     const int slots = 3 * 152;
+    int H = 0;
+    for (int i = 0; i < n; ++i) H = j[i].H > H ? j[i].H : H;
     long best = -1;
     int rows = kSrU;
     for (int r = 4 * kSrU; r < H + kSrU; r += kSrU) {
-        const long ctas = steer_ctas(H, W, r);
+        long ctas = 0;
+        for (int i = 0; i < n; ++i) ctas += steer_ctas(j[i].H, j[i].W, r);
         const long cost = (ctas + slots - 1) / slots * (r + 14);
         if (best < 0 || cost <= best) {
             best = cost;
@@ -908,15 +919,14 @@ cudaError_t launch_steer_any(const T* img, int H, int W, size_t pitch, float* F,
     dim3 grid((W + kTW - 1) / kTW, (H + kTH - 1) / kTH);
     // the paper's scales (0.6, 0.8, 1.0 and 1.5 at 3 sigma: radii 2, 3, 3, 5), six orientations
     if (steer_is_paper(tp)) {
-        ImgJob one;
-        memset(&one, 0, sizeof(one));
-        one.img = img;
-        one.pitch = pitch;
-        one.H = H;
-        one.W = W;
-        one.F = F;
-        one.fpitch = fpitch;
-        const int rows = steer_rows_single(H, W);
+        ImgPair one = img_none();
+        one.j[0].img = img;
+        one.j[0].pitch = pitch;
+        one.j[0].H = H;
+        one.j[0].W = W;
+        one.j[0].F = F;
+        one.j[0].fpitch = fpitch;
+        const int rows = steer_rows_for(&one.j[0], 1);
         k_sfoc_steer_strip<T><<<steer_ctas(H, W, rows), kSrThreads, 0, st>>>(one, nullptr, nullptr, 0, tp, rows);
         return cudaGetLastError();
     }
@@ -948,7 +958,7 @@ namespace {
 
 // the two group launches of the paper's smoothing (sigma_d 1.0 / 1.5, rates
 // 1, 2, 3) over `ctas` CTAs of seg_rows output rows (0: a batch's own)
-cudaError_t launch_smooth_paper(const ImgJob& one, const ImgJob* jobs, const int* begin, int n_jobs, int ctas,
+cudaError_t launch_smooth_paper(const ImgPair& one, const ImgJob* jobs, const int* begin, int n_jobs, int ctas,
                                 int seg_rows, const SmoothTaps& tp, cudaStream_t st) {
     auto run = [&](auto kern, int g, size_t smem) -> cudaError_t {
         const cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -975,16 +985,21 @@ cudaError_t launch_smooth_paper(const ImgJob& one, const ImgJob* jobs, const int
     return e;
 }
 
-// Output rows per CTA for one image: every CTA streams up to four blocks more
-// than it completes, and an SM's time is the blocks of its CTAs (one alone runs
-// a block in about half the time of two together): the rows with the fewest
-// blocks on the fullest SM.
-int strip_rows_single(int H, int W) {
-    const long strips = (W + kStW - 1) / kStW, sms = 152;
+int smooth_ctas_for(const ImgJob& j, int rows) { return ((j.W + kStW - 1) / kStW) * ((j.H + rows - 1) / rows); }
+
+// Output rows per CTA for one or two images: every CTA streams up to four blocks
+// more than it completes, and an SM's time is the blocks of its CTAs (one alone
+// runs a block in about half the time of two together): the rows with the
+// fewest blocks on the fullest SM.
+int strip_rows_for(const ImgJob* j, int n) {
+    const long sms = 152;
+    int H = 0;
+    for (int i = 0; i < n; ++i) H = j[i].H > H ? j[i].H : H;
     long best = -1;
     int rows = kStU;
     for (int r = kStU; r < H + kStU; r += kStU) {
-        const long ctas = strips * ((H + r - 1) / r);
+        long ctas = 0;
+        for (int i = 0; i < n; ++i) ctas += smooth_ctas_for(j[i], r);
         const long cost = (ctas + sms - 1) / sms * (r / kStU + 4);
         if (best < 0 || cost < best) {
             best = cost;
@@ -1005,13 +1020,27 @@ void sfoc_batch_tiles(int H, int W, int* n_steer, int* smooth_ctas) {
     *smooth_ctas = ((W + kStW - 1) / kStW) * ((H + rows - 1) / rows);
 }
 
+cudaError_t launch_sfoc_two(const ImgJob* two, const SteerTaps& st, const SmoothTaps& sm, cudaStream_t s) {
+    if (!sfoc_batch_supported(st, sm)) return cudaErrorNotSupported;
+    ImgPair p;
+    p.j[0] = two[0];
+    p.j[1] = two[1];
+    const int sr = steer_rows_for(two, 2), mr = strip_rows_for(two, 2);
+    p.split = steer_ctas(two[0].H, two[0].W, sr);
+    k_sfoc_steer_strip<float><<<p.split + steer_ctas(two[1].H, two[1].W, sr), kSrThreads, 0, s>>>(p, nullptr, nullptr,
+                                                                                                 0, st, sr);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    p.split = smooth_ctas_for(two[0], mr);
+    return launch_smooth_paper(p, nullptr, nullptr, 0, p.split + smooth_ctas_for(two[1], mr), mr, sm, s);
+}
+
 cudaError_t launch_sfoc_batch(const ImgJob* jobs, int n_jobs, const int* steer_begin, int steer_ctas,
                               const int* smooth_begin, int smooth_ctas, const SteerTaps& st, const SmoothTaps& sm,
                               cudaStream_t s) {
     if (n_jobs <= 0) return cudaSuccess;
     if (!sfoc_batch_supported(st, sm)) return cudaErrorNotSupported;
-    ImgJob none;
-    memset(&none, 0, sizeof(none));
+    const ImgPair none = img_none();
     k_sfoc_steer_strip<float><<<steer_ctas, kSrThreads, 0, s>>>(none, jobs, steer_begin, n_jobs, st, 0);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1023,8 +1052,8 @@ cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, cons
     dim3 grid((W + kSTW - 1) / kSTW, (H + kSTH - 1) / kSTH);
     cudaError_t e;
     if (smooth_is_paper(tp)) {  // sigma_d 1.0 / 1.5 with rates 1, 2, 3 (Sec. 2.1): one launch per group
-        ImgJob one;
-        memset(&one, 0, sizeof(one));
+        ImgPair pair = img_none();
+        ImgJob& one = pair.j[0];
         one.H = H;
         one.W = W;
         one.F = const_cast<float*>(F);
@@ -1036,9 +1065,8 @@ cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, cons
         one.pl = c.pl;
         one.s1 = c.s1;
         one.s2 = c.s2;
-        const int rows = strip_rows_single(H, W);
-        const int ctas = ((W + kStW - 1) / kStW) * ((H + rows - 1) / rows);
-        return launch_smooth_paper(one, nullptr, nullptr, 0, ctas, rows, tp, st);
+        const int rows = strip_rows_for(&one, 1);
+        return launch_smooth_paper(pair, nullptr, nullptr, 0, smooth_ctas_for(one, rows), rows, tp, st);
     }
     const int maxhal = tp.halo[0] > tp.halo[1] ? tp.halo[0] : tp.halo[1];
     const int HR = kSTH + 2 * maxhal, FW = smooth_row_stride(maxhal);

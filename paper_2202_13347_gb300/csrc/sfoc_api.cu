@@ -465,6 +465,89 @@ sfoc_status build_cube(sfoc_ctx* ctx, const T* d_image, int H, int W, size_t pit
     return SFOC_OK;
 }
 
+// The most pixels of a pair whose two cubes are built in one launch per kernel:
+// a pair of 1024 x 1024 images.  A small image leaves most of the chip idle, and
+// its three launches are a chain of latencies; the whole call, one image after
+// the other and both together: 300 x 300, 50 points 155 and 123 us, 512 x 512, 100
+// points 169 and 148, 700 x 700 216 and 202, 1024 x 1024, 300 points 445 and 438.
+// Larger images fill the chip by themselves, and two workspaces of them are large.
+constexpr size_t kPairPixels = (size_t)1 << 21;
+
+// Both cubes of a small pair together (*done), into the context's pair cubes.
+// Whatever is not plain (a null pointer, a shape or parameter that is refused,
+// parameters without the streaming kernels, a workspace that may not grow
+// inside a capture) is left to the two single builds, which report it.
+sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, const float* d_sen, int Hs, int Ws,
+                             const sfoc_params* pin, bool* done) {
+    *done = false;
+    if (!d_ref || !d_sen || Hr < 1 || Wr < 1 || Hs < 1 || Ws < 1) return SFOC_OK;
+    if ((size_t)Hr * Wr + (size_t)Hs * Ws > kPairPixels) return SFOC_OK;
+    sfoc_params p;
+    if (pin) p = *pin;
+    else sfoc_params_default(&p);
+    if (check_params(ctx, p) != SFOC_OK) return SFOC_OK;
+    const SteerTaps st = make_steer(p);
+    const SmoothTaps sm = make_smooth(p);
+    if (!sfoc_batch_supported(st, sm)) return SFOC_OK;
+    const int H[2] = {Hr, Hs}, W[2] = {Wr, Ws}, z = 12;
+    const float* img[2] = {d_ref, d_sen};
+    sfoc_cube** cube[2] = {&ctx->pair_ref, &ctx->pair_sen};
+    size_t at[3] = {0, 0, 0};
+    for (int k = 0; k < 2; ++k) at[k + 1] = at[k] + align256(sizeof(float) * roundup((size_t)W[k], 32) * (size_t)H[k] * z);
+    DeviceGuard g(ctx->device);
+    bool fits[2];
+    for (int k = 0; k < 2; ++k) {
+        const sfoc_cube* c = *cube[k];
+        fits[k] = c && c->c.H == H[k] && c->c.W == W[k] && c->c.z == z && c->c.dtype == p.cube_dtype &&
+                  c->c.device == ctx->device;
+    }
+    // the workspace grows only where a single build would have it grow as well
+    const bool grows = at[2] > ctx->ws_bytes;
+    if (grows && std::max(at[1], at[2] - at[1]) <= ctx->ws_bytes) return SFOC_OK;
+    if ((grows || !fits[0] || !fits[1]) && capturing(ctx->stream)) return SFOC_OK;
+    sfoc_status s = ensure_ws(ctx, at[2]);
+    if (s != SFOC_OK) return s;
+    for (int k = 0; k < 2; ++k) {
+        if (fits[k]) continue;
+        // (the cube it replaces stays, as with sfoc_build: a captured graph may read it)
+        sfoc_cube* c = new (std::nothrow) sfoc_cube();
+        if (!c) return fail(ctx, SFOC_ERR_OOM, "host allocation");
+        s = alloc_cube(ctx, c->c, H[k], W[k], z, p.cube_dtype);
+        if (s != SFOC_OK) {
+            delete c;
+            return s;
+        }
+        *cube[k] = c;
+    }
+    ImgJob two[2];
+    memset(two, 0, sizeof(two));
+    for (int k = 0; k < 2; ++k) {
+        Cube& c = (*cube[k])->c;
+        two[k].img = img[k];
+        two[k].pitch = (size_t)W[k];
+        two[k].H = H[k];
+        two[k].W = W[k];
+        two[k].F = reinterpret_cast<float*>(static_cast<char*>(ctx->ws) + at[k]);
+        two[k].fpitch = roundup((size_t)W[k], 32);
+        two[k].c32 = c.f32;
+        two[k].cpitch = c.pitch;
+        two[k].rm = c.rm;
+        two[k].cm = c.cm;
+        two[k].pl = c.pl;
+        two[k].s1 = c.s1;
+        two[k].s2 = c.s2;
+        c.integ_valid = false;
+    }
+    cudaError_t e;
+    {
+        StageScope sc(ctx, ST_SMOOTH, 3);
+        e = launch_sfoc_two(two, st, sm, ctx->stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "sfoc kernels");
+    *done = true;
+    return SFOC_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -901,10 +984,15 @@ sfoc_status fastncc_register_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int
                                   int Ws, const int32_t* d_points, int n, int template_size, int search_radius,
                                   const sfoc_params* p, const fastncc_opts* opts, fastncc_result* d_out) {
     if (!ctx) return SFOC_ERR_INVALID_ARG;
-    sfoc_status s = sfoc_build(ctx, d_ref, Hr, Wr, (size_t)Wr, nullptr, 0, 0, p, &ctx->pair_ref);
+    bool both = false;
+    sfoc_status s = ctx->timing ? SFOC_OK : build_small_pair(ctx, d_ref, Hr, Wr, d_sen, Hs, Ws, p, &both);
     if (s != SFOC_OK) return s;
-    s = sfoc_build(ctx, d_sen, Hs, Ws, (size_t)Ws, nullptr, 0, 0, p, &ctx->pair_sen);
-    if (s != SFOC_OK) return s;
+    if (!both) {  // (per-stage timing keeps the steering and smoothing launches apart)
+        s = sfoc_build(ctx, d_ref, Hr, Wr, (size_t)Wr, nullptr, 0, 0, p, &ctx->pair_ref);
+        if (s != SFOC_OK) return s;
+        s = sfoc_build(ctx, d_sen, Hs, Ws, (size_t)Ws, nullptr, 0, 0, p, &ctx->pair_sen);
+        if (s != SFOC_OK) return s;
+    }
     return fastncc_match(ctx, ctx->pair_ref, ctx->pair_sen, d_points, n, template_size, search_radius, opts, d_out);
 }
 
