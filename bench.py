@@ -47,7 +47,7 @@ sys.path.insert(0, ROOT)
 METRIC = "matched CPs/sec and SFOC Mpix/sec on 1 GB300, BF16-batched vs plain FP32"
 UNIT = "CP/s"
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12   # SMs x FP32 lanes x 2 flop x max SM clock
-FFT_SIZES = (64, 128)  # transform sides of the Fourier correlation (the smallest with m + 2R <= L)
+FFT_SIZES = (64, 128)  # transform sides of SFOC_CORR_FFT (the smallest with m + 2R <= L); AUTO adds 96, 160, 192, 224
 # DRAM bytes (read + write) per processed point of a correlation kernel on
 # the 2048x2048 workload (m = 81, R = 20), keyed by (form, correlation path),
 # from one ncu capture of the kernel as it stands (the band form: 87.12 MB
@@ -263,7 +263,8 @@ def run_form(b, torch, ctx, pair, form, steps, warmup, flush, corr_name="auto"):
                 t_timed=(t_start, t_end), path=path, option=option)
 
 
-# FP32 operations of one FAST-9 score as k_fast_blocks computes it: 16
+# FP32 operations of one FAST-9 score as k_fast_blocks computes it (for the
+# pixels that pass its quick test; the roofline counts every pixel's): 16
 # differences to the centre, 32 + 32 min/max for the windows of 2 and 4
 # circle pixels (both polarities), 6 per arc for the 16 arcs of 9, 3 to
 # finish
@@ -272,9 +273,9 @@ FP32_OPS_PEAK = 152 * 128 * 2.070e9 / 1e12   # Top/s: one FP32 add / min / max p
 
 
 def fast_roofline(ms, H, W, hbm_gbs, pk=None):
-    """Block FAST is bound by its score arithmetic, not by HBM (the image is
-    read once, 4 B/px): achieved = FAST_OPS_PER_PX per pixel of the image
-    over the launch time, against one FP32 op per lane per clock (half the
+    """Block FAST against the full score at every pixel (the kernel's quick
+    test spares most pixels it), the image read once, 4 B/px: achieved =
+    FAST_OPS_PER_PX per pixel of the image over the launch time, against one FP32 op per lane per clock (half the
     measured scalar FMA flop rate, which counts 2 flop per FMA)."""
     ach = FAST_OPS_PER_PX * H * W / (ms * 1e-3) / 1e12
     gbs = 4.0 * H * W / (ms * 1e-3) / 1e9
@@ -360,10 +361,10 @@ def run_ransac(b, torch, ctx, pair, r, n_hyp=4096, reps=10, seed=7):
                    truth="planted offset of each point")
     return dict(ms=statistics.median(t), hypotheses=n_hyp, points=int(src.shape[0]), valid=int(valid.sum()),
                 inliers=int(info[1]), best_hypothesis=int(info[0]), model="projective", threshold_px=1.5,
-                launches=3,
+                launches=4,
                 rectify={"ms": rect_ms, "mpix_s": pair.sen.size / (rect_ms * 1e-3) / 1e6,
                          "gb_s": 8.0 * pair.sen.size / (rect_ms * 1e-3) / 1e9,
-                         "work": "4 B read + 4 B written per output pixel (bilinear, FP64 mapping)"}), quality
+                         "work": "4 B read + 4 B written per output pixel (bilinear, one FP64 mapping per 32 x 8 tile)"}), quality
 
 
 def run_e2e(b, torch, ctx, pair, p, corr, steps):
@@ -496,8 +497,8 @@ def form_roofline(form, pair, per_launch_ms, processed, pk, workload, path, opti
         ach = fft_flops_mrl(pair.m, pair.R, L) * processed / secs / 1e12
         return {"bound": "alu", "achieved": ach, "peak": peak32, "unit": "TFLOP/s",
                 "frac": ach / peak32, "traffic": traffic,
-                "kernel": "k_corr_fft<%d> (FP32 Fourier correlation, Eq. 13, %s cubes)" % (
-                    L, "BF16" if form == "bf16" else "F32"),
+                "kernel": "%s<%d> (FP32 Fourier correlation, Eq. 13, %s cubes)" % (
+                    "k_corr_fft" if L in FFT_SIZES else "k_corr_fft2", L, "BF16" if form == "bf16" else "F32"),
                 "peak_src": fp32_src,
                 "work": "5 L log2 L flop per length-L transform (z (m+2R+L) forward, L/2+1+2R+1 inverse) "
                         "+ 12 flop per cross-spectrum bin, per processed point"}
