@@ -4,7 +4,8 @@
 // circular correlation equals the linear one at every offset in [0, 2R]),
 // their spectra multiplied (one conjugated) and summed over the channels,
 // and one inverse transform gives the numerator of Eq. 9 at every offset.
-// FP32 throughout, from the F32 cube; one CTA per point.
+// FP32 throughout, from the F32 cube or the planes of the BF16 cube; one CTA per
+// point, two CTAs per SM at side 64.
 //
 // Transforms.  A length-L transform (L = 8E) is done by a group of 8
 // threads: thread t holds x[t + 8j] (j < E), takes the E-point DFT over j in

@@ -481,8 +481,9 @@ __device__ __forceinline__ void smooth_group(int g, const float* __restrict__ F,
 // memory, read back by the vertical pass, 32 x 64 tiles that redo 1.5x of the
 // horizontal work) needed 30 shared words and ~90 instructions per pixel and
 // channel against 17 and ~50 here, with block barriers between its passes.
-// 2048 x 2048, F32 cube: group 0 (KD = 3) 133 -> 105 us, group 1
-// (KD = 5) 187 -> 143 us.
+// The finishing warps are as busy as the channel warps: without a branch per
+// column in them both groups of 1847 x 2891 took 330 us instead of 449.
+// Both groups of a 2048 x 2048 image: 322 -> 207 us (F32 cube), 343 -> 226 (BF16).
 constexpr int kStW = 64;     // strip width: 32 lanes x 2 columns
 constexpr int kStU = 8;      // rows per block
 constexpr int kStH = 4;      // rows between two shifts of the running sums
@@ -517,8 +518,9 @@ __host__ __device__ inline int strip_rows(int H) {
 // one by one, 16 of a row at a time.  (Copying such a strip's rows element by
 // element made its CTAs issue 1.4 times the instructions of the others, and a
 // launch of one wave waited for them: 512 x 512 19.4 and 25.9 us for groups 0 and
-// 1, with this 17.5 and 23.6; 2048 x 2048, two of 32 strips, 146 -> 141.5 for
-// group 1.)
+// 1, with this 17.5 and 23.6.  A right strip of few columns was worse still, until
+// it left out the columns past the halo: both groups of 1847 x 2891, 11 columns in
+// the last strip, 562 -> 449 us.)
 template <int KD>
 __device__ __forceinline__ void strip_rows_async(const float* __restrict__ Fk, size_t fpitch, int H, int W, int x0,
                                                  int i0, float* dst, int lane) {
@@ -546,21 +548,27 @@ __device__ __forceinline__ void strip_rows_async(const float* __restrict__ Fk, s
             }
     };
     if (xs < 0) clamped(0, -xs);
-    // (W > x0, so the first piece that is not whole is right of those)
-    for (int c0 = (W & ~3) - xs; c0 < G::RW; c0 += 16) clamped(c0, G::RW);
+    // (W > x0, so the first piece that is not whole is right of those.)  Columns past
+    // W - 1 + HAL reach no column of the image: they stay as they are
+    const int cend = W + G::HAL - xs < G::RW ? W + G::HAL - xs : G::RW;
+    for (int c0 = (W & ~3) - xs; c0 < cend; c0 += 16) clamped(c0, cend);
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 // The column-order bf16 chunks of a completed block: 8 lanes take the 8 rows of
-// one column, so that a column's 128 contiguous bytes leave together.
+// one column, so that a column's 128 contiguous bytes leave together; a thread
+// keeps its row and steps over every eighth column.  tid: 0 .. 32 kStFin - 1.
 __device__ __forceinline__ void strip_write_cm(const ImgJob& J, int g, const uint4* s_chunk, int cp, int x0, int yb,
-                                               int y1) {
-    uint4* const cm = reinterpret_cast<uint4*>(J.cm) + (size_t)g * J.H * J.W;
-    for (int p = threadIdx.x - kStChan * 32; p < kStU * kStW; p += kStFin * 32) {
-        const int c = p >> 3, u = p & 7;
-        const int gx = x0 + c, gy = yb + u;
-        if (gx < J.W && gy < y1) cm[(size_t)gx * J.H + gy] = s_chunk[u * cp + c];
-    }
+                                               int y1, int tid) {
+    constexpr int kStep = kStFin * 32 / kStU;
+    const int c0 = tid / kStU, u = tid % kStU;
+    if (yb + u >= y1) return;
+    uint4* q = reinterpret_cast<uint4*>(J.cm) + ((size_t)g * J.W + x0 + c0) * J.H + yb + u;
+    const size_t step = (size_t)kStep * J.H;
+    const uint4* src = s_chunk + u * cp + c0;
+#pragma unroll
+    for (int c = 0; c < kStW; c += kStep, q += step)
+        if (x0 + c0 + c < J.W) *q = src[c];
 }
 
 // Where a finishing warp's lane writes: its two pixels of row 0, and what holds
@@ -574,7 +582,10 @@ struct StripOut {
     size_t pitch, plane;
     int W;
     bool two;     // the second pixel is inside the image
-    bool vec;     // pairs of floats are 8-byte aligned in every row
+    bool vec;     // planes take both columns in one store: the pitch is even, so that the second one is inside the
+                  // row's padding at worst, and every row starts on 8 bytes.  (A lane of an odd width that stored
+                  // one column made its strip's warps run both forms: 1 / 6 of the time.)  A dense cube of odd
+                  // width (sfoc_build_static) is not
 };
 
 // One completed row of a strip: a lane normalises its two pixels' six channels
@@ -582,6 +593,7 @@ struct StripOut {
 // per-pixel sums, continued from `sums` (g of both pixels, then g^2).
 // `done`: the row's [channel][8][64] values at the lane's columns; `chunk`: the
 // lane's place in the chunk buffer.
+template <bool VEC>
 __device__ __forceinline__ void strip_finish(const StripOut& o, float eps, const float* done, uint4* chunk, int gy,
                                              const float4& sums) {
     float2 d[6];
@@ -620,7 +632,7 @@ __device__ __forceinline__ void strip_finish(const StripOut& o, float eps, const
     }
     const size_t at = (size_t)gy * o.pitch;
     auto put2 = [&](float* q, float x, float y) {
-        if (o.vec && o.two) {
+        if (VEC) {
             *reinterpret_cast<float2*>(q) = make_float2(x, y);
         } else {
             q[0] = x;
@@ -635,9 +647,7 @@ __device__ __forceinline__ void strip_finish(const StripOut& o, float eps, const
         for (int k = 0; k < 6; ++k, q += o.plane) put2(q, v[0][k], v[1][k]);
     }
     if (bf) {
-        // the planes: both columns in one store (gx is even and the pitch a multiple
-        // of 32, so the second one is inside the row's padding at worst)
-        __nv_bfloat16* q = o.pl + at;
+        __nv_bfloat16* q = o.pl + at;  // (BF16 cubes are padded: both columns in one store)
 #pragma unroll
         for (int k = 0; k < 6; ++k, q += o.plane)
             *reinterpret_cast<unsigned*>(q) = __byte_perm(pk[0][k >> 1], pk[1][k >> 1], (k & 1) ? 0x7632 : 0x5410);
@@ -706,11 +716,17 @@ __global__ void __launch_bounds__(kStThreads, 2)
                 sums[v] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (g > 0 && gy < y1 && gx < W) {
                     const size_t at = (size_t)gy * o.pitch;
-                    sums[v].x = o.s1[at];
-                    sums[v].z = o.s2[at];
-                    if (o.two) {
-                        sums[v].y = o.s1[at + 1];
-                        sums[v].w = o.s2[at + 1];
+                    if (o.vec) {
+                        const float2 a = *reinterpret_cast<const float2*>(o.s1 + at);
+                        const float2 b = *reinterpret_cast<const float2*>(o.s2 + at);
+                        sums[v] = make_float4(a.x, a.y, b.x, b.y);
+                    } else {
+                        sums[v].x = o.s1[at];
+                        sums[v].z = o.s2[at];
+                        if (o.two) {
+                            sums[v].y = o.s1[at + 1];
+                            sums[v].w = o.s2[at + 1];
+                        }
                     }
                 }
             }
@@ -718,15 +734,21 @@ __global__ void __launch_bounds__(kStThreads, 2)
             asm volatile("bar.sync %0, %1;" ::"r"(kFull + b), "n"(kStThreads) : "memory");
             const float* done = s_done + (size_t)b * kStChan * U * kStW + (warp - kStChan) * kStW + 2 * lane;
             uint4* chunk = s_chunk + (size_t)b * U * G::CP + (warp - kStChan) * G::CP + 2 * lane;
+auto finish = [&](auto vec) {
 #pragma unroll
-            for (int v = 0; v < U / kStFin; ++v)
-                if (yb + v * kStFin < y1 && gx < W)
-                    strip_finish(o, tp.eps, done + v * kStFin * kStW, chunk + v * kStFin * G::CP, yb + v * kStFin, sums[v]);
+                for (int v = 0; v < U / kStFin; ++v)
+                    if (yb + v * kStFin < y1 && gx < W)
+                        strip_finish<decltype(vec)::value>(o, tp.eps, done + v * kStFin * kStW,
+                                                           chunk + v * kStFin * G::CP, yb + v * kStFin, sums[v]);
+            };
+            if (o.vec) finish(std::true_type());
+            else finish(std::false_type());
             __syncwarp();
             if (m + 2 < nout) asm volatile("bar.arrive %0, %1;" ::"r"(kEmpty + b), "n"(kStThreads) : "memory");
             if (J.cm) {  // (a chunk buffer's next writer is behind the next block's barrier)
                 asm volatile("bar.sync %0, %1;" ::"r"(kPair), "n"(kStFin * 32) : "memory");
-                strip_write_cm(J, g, s_chunk + (size_t)b * U * G::CP, G::CP, x0, y0 + m * U, y1);
+                strip_write_cm(J, g, s_chunk + (size_t)b * U * G::CP, G::CP, x0, y0 + m * U, y1,
+                               (int)threadIdx.x - kStChan * 32);
                 __syncwarp();
             }
         }

@@ -312,8 +312,8 @@ int auto_rule(int dtype, int m, int R, int family) {
     if (family != 0) return -1;
     if (corr_fft_supported(m, R)) return SFOC_CORR_FFT;
     // beyond, whatever the direct kernel serves (nothing else was ever accepted),
-    // by the Fourier form where that has a side: 4 us a point against 120 at
-    // m = 80, R = 60, 1.6 against 40 at m = 81, R = 36
+    // by the Fourier form where that has a side: 2.9 us a point against 112 at
+    // m = 80, R = 60, 1.4 against 40 at m = 81, R = 36
     if (!corr_f32_supported(m, R)) return -1;
     return corr_fft2_side(m, R) ? SFOC_CORR_FFT : SFOC_CORR_DIRECT_F32;
 }
