@@ -57,9 +57,18 @@ __device__ __forceinline__ float conv_odd(const float* x, int s, const float* t,
 }
 
 // image samples to intensities: float as is; uint16 scaled to [0, 1] by
-// v / 65535 (correctly rounded division)
+// v / 65535, correctly rounded: the product with the rounded reciprocal and one
+// correction by its exact residual (Markstein's step), which gives the rounded
+// quotient for each of the 65536 values (checked in exact arithmetic).  The
+// division and the integer conversion (a quarter of the FP32 rate) took a third of
+// the steering of a 16-bit image: 10000 x 10000, whole build 6342 -> 5704 us.
 __device__ __forceinline__ float to_unit(float v) { return v; }
-__device__ __forceinline__ float to_unit(uint16_t v) { return (float)v / 65535.f; }
+__device__ __forceinline__ float to_unit(uint16_t v) {
+    constexpr float c = 1.f / 65535.f;
+    const float x = __uint_as_float(0x4b000000u | v) - 8388608.f;
+    const float q = __fmul_rn(x, c);
+    return fmaf(fmaf(-q, 65535.f, x), c, q);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_sfoc_steer(const T* __restrict__ img, int H, int W, size_t pitch,

@@ -77,3 +77,10 @@ def test_batch_and_u16_equal_single(b, ctx, dt):
     # scalar as a product with the rounded reciprocal
     f = torch.from_numpy(v.cpu().numpy() / np.float32(65535.0)).cuda()
     assert torch.equal(ctx.sfoc_build_u16(u, p=p).export(), ctx.sfoc_build(f, p=p).export())
+
+
+def test_every_16_bit_value_is_correctly_rounded(b, ctx):
+    v = torch.arange(65536, dtype=torch.int32).reshape(256, 256)
+    u = torch.where(v >= 32768, v - 65536, v).to(torch.int16).cuda()
+    f = torch.from_numpy(v.numpy().astype(np.float32) / np.float32(65535.0)).cuda()
+    assert torch.equal(ctx.sfoc_build_u16(u).export(), ctx.sfoc_build(f).export())
