@@ -214,28 +214,29 @@ struct CubePlanes {
     __device__ __forceinline__ static float at(const T* r, int x) { return (float)r[x]; }
 };
 
-// Items: the points of `one` (items == nullptr) or (job, point) pairs of a
-// batch; with a queue the CTAs take items from an atomic counter (points of
-// uneven cost balance across the SMs), else item k goes to CTA k mod grid.
-// BF: the jobs' cubes are BF16 (12 channels), read from their planes.
-template <int L, bool BF>
-__global__ void __launch_bounds__(FftShape<L>::T, FftShape<L>::MINB)
-    k_corr_fft(const __grid_constant__ MatchJob one, const MatchJob* __restrict__ jobs,
-               const int2* __restrict__ items, int n_items, int* __restrict__ queue) {
+// One item: its window and template rows (in shared memory, read again after each
+// barrier, they hold no registers across the column passes, whose transforms set
+// the register peak), its sizes and its map.
+template <typename Src>
+struct FftItem {
+    Src S, T;
+    float* out;
+    int m, Lw, P1, z;
+    float tmean;
+    int clean;  // the window's non-finite values read as zeros
+};
+
+// The item's map.  Rows of Z at or past Lw are zero.  True (for every thread) where
+// the item is to be done again: a value of the map is not finite, and the
+// window's were read as they are.
+template <int L, typename Src>
+__device__ __forceinline__ bool fft_map(const FftItem<Src>& it, float2* fsm) {
     using Sh = FftShape<L>;
     constexpr int E = Sh::E, ZP = Sh::ZP, kFftGroups = Sh::G, kFftThreads = Sh::T;
-    extern __shared__ __align__(16) float2 fsm[];
-    __shared__ int s_item;
-    typedef CubePlanes<typename std::conditional<BF, __nv_bfloat16, float>::type> Src;
-    __shared__ Src s_src[2];  // the item's window and template rows
-    __shared__ float* s_out;
-    __shared__ int s_par[4];   // the item's m, m + 2R, 2R + 1, channels
-    __shared__ float s_tmean;  // the item's template mean
     float2* Z = fsm;                                       // L x ZP
     float2* scr = Z + (size_t)L * ZP;                      // kFftGroups x SG
     float2* tw = scr + (size_t)kFftGroups * Sh::SG;        // 8E twiddles W_L^{t k1} at 8 k1 + t
     float2* P64 = tw + 8 * E;                              // Nyquist column of the channel sum
-
     const int tid = threadIdx.x;
     const int grp = tid >> 3, t = tid & 7;
     const int lane = tid & 31, gbase = lane & ~7;
@@ -249,6 +250,142 @@ __global__ void __launch_bounds__(FftShape<L>::T, FftShape<L>::MINB)
     // partner of row t + 8m is row -(t + 8m): thread (8 - t) mod 8, index
     // (E - m) mod E for t = 0, E - 1 - m otherwise
     const int tpart = gbase + ((8 - t) & 7);
+
+    float2 acc[E];  // channel sum of X conj(Y) on column pr of this group's pair
+#pragma unroll
+    for (int j = 0; j < E; ++j) acc[j] = make_float2(0.f, 0.f);
+    for (int i = tid; i < L; i += kFftThreads) P64[i] = make_float2(0.f, 0.f);
+
+    for (int c = 0; c < it.z; ++c) {
+        const Src Sc = it.S, Tc = it.T;
+        const int m = it.m, Lw = it.Lw;
+        const float tmean = it.tmean;
+        const bool cl = it.clean;
+        // ---- rows: z = S + i (T - mean), zero outside the window / template
+        for (int y0 = 0; y0 < Lw; y0 += kFftGroups) {
+            const int y = y0 + yrow;
+            const bool rs = y < Lw, rt = y < m;
+            const auto srow = Sc.row(c, rs ? y : 0);
+            const auto trow = Tc.row(c, rt ? y : 0);
+            float2 v[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const int x = t + 8 * j;
+                v[j].x = (rs && x < Lw) ? Src::at(srow, x) : 0.f;
+                if (cl) v[j].x = isfinite(v[j].x) ? v[j].x : 0.f;
+                v[j].y = (rt && x < m) ? Src::at(trow, x) - tmean : 0.f;
+            }
+            group_fft<E, -1>(v, t, sc, tw);
+            if (rs) {
+#pragma unroll
+                for (int j = 0; j < E; ++j) Z[(size_t)y * ZP + t + 8 * j] = v[j];
+            }
+        }
+        __syncthreads();
+        // ---- columns in conjugate pairs, cross spectrum into the sums
+        {
+            const int pr = grp;  // pair pr: columns (pr, L - pr); pair 0: (0, L/2)
+            const int c1 = pr, c2 = pr == 0 ? L / 2 : L - pr;
+            float2 a[E], b[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                a[j] = Z[(size_t)(t + 8 * j) * ZP + c1];
+                b[j] = Z[(size_t)(t + 8 * j) * ZP + c2];
+            }
+            group_fft2<E, -1>(a, b, t, sc, tw);
+            // Z[-k] of column c1 lives in column c2 (in column c1 itself for
+            // pair 0).  Row -(t + 8j) is held by thread (8 - t) mod 8 at index
+            // E - 1 - j; for t = 0 by the thread itself at index (E - j) mod E.
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const float2 sb = make_float2(__shfl_sync(0xffffffffu, b[E - 1 - j].x, tpart),
+                                              __shfl_sync(0xffffffffu, b[E - 1 - j].y, tpart));
+                const float2 pb = t == 0 ? b[(E - j) & (E - 1)] : sb;
+                if (pr != 0) acc[j] = cadd(acc[j], cross_spectrum(a[j], make_float2(pb.x, -pb.y)));
+            }
+            if (pr == 0) {  // lanes 0-7 of warp 0: columns 0 and L/2 each pair with themselves
+#pragma unroll
+                for (int j = 0; j < E; ++j) {
+                    const float2 sa = make_float2(__shfl_sync(0xffu, a[E - 1 - j].x, tpart),
+                                                  __shfl_sync(0xffu, a[E - 1 - j].y, tpart));
+                    const float2 sb = make_float2(__shfl_sync(0xffu, b[E - 1 - j].x, tpart),
+                                                  __shfl_sync(0xffu, b[E - 1 - j].y, tpart));
+                    const float2 pa = t == 0 ? a[(E - j) & (E - 1)] : sa;
+                    const float2 pb = t == 0 ? b[(E - j) & (E - 1)] : sb;
+                    acc[j] = cadd(acc[j], cross_spectrum(a[j], make_float2(pa.x, -pa.y)));
+                    P64[t + 8 * j] = cadd(P64[t + 8 * j], cross_spectrum(b[j], make_float2(pb.x, -pb.y)));
+                }
+            }
+        }
+        __syncthreads();
+    }
+
+    const int P1i = it.P1;
+    // ---- inverse along the columns kx in [0, L/2]: rows y < 2R + 1 of Q in Z
+    {
+        const int pr = grp;
+        group_fft<E, 1>(acc, t, sc, tw);
+#pragma unroll
+        for (int j = 0; j < E; ++j)
+            if (t + 8 * j < P1i) Z[(size_t)(t + 8 * j) * ZP + pr] = acc[j];
+    }
+    {
+        float2 v[E];
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[j] = P64[t + 8 * j];
+        group_fft<E, 1>(v, t, sc, tw);  // every group computes it (uniform); group 0 stores it
+        if (grp == 0) {
+#pragma unroll
+            for (int j = 0; j < E; ++j)
+                if (t + 8 * j < P1i) Z[(size_t)(t + 8 * j) * ZP + L / 2] = v[j];
+        }
+    }
+    __syncthreads();
+    // ---- inverse along the rows (Hermitian extension), real part
+    float* out = it.out;
+    bool bad = false;
+    for (int y0 = 0; y0 < P1i; y0 += kFftGroups) {
+        const int y = y0 + yrow;
+        const int yy = y < P1i ? y : 0;
+        float2 v[E];
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            const int kx = t + 8 * j;
+            const float2 q = Z[(size_t)yy * ZP + (kx <= L / 2 ? kx : L - kx)];
+            v[j] = kx <= L / 2 ? q : make_float2(q.x, -q.y);
+        }
+        group_fft<E, 1>(v, t, sc, tw);
+        if (y < P1i) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const int x = t + 8 * j;
+                if (x < P1i) {
+                    out[(size_t)y * P1i + x] = v[j].x * inv_area;
+                    bad = bad || !isfinite(v[j].x);
+                }
+            }
+        }
+    }
+    return __syncthreads_or(bad && !it.clean) != 0;
+}
+
+// Items: the points of `one` (items == nullptr) or (job, point) pairs of a
+// batch; with a queue the CTAs take items from an atomic counter (points of
+// uneven cost balance across the SMs), else item k goes to CTA k mod grid.
+// BF: the jobs' cubes are BF16 (12 channels), read from their planes.
+template <int L, bool BF>
+__global__ void __launch_bounds__(FftShape<L>::T, FftShape<L>::MINB)
+    k_corr_fft(const __grid_constant__ MatchJob one, const MatchJob* __restrict__ jobs,
+               const int2* __restrict__ items, int n_items, int* __restrict__ queue) {
+    using Sh = FftShape<L>;
+    constexpr int E = Sh::E, ZP = Sh::ZP, kFftThreads = Sh::T;
+    extern __shared__ __align__(16) float2 fsm[];
+    __shared__ int s_item;
+    typedef CubePlanes<typename std::conditional<BF, __nv_bfloat16, float>::type> Src;
+    __shared__ FftItem<Src> s_it;
+    float2* const Z = fsm;                                                          // L x ZP
+    float2* const tw = Z + (size_t)L * ZP + (size_t)Sh::G * Sh::SG;                 // (as in fft_map)
+    const int tid = threadIdx.x;
 
     for (int p = tid; p < 8 * E; p += kFftThreads) {
         double s, c;
@@ -285,138 +422,34 @@ __global__ void __launch_bounds__(FftShape<L>::T, FftShape<L>::MINB)
             __syncthreads();
         }
         zhi = Lw;
-        // the item's window and template rows and its output, in shared memory:
-        // read again after each barrier, they hold no registers across the
-        // column passes (whose transforms set the kernel's register peak)
         if (tid == 0) {
             const int ty0 = J.pts[2 * k + 1] - h, tx0 = J.pts[2 * k] - h;
             const int wy0 = ty0 - R, wx0 = tx0 - R;
             if constexpr (BF) {
-                s_src[0] = Src{J.rpl + (size_t)wy0 * J.rpitch + wx0, J.rplane, (unsigned)J.rpitch};
-                s_src[1] = Src{J.spl + (size_t)ty0 * J.spitch + tx0, J.splane, (unsigned)J.spitch};
+                s_it.S = Src{J.rpl + (size_t)wy0 * J.rpitch + wx0, J.rplane, (unsigned)J.rpitch};
+                s_it.T = Src{J.spl + (size_t)ty0 * J.spitch + tx0, J.splane, (unsigned)J.spitch};
             } else {
-                s_src[0] = Src{J.rf32 + (size_t)wy0 * J.rpitch + wx0, J.rplane, (unsigned)J.rpitch};
-                s_src[1] = Src{J.sf32 + (size_t)ty0 * J.spitch + tx0, J.splane, (unsigned)J.spitch};
+                s_it.S = Src{J.rf32 + (size_t)wy0 * J.rpitch + wx0, J.rplane, (unsigned)J.rpitch};
+                s_it.T = Src{J.sf32 + (size_t)ty0 * J.spitch + tx0, J.splane, (unsigned)J.spitch};
             }
-            s_out = J.maps + (size_t)k * P1 * P1;
-            s_par[0] = m;
-            s_par[1] = Lw;
-            s_par[2] = P1;
-            s_par[3] = z;
-            s_tmean = st.tmean;
+            s_it.out = J.maps + (size_t)k * P1 * P1;
+            s_it.m = m;
+            s_it.Lw = Lw;
+            s_it.P1 = P1;
+            s_it.z = z;
+            s_it.tmean = st.tmean;
+            s_it.clean = 0;
         }
         __syncthreads();
-
-        float2 acc[E];  // channel sum of X conj(Y) on column pr of this group's pair
-#pragma unroll
-        for (int j = 0; j < E; ++j) acc[j] = make_float2(0.f, 0.f);
-        for (int i = tid; i < L; i += kFftThreads) P64[i] = make_float2(0.f, 0.f);
-
-        for (int c = 0; c < s_par[3]; ++c) {
-            const Src Sc = s_src[0], Tc = s_src[1];
-            const int m = s_par[0], Lw = s_par[1];
-            const float tmean = s_tmean;
-            // ---- rows: z = S + i (T - mean), zero outside the window / template
-            for (int y0 = 0; y0 < Lw; y0 += kFftGroups) {
-                const int y = y0 + yrow;
-                const bool rs = y < Lw, rt = y < m;
-                const auto srow = Sc.row(c, rs ? y : 0);
-                const auto trow = Tc.row(c, rt ? y : 0);
-                float2 v[E];
-#pragma unroll
-                for (int j = 0; j < E; ++j) {
-                    const int x = t + 8 * j;
-                    v[j].x = (rs && x < Lw) ? Src::at(srow, x) : 0.f;
-                    v[j].y = (rt && x < m) ? Src::at(trow, x) - tmean : 0.f;
-                }
-                group_fft<E, -1>(v, t, sc, tw);
-                if (rs) {
-#pragma unroll
-                    for (int j = 0; j < E; ++j) Z[(size_t)y * ZP + t + 8 * j] = v[j];
-                }
-            }
-            __syncthreads();
-            // ---- columns in conjugate pairs, cross spectrum into the sums
-            {
-                const int pr = grp;  // pair pr: columns (pr, L - pr); pair 0: (0, L/2)
-                const int c1 = pr, c2 = pr == 0 ? L / 2 : L - pr;
-                float2 a[E], b[E];
-#pragma unroll
-                for (int j = 0; j < E; ++j) {
-                    a[j] = Z[(size_t)(t + 8 * j) * ZP + c1];
-                    b[j] = Z[(size_t)(t + 8 * j) * ZP + c2];
-                }
-                group_fft2<E, -1>(a, b, t, sc, tw);
-                // Z[-k] of column c1 lives in column c2 (in column c1 itself for
-                // pair 0).  Row -(t + 8j) is held by thread (8 - t) mod 8 at index
-                // E - 1 - j; for t = 0 by the thread itself at index (E - j) mod E.
-#pragma unroll
-                for (int j = 0; j < E; ++j) {
-                    const float2 sb = make_float2(__shfl_sync(0xffffffffu, b[E - 1 - j].x, tpart),
-                                                  __shfl_sync(0xffffffffu, b[E - 1 - j].y, tpart));
-                    const float2 pb = t == 0 ? b[(E - j) & (E - 1)] : sb;
-                    if (pr != 0) acc[j] = cadd(acc[j], cross_spectrum(a[j], make_float2(pb.x, -pb.y)));
-                }
-                if (pr == 0) {  // lanes 0-7 of warp 0: columns 0 and L/2 each pair with themselves
-#pragma unroll
-                    for (int j = 0; j < E; ++j) {
-                        const float2 sa = make_float2(__shfl_sync(0xffu, a[E - 1 - j].x, tpart),
-                                                      __shfl_sync(0xffu, a[E - 1 - j].y, tpart));
-                        const float2 sb = make_float2(__shfl_sync(0xffu, b[E - 1 - j].x, tpart),
-                                                      __shfl_sync(0xffu, b[E - 1 - j].y, tpart));
-                        const float2 pa = t == 0 ? a[(E - j) & (E - 1)] : sa;
-                        const float2 pb = t == 0 ? b[(E - j) & (E - 1)] : sb;
-                        acc[j] = cadd(acc[j], cross_spectrum(a[j], make_float2(pa.x, -pa.y)));
-                        P64[t + 8 * j] = cadd(P64[t + 8 * j], cross_spectrum(b[j], make_float2(pb.x, -pb.y)));
-                    }
-                }
-            }
+        // A non-finite value of the window may not reach the offsets whose windows do
+        // not hold it (the tensor-core forms keep it apart too, and which form a window
+        // gets is a matter of measured time): once more, with zeros in its place.
+        // (With the test as a branch around the row's values this cost 2 % at side
+        // 64, with a second body 1 to 3 % at both sides; as a select it costs nothing.)
+        while (fft_map<L>(s_it, fsm)) {
+            if (tid == 0) s_it.clean = 1;
             __syncthreads();
         }
-
-        const int P1i = s_par[2];
-        // ---- inverse along the columns kx in [0, L/2]: rows y < 2R + 1 of Q in Z
-        {
-            const int pr = grp;
-            group_fft<E, 1>(acc, t, sc, tw);
-#pragma unroll
-            for (int j = 0; j < E; ++j)
-                if (t + 8 * j < P1i) Z[(size_t)(t + 8 * j) * ZP + pr] = acc[j];
-        }
-        {
-            float2 v[E];
-#pragma unroll
-            for (int j = 0; j < E; ++j) v[j] = P64[t + 8 * j];
-            group_fft<E, 1>(v, t, sc, tw);  // every group computes it (uniform); group 0 stores it
-            if (grp == 0) {
-#pragma unroll
-                for (int j = 0; j < E; ++j)
-                    if (t + 8 * j < P1i) Z[(size_t)(t + 8 * j) * ZP + L / 2] = v[j];
-            }
-        }
-        __syncthreads();
-        // ---- inverse along the rows (Hermitian extension), real part
-        float* out = s_out;
-        for (int y0 = 0; y0 < P1i; y0 += kFftGroups) {
-            const int y = y0 + yrow;
-            const int yy = y < P1i ? y : 0;
-            float2 v[E];
-#pragma unroll
-            for (int j = 0; j < E; ++j) {
-                const int kx = t + 8 * j;
-                const float2 q = Z[(size_t)yy * ZP + (kx <= L / 2 ? kx : L - kx)];
-                v[j] = kx <= L / 2 ? q : make_float2(q.x, -q.y);
-            }
-            group_fft<E, 1>(v, t, sc, tw);
-            if (y < P1i) {
-#pragma unroll
-                for (int j = 0; j < E; ++j) {
-                    const int x = t + 8 * j;
-                    if (x < P1i) out[(size_t)y * P1i + x] = v[j].x * inv_area;
-                }
-            }
-        }
-        __syncthreads();
     }
 }
 
@@ -444,7 +477,7 @@ cudaError_t launch_corr_fft(const MatchJob& one, const ItemSet& is, int L, bool 
         const int smem = (int)FftShape<LV>::smem;                                                                 \
         e = cudaFuncSetAttribute(k_corr_fft<LV, BV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);         \
         if (e != cudaSuccess) return e;                                                                           \
-        const int slots = sms * FftShape<LV>::MINB, grid = n < slots ? n : slots;                                                                       \
+        const int slots = sms * FftShape<LV>::MINB, grid = n < slots ? n : slots;                                 \
         k_corr_fft<LV, BV><<<grid, FftShape<LV>::T, smem, st>>>(one, is.jobs, is.items, n, is.queue);             \
     }
     if (L == 64) {

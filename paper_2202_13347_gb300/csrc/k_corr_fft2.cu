@@ -761,10 +761,11 @@ __global__ void __launch_bounds__(FftShape<L>::NT, FftShape<L>::MINB)
                     }
                     __syncwarp();
                 }
-                // sides above 128: a non-finite value of the window may not reach the
-                // offsets whose windows do not hold it (the forms that served these
-                // windows before kept them apart): once more, with zeros in their place
-                if (__syncthreads_or(bad && L > 128 && !clean)) again = true;
+                // a non-finite value of the window may not reach the offsets whose windows
+                // do not hold it (the tensor-core forms keep it apart too, and which form a
+                // window gets is a matter of measured time): once more, with zeros in its
+                // place
+                if (__syncthreads_or(bad && !clean)) again = true;
             }
             if (again) break;
         }
