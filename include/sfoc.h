@@ -554,8 +554,9 @@ SFOC_API sfoc_status fastncc_ransac(sfoc_ctx* ctx, const double* d_src, const do
  * into the reference frame with a model H (sensed -> reference, 9 doubles
  * row-major in device memory, e.g. fastncc_ransac's d_model): output pixel
  * (x, y) of the out_h x out_w image d_out takes the bilinear sample of
- * d_image at H^-1 (x, y), or `fill` outside [0, W-1] x [0, H-1].  Mapping in
- * FP64, blend in FP32.  A singular model gives an all-fill image.  Device
+ * d_image at H^-1 (x, y), or `fill` outside [0, W-1] x [0, H-1].  Positions
+ * within 2^-24 px of the FP64 mapping's (2^-27 without perspective), their
+ * fraction rounded to FP32 once; blend in FP32.  A singular model gives an all-fill image.  Device
  * memory owned by the caller; asynchronous on the context stream.
  * INVALID_ARG for null pointers, H, W, out_h or out_w < 1, pitch < W.
  */

@@ -587,32 +587,33 @@ __global__ void __cluster_dims__(kRsCtas, 1, 1) __launch_bounds__(kRsThreads)
 // FP64, (u0, t0) at (x0, y0), and steps from it exactly:
 //   u(x0 + i, y0 + k) = u0 + d / (1 + e),  d = i sx + k sy,  e = i qx + k qy,
 //   sx = (a - g u0) / w0, sy = (b - h u0) / w0, qx = g / w0, qy = h / w0
-// (a, b, g, h the model's x row and its last row).  The steps are kept as a
-// float whose product with i or k is exact plus a float remainder, and the
-// integer parts are split off before the fractions are added, so a position
-// is within ~2^-23 px of the FP64 one wherever it lies (FP32 rounds the
-// fraction to 2^-25 in either form).  Tiles with a strong perspective or
-// scale, and pixels mapped within 2^-10 px of the image's border lines (where
-// a rounding could decide inside or outside), take the FP64 mapping itself.
-// Tiles well inside the image (most) skip the border tests.  2048 x 2048: 25 us
-// (29 with the tests everywhere and the rounding instructions).
+// (a, b, g, h the model's x row and its last row).  Positions and steps are
+// 64-bit integers in 2^-32 px, so that u0 + d is exact but for the steps'
+// roundings (at most 40 x 2^-33 px); the rest, -d e / (1 + e), is below 1/16 px
+// on the tiles that take this route and comes from FP32 with at most
+// 9 x 2^-24 of its size in error.  A position is thus within 2^-24 px of the FP64
+// one wherever it lies (2^-27 without perspective), and its fraction is rounded
+// to FP32 once, as after the FP64 mapping: the values of a noise image are
+// 1.94e-8 rms from float64 either way.  (With FP32 fractions added up they were
+// 3.4e-8, positions up to 2^-22 px off, and the call no faster: 2048 x 2048 25.4
+// us, with this 25.1.)
+// Tiles with a strong perspective or scale, and pixels mapped within 2^-10 px of
+// the image's border lines (where a rounding could decide inside or outside),
+// take the FP64 mapping itself.  Tiles well inside the image (most) skip the
+// border tests.
 // The CTA's first warp prepares up to 32 tiles, one per lane (inverse, tile
 // maps: a chain of ~1500 clocks whose length does not depend on their
 // number), so large images give a warp four tiles (kRectTiles) and small ones
 // one, which keeps more CTAs.
 constexpr int kRectW = 32, kRectH = 8, kRectTiles = 4, kRectB = 4;
+typedef unsigned long long u64;
 struct RectTile {
-    int nu, nt;                 // integer parts of u0, t0
-    float fu, ft;               // fractions
-    float sx[2], sxl[2], sy[2], syl[2];  // per axis (u, t): steps, high part and remainder
+    u64 p[2], sx[2], sy[2];     // per axis (u, t): position of the tile's first pixel and steps, 2^-32 px
+    float fsx[2], fsy[2];       // the steps
     float qx, qy;
     int ok;                     // the steps serve the whole tile: 2 if all of it maps at least a pixel inside
                                 // the image's border lines, else 1
 };
-
-// floor(x) of |x| < 2^22 as the sum x + 1.5 x 2^23 rounded down: its last bits are
-// the integer (the rounding instructions run at a quarter of the FP32 rate)
-constexpr float kFloorM = 12582912.f;
 
 // one pixel by the FP64 mapping
 __device__ __noinline__ float rect_fp64(const float* __restrict__ img, int H, int W, size_t pitch, const double* inv,
@@ -640,15 +641,13 @@ __device__ __forceinline__ void rect_tile(const float* __restrict__ img, int H, 
     constexpr int kB = INSIDE ? kRectB : 2;  // (the general form holds twice as much per row)
     const float fi = (float)lane;
     // inside, samples are addressed by 32-bit offsets from the tile's first one
-    const float* const base = INSIDE ? img + (size_t)T.nt * pitch + T.nu : img;
-    // the column part of the steps: d = i sx split into integer and fraction
-    int npx[2];
-    float fpx[2];
+    const float* const base = INSIDE ? img + (size_t)(T.p[1] >> 32) * pitch + (size_t)(T.p[0] >> 32) : img;
+    u64 pos[2];   // this column at the current row
+    float dx[2];  // its steps from the tile's first pixel
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        const float p = fi * T.sx[q], r = __fadd_rd(p, kFloorM);
-        fpx[q] = p - (r - kFloorM);
-        npx[q] = (INSIDE ? 0 : q ? T.nt : T.nu) + __float_as_int(r) - 3 * __float_as_int(kFloorM);
+        pos[q] = (INSIDE ? T.p[q] & 0xffffffffull : T.p[q]) + (u64)lane * T.sx[q];
+        dx[q] = fi * T.fsx[q];
     }
     // kB rows at a time: their positions, then all their samples in flight,
     // then the blends (with one row after the other the kernel waited for every
@@ -669,13 +668,11 @@ __device__ __forceinline__ void rect_tile(const float* __restrict__ img, int H, 
             float fr[2];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const float p = fk * T.sy[q], rp = __fadd_rd(p, kFloorM), fp = p - (rp - kFloorM);
-                // remainders of the steps, and the perspective term
-                const float corr = fmaf(-e, fmaf(fi, T.sx[q], p), fmaf(fi, T.sxl[q], fk * T.syl[q]));
-                const float f = (q ? T.ft : T.fu) + ((fpx[q] + fp) + corr);
-                const float rc = __fadd_rd(f, kFloorM);
-                fr[q] = f - (rc - kFloorM);
-                ci[q] = npx[q] + __float_as_int(rp) + __float_as_int(rc);
+                const float c = -e * fmaf(fk, T.fsy[q], dx[q]);  // the perspective term
+                const u64 at64 = pos[q] + (u64)(long long)__float2int_rn(c * 4294967296.f);
+                pos[q] += T.sy[q];
+                ci[q] = (int)(at64 >> 32);
+                fr[q] = __uint2float_rn((unsigned)at64) * (1.f / 4294967296.f);
             }
             ld[b] = true;
             if (!INSIDE) {
@@ -763,33 +760,31 @@ __global__ void __launch_bounds__(kRsThreads, 4)
             const double qx = s_inv[6] * rw, qy = s_inv[7] * rw;
             bool ok = s_ok && fabs(p[0]) < 1e8 && fabs(p[1]) < 1e8 &&
                       fabs(qx) * kRectW + fabs(qy) * kRectH < 1.0 / 1024;
-            const double n0 = floor(p[0]), n1 = floor(p[1]);
-            T.fu = (float)(p[0] - n0);
-            T.ft = (float)(p[1] - n1);
+            T.qx = (float)qx;
+            T.qy = (float)qy;
+            const float reach = fabsf(T.qx) * (kRectW - 1) + fabsf(T.qy) * (kRectH - 1);  // the largest |e|
+            constexpr double k32 = 4294967296.0;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const double sx = (s_inv[3 * q] - s_inv[6] * p[q]) * rw, sy = (s_inv[3 * q + 1] - s_inv[7] * p[q]) * rw;
-                ok = ok && fabs(sx) < 4.0 && fabs(sy) < 4.0;
-                // 19 (21) significant bits: the product with i < 32 (k < 8) is exact
-                T.sx[q] = __uint_as_float(__float_as_uint((float)sx) & 0xffffffe0u);
-                T.sy[q] = __uint_as_float(__float_as_uint((float)sy) & 0xfffffff8u);
-                T.sxl[q] = (float)(sx - (double)T.sx[q]);
-                T.syl[q] = (float)(sy - (double)T.sy[q]);
+                T.fsx[q] = (float)sx;
+                T.fsy[q] = (float)sy;
+                ok = ok && fabs(sx) < 4.0 && fabs(sy) < 4.0 &&
+                     (fabsf(T.fsx[q]) * (kRectW - 1) + fabsf(T.fsy[q]) * (kRectH - 1)) * reach < 1.f / 16;
+                T.p[q] = (u64)__double2ll_rn(p[q] * k32);
+                T.sx[q] = (u64)__double2ll_rn(sx * k32);
+                T.sy[q] = (u64)__double2ll_rn(sy * k32);
             }
-            T.qx = (float)qx;
-            T.qy = (float)qy;
             // how far the tile reaches to either side, with 1 % for the perspective
             bool in = ok && pitch < ((size_t)1 << 23);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const float c = (float)p[q], last = (float)((q ? H : W) - 1);
-                const float ex = (kRectW - 1) * T.sx[q], ey = (kRectH - 1) * T.sy[q];
+                const float ex = (kRectW - 1) * T.fsx[q], ey = (kRectH - 1) * T.fsy[q];
                 in = in && c + 1.01f * (fminf(ex, 0.f) + fminf(ey, 0.f)) > 2.f &&
                      c + 1.01f * (fmaxf(ex, 0.f) + fmaxf(ey, 0.f)) < last - 2.f && last < 4194304.f;
             }
             T.ok = in ? 2 : ok ? 1 : 0;
-            T.nu = ok ? (int)n0 : 0;
-            T.nt = ok ? (int)n1 : 0;
             s_tile[lane] = T;
         }
     }
