@@ -117,6 +117,11 @@ struct StageScope {
     int stage, launches;
     cudaEvent_t a = nullptr;
     StageScope(sfoc_ctx* ctx, int st, int nl);
+    // launches known only once they are made
+    void add(int nl) {
+        launches += nl;
+        c->launches += nl;
+    }
     ~StageScope();
 };
 

@@ -875,10 +875,11 @@ sfoc_status fastncc_ransac(sfoc_ctx* ctx, const double* d_src, const double* d_d
     if (s != SFOC_OK) return s;
     cudaError_t e;
     {
-        StageScope sc(ctx, ST_OTHER, n_hyp > 0 ? 3 : 2);
+        StageScope sc(ctx, ST_OTHER, 0);
         int nl = 0;
         e = launch_ransac(d_src, d_dst, d_valid, n, model == SFOC_MODEL_PROJECTIVE ? 1 : 0, d_samples, n_hyp,
                           threshold, refits, d_model, d_inlier, d_info, d_scores, ctx->ws, ctx->stream, &nl);
+        sc.add(nl);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "ransac launch");
     return SFOC_OK;

@@ -1,0 +1,83 @@
+"""Host-side state of the C ABI on the CPU: the library's host sources over a fake
+CUDA runtime (host_fake.cpp), where allocations are counted and limited, launches
+counted and timed by a table."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CSRC = os.path.join(ROOT, "paper_2202_13347_gb300", "csrc")
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+F32, BF16 = 0, 1
+AUTO, DIRECT, BAND, FFT = 0, 1, 5, 6
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("host")
+    fake = os.path.join(HERE, "host_fake.cpp")
+    flags = ["-std=c++17", "-O1", "-w", "-Wno-psabi", "-fPIC", "-I", os.path.join(CUDA, "include"), "-I", os.path.join(ROOT, "include"),
+             "-I", CSRC, "-x", "c++"]
+    objs = []
+    for src in (os.path.join(CSRC, "sfoc_api.cu"), os.path.join(CSRC, "batch.cu"), fake):
+        objs.append(str(d / (os.path.basename(src) + ".o")))
+        shim = [] if src == fake else ["-DHOST_SHIM", "-include", fake]
+        subprocess.run(["g++"] + flags + shim + ["-c", src, "-o", objs[-1]], check=True)
+    so = str(d / "host.so")
+    subprocess.run(["g++", "-shared", "-o", so, "-Wl,-z,lazy"] + objs, check=True)   # the rest is bound when called
+    L = C.CDLL(so, mode=os.RTLD_LAZY)
+    L.fk_live.restype = L.fk_bytes.restype = C.c_size_t
+    L.fk_limit.argtypes = [C.c_size_t]
+    L.fk_cost.argtypes = [C.c_int, C.c_int, C.c_double]
+    L.sfoc_ctx_launch_count.restype = C.c_int64
+    L.sfoc_ctx_launch_count.argtypes = [C.c_void_p]
+    return L
+
+
+class Ctx:
+    """A context of the faked library; points and images are addresses nothing reads."""
+
+    def __init__(self, lib):
+        self.L, self.h = lib, C.c_void_p()
+        lib.fk_limit(C.c_size_t(-1).value)
+        lib.fk_capturing(0)
+        assert lib.sfoc_ctx_create(C.byref(self.h), 0, None) == 0
+        lib.fk_reset()
+
+    def close(self):
+        assert self.L.sfoc_ctx_destroy(self.h) == 0
+
+    def pair(self, ref, sen, n=10, m=41, R=10, p=None):
+        a = C.c_void_p(4096)
+        return self.L.fastncc_register_pair(self.h, a, ref[0], ref[1], a, sen[0], sen[1], a, n, m, R, p, None, a)
+
+    def build(self, H, W, p=None, out=None):
+        c = C.c_void_p(out)
+        assert self.L.sfoc_build(self.h, C.c_void_p(4096), H, W, C.c_size_t(W), None, 0, 0, p, C.byref(c)) == 0
+        return c
+
+    def match(self, a, b, n, m, R):
+        p = C.c_void_p(4096)
+        assert self.L.fastncc_match(self.h, a, b, p, n, m, R, None, p) == 0
+        return self.L.fk_last_form()
+
+    def launches(self):
+        return self.L.sfoc_ctx_launch_count(self.h)
+
+
+@pytest.fixture()
+def ctx(lib):
+    c = Ctx(lib)
+    yield c
+    c.close()
+
+
+def test_ransac_counts_the_launches_its_launcher_reports(ctx):
+    a, before = C.c_void_p(4096), ctx.launches()
+    for hyps, want in ((16, 4), (0, 2)):
+        assert ctx.L.fastncc_ransac(ctx.h, a, a, None, 8, 1, a, hyps, C.c_double(1.5), 1, a, a, a, None) == 0
+        assert ctx.launches() - before == want
+        before = ctx.launches()
