@@ -735,6 +735,7 @@ void key_cube(KeyWriter& k, const sfoc_cube* c) {
     k.p(c->c.f32);
     k.p(c->c.rm);
     k.p(c->c.cm);
+    k.p(c->c.pl);
     k.p(c->c.s1);
     k.p(c->c.s2);
     k.p(c->c.integ);

@@ -27,11 +27,13 @@ def lib(tmp_path_factory):
         shim = [] if src == fake else ["-DHOST_SHIM", "-include", fake]
         subprocess.run(["g++"] + flags + shim + ["-c", src, "-o", objs[-1]], check=True)
     so = str(d / "host.so")
-    subprocess.run(["g++", "-shared", "-o", so, "-Wl,-z,lazy"] + objs, check=True)   # the rest is bound when called
+    subprocess.run(["g++", "-shared", "-o", so, "-Wl,-z,lazy", "-Wl,-Bsymbolic"] + objs, check=True)   # the rest is bound when called
     L = C.CDLL(so, mode=os.RTLD_LAZY)
     L.fk_live.restype = L.fk_bytes.restype = C.c_size_t
     L.fk_limit.argtypes = [C.c_size_t]
     L.fk_cost.argtypes = [C.c_int, C.c_int, C.c_double]
+    L.sfoc_last_error_string.restype = C.c_char_p
+    L.sfoc_last_error_string.argtypes = [C.c_void_p]
     L.sfoc_ctx_launch_count.restype = C.c_int64
     L.sfoc_ctx_launch_count.argtypes = [C.c_void_p]
     return L
@@ -46,6 +48,9 @@ class Ctx:
         lib.fk_capturing(0)
         assert lib.sfoc_ctx_create(C.byref(self.h), 0, None) == 0
         lib.fk_reset()
+
+    def ok(self, rc):
+        assert rc == 0, self.L.sfoc_last_error_string(self.h).decode()
 
     def close(self):
         assert self.L.sfoc_ctx_destroy(self.h) == 0
@@ -81,3 +86,49 @@ def test_ransac_counts_the_launches_its_launcher_reports(ctx):
         assert ctx.L.fastncc_ransac(ctx.h, a, a, None, 8, 1, a, hyps, C.c_double(1.5), 1, a, a, a, None) == 0
         assert ctx.launches() - before == want
         before = ctx.launches()
+
+
+def params(ctx, dtype):
+    from paper_2202_13347_gb300.binding import Params
+    p = Params()
+    assert ctx.L.sfoc_params_default(C.byref(p)) == 0
+    p.cube_dtype = dtype
+    return C.byref(p)
+
+
+def plans_built(ctx):
+    n = C.c_size_t()
+    assert ctx.L.sfoc_ctx_plan_info(ctx.h, None, 0, C.byref(n)) == 0
+    buf = C.create_string_buffer(n.value)
+    assert ctx.L.sfoc_ctx_plan_info(ctx.h, buf, n.value, C.byref(n)) == 0
+    return int(buf.value.decode().split('"plans_built": ')[1].split(",")[0].split("}")[0])
+
+
+def test_a_batch_plan_is_not_kept_for_a_cube_whose_planes_moved(ctx):
+    """A cube freed and built again may come back at the same addresses but for one
+    buffer: a plan holds that buffer's address in its tables."""
+    H, W = 300, 320
+    plane = 2 * 12 * 320 * H      # the BF16 planes: rows of 32 elements' multiples
+    p = params(ctx, BF16)
+    arr = lambda t, v: (t * 1)(v)  # noqa: E731
+    sen = ctx.build(H, W, p)
+
+    def match(ref):
+        ctx.ok(ctx.L.fastncc_match_batch(ctx.h, 1, arr(C.c_void_p, ref.value), arr(C.c_void_p, sen.value),
+                                         arr(C.c_void_p, 4096), arr(C.c_int, 50), arr(C.c_int, 41), arr(C.c_int, 10),
+                                         None, arr(C.c_void_p, 4096)))
+        return plans_built(ctx)
+
+    ref = ctx.build(H, W, p)
+    n = match(ref)
+    assert match(ref) == n
+    assert ctx.L.sfoc_cube_free(ref) == 0
+    held = C.c_void_p()
+    assert ctx.L.cudaMalloc(C.byref(held), C.c_size_t(plane)) == 0   # takes the freed planes' place
+    again = ctx.build(H, W, p)
+    if again.value != ref.value:
+        pytest.skip("the host allocator moved the cube itself")
+    assert match(again) == n + 1
+    for c in (again, sen):
+        assert ctx.L.sfoc_cube_free(c) == 0
+    assert ctx.L.cudaFree(held) == 0
