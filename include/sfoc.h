@@ -312,7 +312,9 @@ SFOC_API sfoc_status fastncc_match(sfoc_ctx* ctx, sfoc_cube* ref, sfoc_cube* sen
 /*
  * fastncc_register_pair - the whole fine-registration path for one pair:
  * sfoc_build of both images, then fastncc_match.  Device buffers.  The two
- * cubes are cached in the context and reused while the shapes stay equal.
+ * cubes are cached in the context and reused while the shapes stay equal; a
+ * call of other shapes or another cube type frees them (after the stream's
+ * queued work), unless a captured graph uses them.
  */
 SFOC_API sfoc_status fastncc_register_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, const float* d_sen,
                                   int Hs, int Ws, const int32_t* d_points, int n, int template_size,

@@ -51,6 +51,7 @@ struct sfoc_ctx {
     // cached cubes and staging for the pair pipeline
     sfoc_cube* pair_ref = nullptr;
     sfoc_cube* pair_sen = nullptr;
+    std::vector<sfoc_cube*> retired;  // replaced ones that a captured graph may still read
     void* stage = nullptr;
     size_t stage_bytes = 0;
     // second stream for the sensed image's host copy (overlaps the reference cube)
@@ -92,6 +93,7 @@ struct sfoc_ctx {
 
 struct sfoc_cube {
     sfoc::Cube c;
+    bool in_graph = false;  // a pair cube that work captured into a graph uses
 };
 
 namespace sfoc {

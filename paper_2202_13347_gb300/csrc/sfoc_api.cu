@@ -465,6 +465,32 @@ sfoc_status build_cube(sfoc_ctx* ctx, const T* d_image, int H, int W, size_t pit
     return SFOC_OK;
 }
 
+// Puts a cube into one of the context's pair slots.  The cube it replaces (of
+// another shape or type) is freed once the work queued on the stream is done
+// with it; one that a captured graph may read lives as long as the context.
+void set_pair_cube(sfoc_ctx* ctx, sfoc_cube** slot, sfoc_cube* cube) {
+    sfoc_cube* const old = *slot;
+    const bool cap = capturing(ctx->stream);
+    *slot = cube;
+    cube->in_graph = cube->in_graph || cap;
+    if (!old || old == cube) return;
+    if (cap || old->in_graph) {
+        ctx->retired.push_back(old);
+        return;
+    }
+    cudaStreamSynchronize(ctx->stream);
+    sfoc_cube_free(old);
+}
+
+// sfoc_build of a dense image into a pair slot
+sfoc_status build_pair_cube(sfoc_ctx* ctx, const float* d_image, int H, int W, const sfoc_params* p,
+                            sfoc_cube** slot) {
+    sfoc_cube* cube = *slot;
+    const sfoc_status s = build_cube(ctx, d_image, H, W, (size_t)W, nullptr, 0, 0, p, &cube);
+    if (s == SFOC_OK) set_pair_cube(ctx, slot, cube);
+    return s;
+}
+
 // The most pixels of a pair whose two cubes are built in one launch per kernel:
 // a pair of 1024 x 1024 images.  A small image leaves most of the chip idle, and
 // its three launches are a chain of latencies; the whole call, one image after
@@ -508,16 +534,17 @@ sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, 
     sfoc_status s = ensure_ws(ctx, at[2]);
     if (s != SFOC_OK) return s;
     for (int k = 0; k < 2; ++k) {
-        if (fits[k]) continue;
-        // (the cube it replaces stays, as with sfoc_build: a captured graph may read it)
-        sfoc_cube* c = new (std::nothrow) sfoc_cube();
-        if (!c) return fail(ctx, SFOC_ERR_OOM, "host allocation");
-        s = alloc_cube(ctx, c->c, H[k], W[k], z, p.cube_dtype);
-        if (s != SFOC_OK) {
-            delete c;
-            return s;
+        sfoc_cube* c = *cube[k];
+        if (!fits[k]) {
+            c = new (std::nothrow) sfoc_cube();
+            if (!c) return fail(ctx, SFOC_ERR_OOM, "host allocation");
+            s = alloc_cube(ctx, c->c, H[k], W[k], z, p.cube_dtype);
+            if (s != SFOC_OK) {
+                delete c;
+                return s;
+            }
         }
-        *cube[k] = c;
+        set_pair_cube(ctx, cube[k], c);
     }
     ImgJob two[2];
     memset(two, 0, sizeof(two));
@@ -578,6 +605,7 @@ sfoc_status sfoc_ctx_destroy(sfoc_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
     if (ctx->pair_ref) sfoc_cube_free(ctx->pair_ref);
     if (ctx->pair_sen) sfoc_cube_free(ctx->pair_sen);
+    for (sfoc_cube* c : ctx->retired) sfoc_cube_free(c);
     cudaFree(ctx->ws);
     cudaFree(ctx->stage);
     cudaFree(ctx->d_err);
@@ -989,9 +1017,9 @@ sfoc_status fastncc_register_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int
     sfoc_status s = ctx->timing ? SFOC_OK : build_small_pair(ctx, d_ref, Hr, Wr, d_sen, Hs, Ws, p, &both);
     if (s != SFOC_OK) return s;
     if (!both) {  // (per-stage timing keeps the steering and smoothing launches apart)
-        s = sfoc_build(ctx, d_ref, Hr, Wr, (size_t)Wr, nullptr, 0, 0, p, &ctx->pair_ref);
+        s = build_pair_cube(ctx, d_ref, Hr, Wr, p, &ctx->pair_ref);
         if (s != SFOC_OK) return s;
-        s = sfoc_build(ctx, d_sen, Hs, Ws, (size_t)Ws, nullptr, 0, 0, p, &ctx->pair_sen);
+        s = build_pair_cube(ctx, d_sen, Hs, Ws, p, &ctx->pair_sen);
         if (s != SFOC_OK) return s;
     }
     return fastncc_match(ctx, ctx->pair_ref, ctx->pair_sen, d_points, n, template_size, search_radius, opts, d_out);
@@ -1052,11 +1080,11 @@ sfoc_status fastncc_register_pair_host(sfoc_ctx* ctx, const float* h_ref, int Hr
         return st;
     };
     if (e != cudaSuccess) return drained(cuda_fail(ctx, e, "host to device copy"));
-    sfoc_status s = sfoc_build(ctx, d_ref, Hr, Wr, (size_t)Wr, nullptr, 0, 0, p, &ctx->pair_ref);
+    sfoc_status s = build_pair_cube(ctx, d_ref, Hr, Wr, p, &ctx->pair_ref);
     if (s != SFOC_OK) return drained(s);
     e = cudaStreamWaitEvent(ctx->stream, ctx->ev_copied, 0);
     if (e != cudaSuccess) return drained(cuda_fail(ctx, e, "cudaStreamWaitEvent"));
-    s = sfoc_build(ctx, d_sen, Hs, Ws, (size_t)Ws, nullptr, 0, 0, p, &ctx->pair_sen);
+    s = build_pair_cube(ctx, d_sen, Hs, Ws, p, &ctx->pair_sen);
     if (s == SFOC_OK)
         s = fastncc_match(ctx, ctx->pair_ref, ctx->pair_sen, d_pts, n, template_size, search_radius, opts, d_out);
     if (s != SFOC_OK) return drained(s);

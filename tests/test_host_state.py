@@ -132,3 +132,34 @@ def test_a_batch_plan_is_not_kept_for_a_cube_whose_planes_moved(ctx):
     for c in (again, sen):
         assert ctx.L.sfoc_cube_free(c) == 0
     assert ctx.L.cudaFree(held) == 0
+
+
+def test_pair_cubes_of_changing_shapes_do_not_pile_up(lib):
+    """fastncc_register_pair keeps one pair of cubes: those a change of shape or type
+    replaces are freed, but for cubes that a captured graph may read, which live
+    as long as the context."""
+    shapes = [((300, 280), (310, 290)), ((500, 400), (300, 280)), ((1500, 1400), (1400, 1500))]   # joint and single builds
+    live = lib.fk_live()
+    ctx = Ctx(lib)
+    for dt in (F32, BF16, F32):
+        for ref, sen in shapes * 2:
+            ctx.ok(ctx.pair(ref, sen, p=params(ctx, dt)))
+    seen = set()
+    for _ in range(3):
+        for dt in (F32, BF16):
+            for ref, sen in shapes:
+                ctx.ok(ctx.pair(ref, sen, p=params(ctx, dt)))
+                seen.add((dt, ref, lib.fk_bytes()))
+    assert len(seen) == 2 * len(shapes)          # the same memory in use each time a shape comes back
+    ref, sen = shapes[0]
+    ctx.ok(ctx.pair(ref, sen))
+    lib.fk_capturing(1)
+    ctx.ok(ctx.pair(ref, sen))                   # into a graph: these cubes stay
+    lib.fk_capturing(0)
+    held = lib.fk_live()
+    ctx.ok(ctx.pair(*shapes[1]))
+    ctx.ok(ctx.pair(ref, sen))
+    ctx.ok(ctx.pair(*shapes[1]))
+    assert lib.fk_live() > held
+    ctx.close()
+    assert lib.fk_live() == live
