@@ -502,7 +502,7 @@ constexpr size_t kPairPixels = (size_t)1 << 21;
 // Both cubes of a small pair together (*done), into the context's pair cubes.
 // Whatever is not plain (a null pointer, a shape or parameter that is refused,
 // parameters without the streaming kernels, a workspace that may not grow
-// inside a capture) is left to the two single builds, which report it.
+// inside a capture or finds no room) is left to the two single builds, which report it.
 sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, const float* d_sen, int Hs, int Ws,
                              const sfoc_params* pin, bool* done) {
     *done = false;
@@ -531,8 +531,7 @@ sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, 
     const bool grows = at[2] > ctx->ws_bytes;
     if (grows && std::max(at[1], at[2] - at[1]) <= ctx->ws_bytes) return SFOC_OK;
     if ((grows || !fits[0] || !fits[1]) && capturing(ctx->stream)) return SFOC_OK;
-    sfoc_status s = ensure_ws(ctx, at[2]);
-    if (s != SFOC_OK) return s;
+    sfoc_status s = SFOC_OK;
     for (int k = 0; k < 2; ++k) {
         sfoc_cube* c = *cube[k];
         if (!fits[k]) {
@@ -546,6 +545,9 @@ sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, 
         }
         set_pair_cube(ctx, cube[k], c);
     }
+    s = ensure_ws(ctx, at[2]);
+    if (s == SFOC_ERR_OOM) return SFOC_OK;  // one image's workspace may still fit
+    if (s != SFOC_OK) return s;
     ImgJob two[2];
     memset(two, 0, sizeof(two));
     for (int k = 0; k < 2; ++k) {

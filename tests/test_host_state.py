@@ -163,3 +163,20 @@ def test_pair_cubes_of_changing_shapes_do_not_pile_up(lib):
     assert lib.fk_live() > held
     ctx.close()
     assert lib.fk_live() == live
+
+
+def test_a_pair_whose_joint_workspace_does_not_fit_is_built_one_by_one(ctx):
+    """Both cubes of a small pair are built together with a workspace for two; where
+    the device has no room for that, the two builds of one workspace still run."""
+    H, W = 512, 480
+    one = 4 * 12 * 480 * H
+    room = 2 * (4 * 480 * H * 14 + 16 * (H + 1) * (W + 1)) + one + (3 << 20)   # two cubes, one workspace
+    ctx.L.fk_limit(C.c_size_t(ctx.L.fk_bytes() + room))
+    ctx.L.fk_reset()
+    ctx.ok(ctx.pair((H, W), (H, W)))
+    assert (ctx.L.fk_count(b"two"), ctx.L.fk_count(b"steer")) == (0, 2)
+    ctx.L.fk_limit(C.c_size_t(-1).value)
+    again = Ctx(ctx.L)
+    again.ok(again.pair((H, W), (H, W)))
+    assert (ctx.L.fk_count(b"two"), ctx.L.fk_count(b"steer")) == (1, 0)
+    again.close()
