@@ -145,7 +145,9 @@ bool sfoc_batch_supported(const SteerTaps& st, const SmoothTaps& sm);
 void sfoc_batch_tiles(int H, int W, int* steer_ctas, int* smooth_ctas);
 // Two float images in one launch per kernel (both within the batched forms'
 // parameters): small images leave most of the chip idle one after the other.
-cudaError_t launch_sfoc_two(const ImgJob* two, const SteerTaps& st, const SmoothTaps& sm, cudaStream_t s);
+// The steering is one launch, the smoothing smooth_launch_count.
+cudaError_t launch_steer_two(const ImgJob* two, const SteerTaps& st, cudaStream_t s);
+cudaError_t launch_smooth_two(const ImgJob* two, const SmoothTaps& sm, cudaStream_t s);
 cudaError_t launch_sfoc_batch(const ImgJob* jobs, int n_jobs, const int* steer_begin, int steer_ctas,
                               const int* smooth_begin, int smooth_ctas, const SteerTaps& st, const SmoothTaps& sm,
                               cudaStream_t s);

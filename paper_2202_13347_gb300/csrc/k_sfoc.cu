@@ -1051,19 +1051,26 @@ void sfoc_batch_tiles(int H, int W, int* n_steer, int* smooth_ctas) {
     *smooth_ctas = ((W + kStW - 1) / kStW) * ((H + rows - 1) / rows);
 }
 
-cudaError_t launch_sfoc_two(const ImgJob* two, const SteerTaps& st, const SmoothTaps& sm, cudaStream_t s) {
-    if (!sfoc_batch_supported(st, sm)) return cudaErrorNotSupported;
+cudaError_t launch_steer_two(const ImgJob* two, const SteerTaps& st, cudaStream_t s) {
+    if (!steer_is_paper(st)) return cudaErrorNotSupported;
     ImgPair p;
     p.j[0] = two[0];
     p.j[1] = two[1];
-    const int sr = steer_rows_for(two, 2), mr = strip_rows_for(two, 2);
-    p.split = steer_ctas(two[0].H, two[0].W, sr);
-    k_sfoc_steer_strip<float><<<p.split + steer_ctas(two[1].H, two[1].W, sr), kSrThreads, 0, s>>>(p, nullptr, nullptr,
-                                                                                                 0, st, sr);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    p.split = smooth_ctas_for(two[0], mr);
-    return launch_smooth_paper(p, nullptr, nullptr, 0, p.split + smooth_ctas_for(two[1], mr), mr, sm, s);
+    const int rows = steer_rows_for(two, 2);
+    p.split = steer_ctas(two[0].H, two[0].W, rows);
+    k_sfoc_steer_strip<float><<<p.split + steer_ctas(two[1].H, two[1].W, rows), kSrThreads, 0, s>>>(
+        p, nullptr, nullptr, 0, st, rows);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_smooth_two(const ImgJob* two, const SmoothTaps& sm, cudaStream_t s) {
+    if (!smooth_is_paper(sm)) return cudaErrorNotSupported;
+    ImgPair p;
+    p.j[0] = two[0];
+    p.j[1] = two[1];
+    const int rows = strip_rows_for(two, 2);
+    p.split = smooth_ctas_for(two[0], rows);
+    return launch_smooth_paper(p, nullptr, nullptr, 0, p.split + smooth_ctas_for(two[1], rows), rows, sm, s);
 }
 
 cudaError_t launch_sfoc_batch(const ImgJob* jobs, int n_jobs, const int* steer_begin, int steer_ctas,

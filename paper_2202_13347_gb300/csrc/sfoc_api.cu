@@ -569,8 +569,12 @@ sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, 
     }
     cudaError_t e;
     {
-        StageScope sc(ctx, ST_SMOOTH, 3);
-        e = launch_sfoc_two(two, st, sm, ctx->stream);
+        StageScope sc(ctx, ST_STEER, 1);
+        e = launch_steer_two(two, st, ctx->stream);
+    }
+    if (e == cudaSuccess) {
+        StageScope sc(ctx, ST_SMOOTH, smooth_launch_count(sm));
+        e = launch_smooth_two(two, sm, ctx->stream);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "sfoc kernels");
     *done = true;
@@ -1016,9 +1020,9 @@ sfoc_status fastncc_register_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int
                                   const sfoc_params* p, const fastncc_opts* opts, fastncc_result* d_out) {
     if (!ctx) return SFOC_ERR_INVALID_ARG;
     bool both = false;
-    sfoc_status s = ctx->timing ? SFOC_OK : build_small_pair(ctx, d_ref, Hr, Wr, d_sen, Hs, Ws, p, &both);
+    sfoc_status s = build_small_pair(ctx, d_ref, Hr, Wr, d_sen, Hs, Ws, p, &both);
     if (s != SFOC_OK) return s;
-    if (!both) {  // (per-stage timing keeps the steering and smoothing launches apart)
+    if (!both) {
         s = build_pair_cube(ctx, d_ref, Hr, Wr, p, &ctx->pair_ref);
         if (s != SFOC_OK) return s;
         s = build_pair_cube(ctx, d_sen, Hs, Ws, p, &ctx->pair_sen);

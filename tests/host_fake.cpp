@@ -152,7 +152,8 @@ cudaError_t launch_sfoc_batch(const ImgJob*, int, const int*, int, const int*, i
                               cudaStream_t) {
     return count("build_batch");
 }
-cudaError_t launch_sfoc_two(const ImgJob*, const SteerTaps&, const SmoothTaps&, cudaStream_t) { return count("two"); }
+cudaError_t launch_steer_two(const ImgJob*, const SteerTaps&, cudaStream_t) { return count("steer_two"); }
+cudaError_t launch_smooth_two(const ImgJob*, const SmoothTaps&, cudaStream_t) { return count("smooth_two"); }
 size_t integral_scratch_bytes(int, int) { return 256; }
 size_t integral_export_scratch_bytes(int, int) { return 256; }
 size_t integral_batch_scratch_bytes(const Cube* const*, int) { return 256; }

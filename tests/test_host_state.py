@@ -174,9 +174,26 @@ def test_a_pair_whose_joint_workspace_does_not_fit_is_built_one_by_one(ctx):
     ctx.L.fk_limit(C.c_size_t(ctx.L.fk_bytes() + room))
     ctx.L.fk_reset()
     ctx.ok(ctx.pair((H, W), (H, W)))
-    assert (ctx.L.fk_count(b"two"), ctx.L.fk_count(b"steer")) == (0, 2)
+    assert (ctx.L.fk_count(b"steer_two"), ctx.L.fk_count(b"steer")) == (0, 2)
     ctx.L.fk_limit(C.c_size_t(-1).value)
     again = Ctx(ctx.L)
     again.ok(again.pair((H, W), (H, W)))
-    assert (ctx.L.fk_count(b"two"), ctx.L.fk_count(b"steer")) == (1, 0)
+    assert (ctx.L.fk_count(b"steer_two"), ctx.L.fk_count(b"steer")) == (1, 0)
     again.close()
+
+
+def test_stage_timing_times_the_launches_that_run_without_it(ctx):
+    """Both cubes of a small pair come from one launch per kernel, with stage timing
+    as without: one steering and two smoothing launches."""
+    shape = (512, 480)
+    for timing in (0, 1):
+        assert ctx.L.sfoc_ctx_enable_timing(ctx.h, timing) == 0
+        ctx.L.fk_reset()
+        before = ctx.launches()
+        ctx.ok(ctx.pair(shape, shape))
+        made = [ctx.L.fk_count(k) for k in (b"steer_two", b"smooth_two", b"steer", b"smooth")]
+        assert made == [1, 1, 0, 0]
+        if timing:
+            ms, n = (C.c_double * 7)(), (C.c_int64 * 7)()
+            assert ctx.L.sfoc_ctx_stage_times(ctx.h, ms, n) == 0
+            assert list(n)[:2] == [1, 2] and sum(n) == ctx.launches() - before
