@@ -446,8 +446,11 @@ SFOC_API sfoc_status sfoc_ctx_plan_info(const sfoc_ctx* ctx, char* buf, size_t c
  * correlation form of a (cube dtype, m, R) is measured, not ruled: on the
  * first match of that key (outside a stream capture) every form of the
  * family that runs for it is launched on the first min(n, 4 x SMs) points
- * of that call (one warm-up launch, then the better of two timed with CUDA
- * events), and the fastest is kept in the context and used from then on.
+ * of that call (the better of two timed with CUDA events) and, where that is
+ * more than a point per SM, on one point per SM.  The fastest on the sample is
+ * kept in the context and used from then on; calls of another number of points
+ * per SM (1 to 4, more as 4) than the sample's take the form that the two times
+ * give for it, since the forms differ in how many points an SM works on at a time.
  *   family 0, F32 cubes:  the Fourier correlation (sides 64 and 128; where
  *                         m + 2R is in (64, 96] also 96, in (128, 224] also
  *                         160, 192 or 224, the least that holds it; where
@@ -468,7 +471,7 @@ SFOC_API sfoc_status sfoc_ctx_set_autotune(sfoc_ctx* ctx, int enable);
 /* The entry of (dtype, m, R): *corr_path = the chosen sfoc_corr_path (-1 when
  * there is none), *option = its FFT side (else 0), and per candidate timed
  * (*n_cand <= 6) its path, option and milliseconds (-1 = it failed to run);
- * *sample = the points timed.  Output pointers other than corr_path may be
+ * *sample = the points timed (the choice is that for as many points).  Output pointers other than corr_path may be
  * NULL. */
 SFOC_API sfoc_status sfoc_ctx_autotune_entry(const sfoc_ctx* ctx, int dtype, int m, int R, int family,
                                              int* corr_path, int* option, int* n_cand, int* cand_path,

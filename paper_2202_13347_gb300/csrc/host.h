@@ -26,9 +26,14 @@ struct TuneKey {
         return R < o.R;
     }
 };
+constexpr int kTuneWaves = 4;  // points per SM of the largest sample
 struct TuneEntry {
     int path;        // sfoc_corr_path of the winner (a concrete form, never AUTO or IGEMM_TC)
     int option;      // FFT: transform side; otherwise 0
+    // the form for calls of up to (w + 1) points per SM, the last for more
+    struct Form {
+        int path, option;
+    } wave[kTuneWaves];
     int n_cand;      // candidates timed
     int cand_path[6];
     int cand_option[6];
@@ -158,7 +163,8 @@ int auto_rule(int dtype, int m, int R, int family);
 const TuneEntry* autotune_pair(sfoc_ctx* ctx, int dtype, int family, MatchJob one);
 // The concrete form for a match with corr_path `path` (AUTO, IGEMM_TC or a
 // concrete one): the tuned entry, measured now when allowed, else the rule.
-// *option receives the FFT side (0 otherwise); -1 when no form runs.
+// *option receives the FFT side (0 otherwise); -1 when no form runs.  The same
+// entry gives calls of few points and of many different forms (one->n).
 int resolve_path(sfoc_ctx* ctx, int path, int dtype, const MatchJob* one, bool may_measure, int* option);
 // whether a concrete path computes the zero-mean numerator of Eq. 9
 inline bool centered_path(int path) { return path == SFOC_CORR_DIRECT_F32 || path == SFOC_CORR_FFT; }

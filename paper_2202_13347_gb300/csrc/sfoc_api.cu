@@ -318,6 +318,29 @@ int auto_rule(int dtype, int m, int R, int family) {
     return corr_fft2_side(m, R) ? SFOC_CORR_FFT : SFOC_CORR_DIRECT_F32;
 }
 
+// points per SM of a call, 1 .. kTuneWaves
+static int tune_waves(int n, int sms) {
+    const int w = (n + sms - 1) / sms;
+    return w < 1 ? 1 : w > kTuneWaves ? kTuneWaves : w;
+}
+
+// A candidate's time for w points per SM from its times for one (t1) and for
+// K > 1 (tK).  Most forms run one CTA per SM and take as much longer for every
+// further point; two of the Fourier sides run two points together on an SM, side
+// 96 four, with 0.25, 0.7 and 1 of the fourth's extra time for the second to
+// fourth (m = 41, R = 25: 123, 155, 215 and 253 us; BF16 cubes 145, 182, 248, 290).
+static double tune_predict(int path, int option, double t1, double tK, int K, int w) {
+    if (path == SFOC_CORR_FFT && (option == 64 || option == 160)) {
+        const double t2 = K == 2 ? tK : K == 3 ? tK - t1 : tK / 2;
+        return (w / 2) * t2 + (w % 2) * t1;
+    }
+    if (path == SFOC_CORR_FFT && option == 96) {
+        static const double extra[kTuneWaves] = {0.0, 0.25, 0.7, 1.0};
+        return t1 + extra[w - 1] / extra[K - 1] * (tK - t1);
+    }
+    return t1 + (w - 1) * (tK - t1) / (K - 1);
+}
+
 const TuneEntry* autotune_pair(sfoc_ctx* ctx, int dtype, int family, MatchJob one) {
     const int m = one.m, R = one.R;
     TuneEntry t;
@@ -343,29 +366,46 @@ const TuneEntry* autotune_pair(sfoc_ctx* ctx, int dtype, int family, MatchJob on
     if (family == 0 && dtype == SFOC_DTYPE_F32 && corr_f32_supported(m, R)) add(SFOC_CORR_DIRECT_F32, 0);
     if (t.n_cand == 0) return nullptr;
     // a sample of up to four points per SM (the Fourier form of side 96 runs four
-    // CTAs on one), timed per candidate: one
-    // warm-up launch, then the better of two
+    // CTAs on one), timed per candidate: the better of two, after one launch for a
+    // point per SM, timed too (after a warm-up): the forms differ in how many points
+    // an SM works on at a time, so the fastest for many points may not be the one
+    // for few (m = 41, R = 25 of F32 cubes: side 96 takes 162 us for 100 points and
+    // 307 for 608, side 128 117 and 422)
     const int sms = sm_count(ctx->device);
-    one.n = one.n < 4 * sms ? one.n : 4 * sms;
+    one.n = one.n < kTuneWaves * sms ? one.n : kTuneWaves * sms;
     t.sample = one.n;
-    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+    const int K = tune_waves(one.n, sms);
+    MatchJob few = one;
+    if (K > 1) few.n = sms;
+    float t1[6];
+    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+    bool events = true;
     for (auto& e : ev)
-        if (cudaEventCreate(&e) != cudaSuccess) e = nullptr;
+        if (cudaEventCreate(&e) != cudaSuccess) {
+            e = nullptr;
+            events = false;
+        }
     int best = -1;
     for (int c = 0; c < t.n_cand; ++c) {
-        t.cand_ms[c] = -1.f;
-        if (!ev[0] || !ev[1] || !ev[2]) continue;
-        bool ok = launch_corr_path(ctx, t.cand_path[c], t.cand_option[c], one) == cudaSuccess;
+        t.cand_ms[c] = t1[c] = -1.f;
+        if (!events) continue;
+        auto run = [&](MatchJob& j) {
+            ++ctx->launches;
+            return launch_corr_path(ctx, t.cand_path[c], t.cand_option[c], j) == cudaSuccess;
+        };
+        bool ok = run(few);
         ok = ok && cudaEventRecord(ev[0], ctx->stream) == cudaSuccess;
-        ok = ok && launch_corr_path(ctx, t.cand_path[c], t.cand_option[c], one) == cudaSuccess;
+        if (K > 1) ok = ok && run(few);
         ok = ok && cudaEventRecord(ev[1], ctx->stream) == cudaSuccess;
-        ok = ok && launch_corr_path(ctx, t.cand_path[c], t.cand_option[c], one) == cudaSuccess;
+        ok = ok && run(one);
         ok = ok && cudaEventRecord(ev[2], ctx->stream) == cudaSuccess;
-        ok = ok && cudaEventSynchronize(ev[2]) == cudaSuccess;
-        ctx->launches += 3;
+        ok = ok && run(one);
+        ok = ok && cudaEventRecord(ev[3], ctx->stream) == cudaSuccess;
+        ok = ok && cudaEventSynchronize(ev[3]) == cudaSuccess;
         float a = 0.f, b = 0.f;
-        if (ok && cudaEventElapsedTime(&a, ev[0], ev[1]) == cudaSuccess &&
-            cudaEventElapsedTime(&b, ev[1], ev[2]) == cudaSuccess) {
+        if (ok && cudaEventElapsedTime(&t1[c], ev[0], ev[1]) == cudaSuccess &&
+            cudaEventElapsedTime(&a, ev[1], ev[2]) == cudaSuccess &&
+            cudaEventElapsedTime(&b, ev[2], ev[3]) == cudaSuccess) {
             t.cand_ms[c] = a < b ? a : b;
             if (best < 0 || t.cand_ms[c] < t.cand_ms[best]) best = c;
         } else {
@@ -377,6 +417,22 @@ const TuneEntry* autotune_pair(sfoc_ctx* ctx, int dtype, int family, MatchJob on
     if (best < 0) return nullptr;
     t.path = t.cand_path[best];
     t.option = t.cand_option[best];
+    for (int w = 1; w <= kTuneWaves; ++w) {
+        int pick = best;  // of the sample's own size, or where only that is known
+        if (K > 1 && w != K) {
+            double least = 0.0;
+            pick = -1;
+            for (int c = 0; c < t.n_cand; ++c) {
+                if (t.cand_ms[c] < 0.f) continue;
+                const double ms = tune_predict(t.cand_path[c], t.cand_option[c], t1[c], t.cand_ms[c], K, w);
+                if (pick < 0 || ms < least) {
+                    pick = c;
+                    least = ms;
+                }
+            }
+        }
+        t.wave[w - 1] = {t.cand_path[pick], t.cand_option[pick]};
+    }
     auto& slot = ctx->tune[TuneKey{dtype, m, R, family}];
     slot = t;
     return &slot;
@@ -392,8 +448,9 @@ int resolve_path(sfoc_ctx* ctx, int path, int dtype, const MatchJob* one, bool m
     const TuneEntry* te = it != ctx->tune.end() ? &it->second : nullptr;
     if (!te && may_measure && ctx->autotune && !capturing(ctx->stream)) te = autotune_pair(ctx, dtype, family, *one);
     if (te) {
-        *option = te->option;
-        return te->path;
+        const TuneEntry::Form& f = te->wave[tune_waves(one->n, sm_count(ctx->device)) - 1];
+        *option = f.option;
+        return f.path;
     }
     const int rule = auto_rule(dtype, m, R, family);
     if (rule == SFOC_CORR_FFT && !corr_fft_supported(m, R)) *option = corr_fft2_side(m, R);
@@ -1140,9 +1197,14 @@ sfoc_status sfoc_ctx_autotune_export(const sfoc_ctx* ctx, char* buf, size_t cap,
     for (const auto& kv : ctx->tune) {
         const TuneEntry& t = kv.second;
         snprintf(tmp, sizeof(tmp), "%s{\"dtype\": %d, \"family\": %d, \"m\": %d, \"R\": %d, \"path\": %d, "
-                 "\"option\": %d, \"sample\": %d, \"candidates\": [", first ? "" : ", ", kv.first.dtype,
+                 "\"option\": %d, \"sample\": %d, \"waves\": [", first ? "" : ", ", kv.first.dtype,
                  kv.first.family, kv.first.m, kv.first.R, t.path, t.option, t.sample);
         j += tmp;
+        for (int w = 0; w < kTuneWaves; ++w) {
+            snprintf(tmp, sizeof(tmp), "%s%d, %d", w ? ", " : "", t.wave[w].path, t.wave[w].option);
+            j += tmp;
+        }
+        j += "], \"candidates\": [";
         for (int i = 0; i < t.n_cand; ++i) {
             snprintf(tmp, sizeof(tmp), "%s[%d, %d, %.6g]", i ? ", " : "", t.cand_path[i], t.cand_option[i],
                      (double)t.cand_ms[i]);
@@ -1175,6 +1237,24 @@ bool json_int(const char* p, const char* end, const char* key, int* out) {
     return true;
 }
 
+// the n integers of `"key": [...]` inside [p, end); false when the key is absent
+// or holds something else
+bool json_ints(const char* p, const char* end, const char* key, int n, int* out) {
+    std::string k = std::string("\"") + key + "\"";
+    const char* q = std::search(p, end, k.begin(), k.end());
+    if (q == end) return false;
+    q += k.size();
+    for (int i = 0; i < n; ++i) {
+        while (q < end && (*q == ' ' || *q == ':' || *q == '[' || *q == ',')) ++q;
+        char* e = nullptr;
+        const long v = strtol(q, &e, 10);
+        if (e == q) return false;
+        out[i] = (int)v;
+        q = e;
+    }
+    return true;
+}
+
 }  // namespace
 
 sfoc_status sfoc_ctx_autotune_import(sfoc_ctx* ctx, const char* text) {
@@ -1195,23 +1275,33 @@ sfoc_status sfoc_ctx_autotune_import(sfoc_ctx* ctx, const char* text) {
             return fail(ctx, SFOC_ERR_INVALID_ARG, "autotune entry without dtype, m, R, path or option");
         json_int(p, end, "sample", &t.sample);
         json_int(p, end, "family", &family);
-        const bool ok_path = t.path == SFOC_CORR_DIRECT_F32 || t.path == SFOC_CORR_FFT || t.path == SFOC_CORR_TC_TOEPLITZ ||
-                             t.path == SFOC_CORR_TC_COLUMN || t.path == SFOC_CORR_TC_BAND;
-        if (!ok_path || (dtype != SFOC_DTYPE_F32 && dtype != SFOC_DTYPE_BF16) || !path_serves(t.path, dtype) ||
-            (family != 0 && family != 1) || (family == 1 && (dtype != SFOC_DTYPE_BF16 || centered_path(t.path))) ||
-            m < 1 || m > kMaxTemplate || R < 0 || R > kMaxRadius)
-            return fail(ctx, SFOC_ERR_INVALID_ARG, "autotune entry out of range");
-        const int opt = t.path == SFOC_CORR_FFT ? t.option : 0;
-        const bool half = t.path == SFOC_CORR_FFT && opt && opt == corr_fft2_side(m, R);
-        if (t.path == SFOC_CORR_FFT && !half && opt != 64 && opt != 128)
-            return fail(ctx, SFOC_ERR_INVALID_ARG, "bad FFT side");
-        // the entry must name a form that runs for (m, R)
-        if (half ? auto_rule(dtype, m, R, 0) < 0
-            : t.path == SFOC_CORR_FFT ? (!corr_fft_supported(m, R) || m + 2 * R > opt)
-            : t.path == SFOC_CORR_DIRECT_F32 ? !corr_f32_supported(m, R)
-                                             : corr_tc_class(t.path == SFOC_CORR_TC_TOEPLITZ ? 1
-                                                             : t.path == SFOC_CORR_TC_COLUMN ? 2 : 3, m, R) == 0)
-            return fail(ctx, SFOC_ERR_INVALID_ARG, "autotune entry names a form that does not run for its m / R");
+        // the form for each number of points: one for all where the text (of an
+        // earlier version, say) has no more
+        for (auto& f : t.wave) f = {t.path, t.option};
+        int waves[2 * kTuneWaves];
+        if (json_ints(p, end, "waves", 2 * kTuneWaves, waves))
+            for (int w = 0; w < kTuneWaves; ++w) t.wave[w] = {waves[2 * w], waves[2 * w + 1]};
+        for (int w = -1; w < kTuneWaves; ++w) {
+            const TuneEntry::Form f = w < 0 ? TuneEntry::Form{t.path, t.option} : t.wave[w];
+            const bool ok_path = f.path == SFOC_CORR_DIRECT_F32 || f.path == SFOC_CORR_FFT ||
+                                 f.path == SFOC_CORR_TC_TOEPLITZ || f.path == SFOC_CORR_TC_COLUMN ||
+                                 f.path == SFOC_CORR_TC_BAND;
+            if (!ok_path || (dtype != SFOC_DTYPE_F32 && dtype != SFOC_DTYPE_BF16) || !path_serves(f.path, dtype) ||
+                (family != 0 && family != 1) || (family == 1 && (dtype != SFOC_DTYPE_BF16 || centered_path(f.path))) ||
+                m < 1 || m > kMaxTemplate || R < 0 || R > kMaxRadius)
+                return fail(ctx, SFOC_ERR_INVALID_ARG, "autotune entry out of range");
+            const int opt = f.path == SFOC_CORR_FFT ? f.option : 0;
+            const bool half = f.path == SFOC_CORR_FFT && opt && opt == corr_fft2_side(m, R);
+            if (f.path == SFOC_CORR_FFT && !half && opt != 64 && opt != 128)
+                return fail(ctx, SFOC_ERR_INVALID_ARG, "bad FFT side");
+            // the entry must name a form that runs for (m, R)
+            if (half ? auto_rule(dtype, m, R, 0) < 0
+                : f.path == SFOC_CORR_FFT ? (!corr_fft_supported(m, R) || m + 2 * R > opt)
+                : f.path == SFOC_CORR_DIRECT_F32 ? !corr_f32_supported(m, R)
+                                                 : corr_tc_class(f.path == SFOC_CORR_TC_TOEPLITZ ? 1
+                                                                 : f.path == SFOC_CORR_TC_COLUMN ? 2 : 3, m, R) == 0)
+                return fail(ctx, SFOC_ERR_INVALID_ARG, "autotune entry names a form that does not run for its m / R");
+        }
         got[TuneKey{dtype, m, R, family}] = t;
         p = end + 2;
     }

@@ -197,3 +197,57 @@ def test_stage_timing_times_the_launches_that_run_without_it(ctx):
             ms, n = (C.c_double * 7)(), (C.c_int64 * 7)()
             assert ctx.L.sfoc_ctx_stage_times(ctx.h, ms, n) == 0
             assert list(n)[:2] == [1, 2] and sum(n) == ctx.launches() - before
+
+
+# milliseconds of a form for 1 .. period points per SM (fk_cost; more points repeat the period), after
+# measurements: one CTA per SM, four (side 96), two (side 160)
+COSTS = {"f32_96": {(FFT, 128): {1: 0.088}, (FFT, 96): {1: 0.123, 2: 0.155, 3: 0.215, 4: 0.253}, (DIRECT, 0): {1: 5.0}},
+         "bf16_96": {(BAND, 0): {1: 0.080}, (FFT, 128): {1: 0.100}, (FFT, 96): {1: 0.145, 2: 0.182, 3: 0.248, 4: 0.290}},
+         "bf16_160": {(BAND, 0): {1: 0.196}, (FFT, 160): {1: 0.288, 2: 0.380}}}
+
+
+@pytest.mark.parametrize("case,dtype,m,R", [("f32_96", F32, 41, 25), ("bf16_96", BF16, 41, 25), ("bf16_160", BF16, 81, 30)])
+@pytest.mark.parametrize("first", [100, 304, 456, 2000])
+def test_few_points_and_many_take_the_form_that_is_faster_for_them(lib, case, dtype, m, R, first):
+    """One measurement per (dtype, m, R), on the first call's points, serves calls of any
+    number of points: none takes a form that is over 10 % slower than the best for
+    it (a first call of up to a point per SM knows only that and keeps its choice)."""
+    ctx = Ctx(lib)
+    forms = COSTS[case]
+    for (path, side), by_waves in forms.items():
+        for w, ms in by_waves.items():
+            lib.fk_cost(1000 * path + side, w, ms)
+
+    def cost(path, side, n):
+        by, k = forms[path, side], (n + 151) // 152
+        period = max(by)
+        return k // period * by[period] + (by[k % period] if k % period else 0.0)
+
+    cubes = [ctx.build(700, 700, params(ctx, dtype)) for _ in range(2)]
+    other = Ctx(lib)
+    ctx.match(*cubes, first, m, R)
+    counted = ctx.launches()
+    n = C.c_size_t()
+    ctx.ok(lib.sfoc_ctx_autotune_export(ctx.h, None, 0, C.byref(n)))
+    text = C.create_string_buffer(n.value)
+    ctx.ok(lib.sfoc_ctx_autotune_export(ctx.h, text, n, C.byref(n)))
+    other.ok(lib.sfoc_ctx_autotune_import(other.h, text))
+    for points in (1, 100, 152, 153, 304, 400, 456, 608, 1216, 5000):
+        form = ctx.match(*cubes, points, m, R)
+        assert other.match(*cubes, points, m, R) == form        # and after a round trip through the text
+        if first > 152 or points <= 152:
+            best = min(cost(p, s, points) for p, s in forms)
+            assert cost(*divmod(form, 1000), points) <= 1.1 * best, (points, form)
+    assert ctx.launches() - counted < 10 * 8                   # nothing is measured again
+    # text without the numbers of points: its form for every call
+    path, side = list(forms)[-1]
+    plain = ('{"entries": [{"dtype": %d, "family": 0, "m": %d, "R": %d, "path": %d, "option": %d, "sample": 1, '
+             '"candidates": []}]}' % (dtype, m, R, path, side)).encode()
+    ctx.ok(lib.sfoc_ctx_autotune_import(ctx.h, plain))
+    assert {ctx.match(*cubes, k, m, R) for k in (1, 500, 5000)} == {1000 * path + side}
+    bad = plain.replace(b'"candidates"', b'"waves": [%d, %d, 7, 0, 6, 64, 6, 64], "candidates"' % (path, side))
+    assert lib.sfoc_ctx_autotune_import(ctx.h, bad) != 0
+    for c in cubes:
+        assert lib.sfoc_cube_free(c) == 0
+    other.close()
+    ctx.close()
