@@ -53,6 +53,43 @@ __device__ __forceinline__ bool better(float s, int y, int x, float bs, int by, 
     return y < by || (y == by && x < bx);
 }
 
+// the score of the pixel at staged position (iy, ix), 0 where it is no corner
+__device__ __forceinline__ float fast_score(const float (*s_img)[kIn + 1], int iy, int ix, float t) {
+    const float c = s_img[iy][ix];
+    float d[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) d[k] = s_img[iy + cdy(k)][ix + cdx(k)] - c;
+    // smallest and largest difference over every arc of 9 (cyclic),
+    // by doubling: windows of 2, 4, 8, then one more pixel
+    float lo[16], hi[16], l2[16], h2[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        lo[k] = fminf(d[k], d[(k + 1) & 15]);
+        hi[k] = fmaxf(d[k], d[(k + 1) & 15]);
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        l2[k] = fminf(lo[k], lo[(k + 2) & 15]);
+        h2[k] = fmaxf(hi[k], hi[(k + 2) & 15]);
+    }
+    float bright = -INFINITY, dark = INFINITY;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float mn = fminf(fminf(l2[k], l2[(k + 4) & 15]), d[(k + 8) & 15]);
+        const float mx = fmaxf(fmaxf(h2[k], h2[(k + 4) & 15]), d[(k + 8) & 15]);
+        bright = fmaxf(bright, mn);   // brighter arc: its smallest rise
+        dark = fminf(dark, mx);       // darker arc: minus its smallest drop
+    }
+    const float best = fmaxf(bright, -dark);
+    return best > t ? best : 0.f;
+}
+
+// QUICK: the quick test first.  Without it (a threshold of 0, which turns away
+// nothing but flat pixels) every pixel is scored and the corners are listed: 2048 x
+// 2048 texture, threshold 0, blocks of 512 x 512 1163 us with the test, 1010 without,
+// of 64 x 64 77 and 67.  (Scoring at once the pixels of a warp that passes mostly,
+// or a sub-tile after one that did, made the usual thresholds 3 to 15 % slower.)
+template <bool QUICK>
 __global__ void __launch_bounds__(kFastThreads)
     k_fast_blocks(const float* __restrict__ img, int H, int W, size_t pitch, float t, int grid_y, int grid_x,
                   int margin, int32_t* __restrict__ points, float* __restrict__ scores) {
@@ -95,7 +132,12 @@ __global__ void __launch_bounds__(kFastThreads)
                 int ly = threadIdx.x / nsx, lx = threadIdx.x - ly * nsx;
                 while (ly < nsy) {
                     const int gy = sy0 - 1 + ly, gx = sx0 - 1 + lx;
-                    if (gy >= 3 && gy < H - 3 && gx >= 3 && gx < W - 3) {
+                    if (!QUICK) {
+                        float sc = 0.f;
+                        if (gy >= 3 && gy < H - 3 && gx >= 3 && gx < W - 3) sc = fast_score(s_img, ly + 3, lx + 3, t);
+                        if (sc > 0.f) s_list[atomicAdd(&s_n, 1)] = (unsigned short)(ly * kSc + lx);
+                        s_sc[ly][lx] = sc;
+                    } else if (gy >= 3 && gy < H - 3 && gx >= 3 && gx < W - 3) {
                         const int iy = ly + 3, ix = lx + 3;
                         const float c = s_img[iy][ix];
                         bool bright = true, dark = true;
@@ -109,7 +151,7 @@ __global__ void __launch_bounds__(kFastThreads)
                         }
                         if (bright || dark) s_list[atomicAdd(&s_n, 1)] = (unsigned short)(ly * kSc + lx);
                     }
-                    s_sc[ly][lx] = 0.f;
+                    if (QUICK) s_sc[ly][lx] = 0.f;
                     ly += dq;
                     lx += dr;
                     if (lx >= nsx) {
@@ -120,36 +162,10 @@ __global__ void __launch_bounds__(kFastThreads)
             }
             __syncthreads();
             const int nl = s_n;
-            for (int i = threadIdx.x; i < nl; i += kFastThreads) {
+            for (int i = threadIdx.x; i < (QUICK ? nl : 0); i += kFastThreads) {
                 const int ly = s_list[i] / kSc, lx = s_list[i] - ly * kSc;
                 const int iy = ly + 3, ix = lx + 3;  // staged position
-                const float c = s_img[iy][ix];
-                float d[16];
-#pragma unroll
-                for (int k = 0; k < 16; ++k) d[k] = s_img[iy + cdy(k)][ix + cdx(k)] - c;
-                // smallest and largest difference over every arc of 9 (cyclic),
-                // by doubling: windows of 2, 4, 8, then one more pixel
-                float lo[16], hi[16], l2[16], h2[16];
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    lo[k] = fminf(d[k], d[(k + 1) & 15]);
-                    hi[k] = fmaxf(d[k], d[(k + 1) & 15]);
-                }
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    l2[k] = fminf(lo[k], lo[(k + 2) & 15]);
-                    h2[k] = fmaxf(hi[k], hi[(k + 2) & 15]);
-                }
-                float bright = -INFINITY, dark = INFINITY;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const float mn = fminf(fminf(l2[k], l2[(k + 4) & 15]), d[(k + 8) & 15]);
-                    const float mx = fmaxf(fmaxf(h2[k], h2[(k + 4) & 15]), d[(k + 8) & 15]);
-                    bright = fmaxf(bright, mn);   // brighter arc: its smallest rise
-                    dark = fminf(dark, mx);       // darker arc: minus its smallest drop
-                }
-                const float best = fmaxf(bright, -dark);
-                s_sc[ly][lx] = best > t ? best : 0.f;
+                s_sc[ly][lx] = fast_score(s_img, iy, ix, t);
             }
             __syncthreads();
             for (int i = threadIdx.x; i < nl; i += kFastThreads) {
@@ -211,7 +227,10 @@ __global__ void __launch_bounds__(kFastThreads)
 cudaError_t launch_fast_blocks(const float* img, int H, int W, size_t pitch, float t, int grid_y, int grid_x,
                                int margin, int32_t* points, float* scores, cudaStream_t st) {
     dim3 grid((unsigned)grid_x, (unsigned)grid_y);
-    k_fast_blocks<<<grid, kFastThreads, 0, st>>>(img, H, W, pitch, t, grid_y, grid_x, margin, points, scores);
+    if (t > 0.f)
+        k_fast_blocks<true><<<grid, kFastThreads, 0, st>>>(img, H, W, pitch, t, grid_y, grid_x, margin, points, scores);
+    else
+        k_fast_blocks<false><<<grid, kFastThreads, 0, st>>>(img, H, W, pitch, t, grid_y, grid_x, margin, points, scores);
     return cudaGetLastError();
 }
 
