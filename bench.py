@@ -82,6 +82,9 @@ def parse():
     ap.add_argument("--scale", type=float, default=1.0, help="mixed64: side and point-count scale (1 = full size)")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--detail", default=None, metavar="FILE",
+                    help="mixed64: also writes the whole record (every correlation class, every tuned form with its "
+                         "candidates' times, the stages of every form), of which the printed line is a short form")
     ap.add_argument("--noise-sweep", action="store_true",
                     help="instead of the benchmark: CMR of the descriptor variants under the noise series of Sec. 4.3")
     return ap.parse_args()
@@ -915,6 +918,52 @@ def reference_batch(args, rank):
     print(json.dumps(line))
 
 
+def rounded(v, digits=6):
+    """A record with its floats to `digits` significant digits."""
+    if isinstance(v, float):
+        return float("%.*g" % (digits, v)) if math.isfinite(v) else v
+    if isinstance(v, dict):
+        return {k: rounded(x, digits) for k, x in v.items()}
+    return [rounded(x, digits) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def short_line(line):
+    """The batched workload's record as one line that a log's last 3 kB hold (the
+    whole record of three forms over 55 (m, R) is 22 kB): of the roofline the two
+    classes with the longest launches, of each form its value, times and
+    roofline fraction, of its tuned (m, R) how many took each path/option, of a
+    list of step times the first five."""
+    out = dict(line)
+
+    def roof(r, classes):
+        r = dict(r, classes=sorted(r["classes"], key=lambda c: -c["ms"])[:classes])
+        r["classes"] = [{k: c[k] for k in ("path", "cls", "items", "ms", "frac") if k in c} for c in r["classes"]]
+        keep = (("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "launch_ms", "classes") if classes
+                else ("kernel", "frac", "launch_ms"))
+        return {k: r[k] for k in keep}
+
+    def form(s):
+        s = {k: s[k] for k in ("value", "ms_per_step", "roofline", "autotune") if s[k] is not None}
+        s["roofline"] = roof(s["roofline"], 0)
+        if s.get("autotune"):
+            count = {}
+            for e in s["autotune"].values():
+                k = "%d/%d" % (e["path"], e["option"])
+                count[k] = count.get(k, 0) + 1
+            s["autotune"] = count
+        return s
+
+    out["roofline"] = roof(line["roofline"], 2)
+    out["forms"] = {f: form(s) for f, s in line["forms"].items()}
+    out["peaks"] = {k: v for k, v in line["peaks"].items() if k != "microbench"}
+    drop = {"e2e": ("sync_call", "plans_built_in_timed_calls"), "cpu_baseline": ("sfoc_sample",),
+            "config": ("pixels_per_rank",)}
+    for key, names in drop.items():
+        if line[key]:
+            out[key] = {k: v[:5] if isinstance(v, list) else v for k, v in line[key].items() if k not in names}
+    return {k: v for k, v in rounded(out).items() if v is not None or k in ("vs_baseline", "cpu_baseline", "e2e")}
+
+
 def main_batch(args, torch, dist, rank, world, gpu_index):
     import paper_2202_13347_gb300 as pkg
     pkg.build()
@@ -999,8 +1048,7 @@ def main_batch(args, torch, dist, rank, world, gpu_index):
         ms_max, matched_all = reduce_over_ranks(dist, torch, er["ms"], er["matched"] * er["steps"], "cuda")
         e2e = dict(value=matched_all / (ms_max * 1e-3), unit=UNIT, h2d_bytes_per_step=er["h2d_bytes_per_step"],
                    d2h_bytes_per_step=er["d2h_bytes_per_step"], ms_per_step=ms_max / er["steps"],
-                   call="fastncc_submit_batch_host + fastncc_wait_batch_host (pinned host buffers; step k+1 "
-                        "submitted before step k is waited for)",
+                   call="fastncc_submit_batch_host + wait (pinned host buffers, step k+1 submitted before step k's wait)",
                    step_done_ms=er["step_done_ms"], results_equal_across_steps=er["results_equal_across_steps"],
                    sync_call="fastncc_register_batch_host", sync_call_ms=er["sync_call_ms"],
                    h2d_gbs_alone=er["h2d_gbs_alone"], plans_built_in_timed_calls=er["plans_built_in_timed_calls"])
@@ -1036,7 +1084,11 @@ def main_batch(args, torch, dist, rank, world, gpu_index):
             "peaks": {"hbm_gbs": pk["hbm"], "bf16_tflops": pk["bf16"], "bf16_tflops_sustained": pk["bf16_sus"],
                       "src": pk["src"] + " (MEASURED_PEAKS.json)", "microbench": pk.get("microbench")},
             "errors": {f: results[f]["error"] for f in forms if "error" in results[f]} or None}
-    print(json.dumps(line))
+    if args.detail:
+        with open(args.detail, "w") as f:
+            json.dump(line, f)
+            f.write("\n")
+    print(json.dumps(short_line(line)))
 
 
 def main():
