@@ -276,18 +276,25 @@ FP32_OPS_PEAK = 152 * 128 * 2.070e9 / 1e12   # Top/s: one FP32 add / min / max p
 
 
 def fast_roofline(ms, H, W, hbm_gbs, pk=None):
-    """Block FAST against the full score at every pixel (the kernel's quick
-    test spares most pixels it), the image read once, 4 B/px: achieved =
-    FAST_OPS_PER_PX per pixel of the image over the launch time, against one FP32 op per lane per clock (half the
-    measured scalar FMA flop rate, which counts 2 flop per FMA)."""
+    """Block FAST against its two floors.  The image read once, 4 B/px: hbm_gbs
+    and hbm_frac.  The full score at every pixel: achieved = FAST_OPS_PER_PX per
+    pixel of the image over the launch time, against one FP32 op per lane per
+    clock (half the measured scalar FMA flop rate, which counts 2 flop per FMA).
+    The kernel's quick test spares most pixels the score, so that these are the
+    operations of the definition, not the ones it executes, and frac may pass
+    1; executed_floor_ops is what it executes at least, the quick test's 8
+    differences and 16 comparisons at every pixel, with its own fraction."""
     ach = FAST_OPS_PER_PX * H * W / (ms * 1e-3) / 1e12
     gbs = 4.0 * H * W / (ms * 1e-3) / 1e9
+    quick = 8 + 16
     if pk and pk.get("fp32_scalar"):
         peak, src = pk["fp32_scalar"] / 2.0, "scalar FFMA chains of sfoc_measure_peaks, one op per lane per clock"
     else:
         peak, src = FP32_OPS_PEAK, "152 SMs x 128 FP32 lanes x 2070 MHz (nominal)"
     return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "Top/s", "frac": ach / peak,
-            "work": "%d FP32 ops per pixel (FAST-9 score by windowed min / max)" % FAST_OPS_PER_PX,
+            "work": "%d FP32 ops per pixel (FAST-9 score by windowed min / max), spared most pixels by the quick test"
+                    % FAST_OPS_PER_PX,
+            "executed_floor_ops": quick, "executed_floor_frac": ach * quick / FAST_OPS_PER_PX / peak,
             "peak_src": src, "hbm_gbs": gbs, "hbm_frac": gbs / hbm_gbs}
 
 

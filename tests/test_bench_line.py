@@ -49,3 +49,12 @@ def test_the_line_is_short_and_whole():
 
 def test_the_longest_runs_still_fit():
     assert len(json.dumps(bench.short_line(record(steps=500, keys=200, classes=40)))) < 3000
+
+
+def test_fast_reports_what_the_kernel_executes_beside_the_definition():
+    """2048 x 2048 in 24.6 us: the score at every pixel, most of which the quick test
+    spares, and the quick test itself."""
+    r = bench.fast_roofline(0.0246, 2048, 2048, 6780.0)
+    assert "spared" in r["work"] and r["executed_floor_ops"] == 24
+    assert abs(r["executed_floor_frac"] * r["peak"] * 1e12 / (24 * 2048 * 2048 / 24.6e-6) - 1) < 1e-9
+    assert r["executed_floor_frac"] < r["frac"]
