@@ -27,6 +27,14 @@ constexpr int kMaxRadius = 63;
 // A separable 2-D kernel a(x) b(y) is applied as a horizontal pass with a
 // and a vertical pass with b; "odd" taps satisfy t(-q) = -t(q) and "even"
 // taps t(-q) = t(q), so only q = 0..K are stored.
+// SMs of the current device: the launchers' plans fill them
+inline int device_sms() {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 struct SteerTaps {
     int ns;                                   // first-order scales
     int K1[kMaxScales];                       // radius per scale

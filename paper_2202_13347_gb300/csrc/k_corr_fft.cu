@@ -468,9 +468,7 @@ cudaError_t launch_corr_fft(const MatchJob& one, const ItemSet& is, int L, bool 
     if (!is.items && (bf16 ? (one.rpl == nullptr || one.spl == nullptr || one.z != 12)
                            : (one.rf32 == nullptr || one.sf32 == nullptr)))
         return cudaErrorNotSupported;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sms();
     cudaError_t e;
 #define SFOC_FFT_LAUNCH(LV, BV)                                                                                   \
     {                                                                                                             \

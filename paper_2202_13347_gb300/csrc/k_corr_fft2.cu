@@ -794,9 +794,7 @@ cudaError_t launch_corr_fft2(const MatchJob& one, const ItemSet& is, int L, bool
         return cudaErrorNotSupported;
     const int lw = one.m + 2 * one.R;
     if (!is.items && (lw > L || lw <= L - 32)) return cudaErrorNotSupported;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sms();
     auto run = [&](auto kern, auto shape) -> cudaError_t {
         using Sh = decltype(shape);
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem);

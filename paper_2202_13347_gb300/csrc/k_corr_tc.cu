@@ -1030,9 +1030,7 @@ cudaError_t launch_corr_tc(int form, int cls, const MatchJob& one, const ItemSet
                            int cnt, int* err_flag, cudaStream_t st) {
     const int n = is.items ? is.n : one.n;
     if (n <= 0) return cudaSuccess;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sms();
     const int grid = n < sms ? n : sms;
     if (form == 3) return launch_corr_band(one, is, cls, ms, Rs, cnt, err_flag, sms, st);
     if (form == 2) {

@@ -414,7 +414,7 @@ cudaError_t launch_integral_export(const Cube& c, void* scratch, double* out, cu
     int* C = static_cast<int*>(scratch);
     k_nf_rows<<<(2 * c.H + 127) / 128, 128, 0, st>>>(c.s1, c.s2, c.pitch, c.H, c.W, C);
     k_nf_cols<<<(2 * (c.W + 1) + 127) / 128, 128, 0, st>>>(c.H, c.W, C);
-    k_int_to_f64<<<152 * 8, 256, 0, st>>>(c.integ, c.ipitch, C, c.H, c.W, out);
+    k_int_to_f64<<<8 * device_sms(), 256, 0, st>>>(c.integ, c.ipitch, C, c.H, c.W, out);
     return cudaGetLastError();
 }
 

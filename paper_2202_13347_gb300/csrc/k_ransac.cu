@@ -855,7 +855,9 @@ cudaError_t launch_rectify(const float* img, int H, int W, size_t pitch, const d
     constexpr int rows = kRectH * (kRsThreads / 32);
     const unsigned gy = (unsigned)((out_h + rows - 1) / rows);
     // four tiles a warp once that still leaves two CTAs per SM
-    const int per = (size_t)gy * ((out_w + kRectTiles * kRectW - 1) / (kRectTiles * kRectW)) >= 2 * 152 ? kRectTiles : 1;
+    const int per = (size_t)gy * ((out_w + kRectTiles * kRectW - 1) / (kRectTiles * kRectW)) >= 2 * (size_t)device_sms()
+                        ? kRectTiles
+                        : 1;
     dim3 grid((unsigned)((out_w + per * kRectW - 1) / (per * kRectW)), gy);
     k_rectify<<<grid, kRsThreads, 0, st>>>(img, H, W, pitch, Hm, fill, out_h, out_w, out, per);
     return cudaGetLastError();

@@ -926,7 +926,7 @@ ImgPair img_none() {
 // (three CTAs of four warps per SM) x rows streamed (10 more than the output
 // rows).
 int steer_rows_for(const ImgJob* j, int n) {
-    const int slots = 3 * 152;
+    const int slots = 3 * device_sms();
     int H = 0;
     for (int i = 0; i < n; ++i) H = j[i].H > H ? j[i].H : H;
     long best = -1;
@@ -1023,7 +1023,7 @@ int smooth_ctas_for(const ImgJob& j, int rows) { return ((j.W + kStW - 1) / kStW
 // runs a block in about half the time of two together): the rows with the
 // fewest blocks on the fullest SM.
 int strip_rows_for(const ImgJob* j, int n) {
-    const long sms = 152;
+    const long sms = device_sms();
     int H = 0;
     for (int i = 0; i < n; ++i) H = j[i].H > H ? j[i].H : H;
     long best = -1;
@@ -1125,7 +1125,7 @@ cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, cons
 }
 
 cudaError_t launch_cube_export(const Cube& c, float* out, cudaStream_t st) {
-    int blocks = 152 * 8;
+    const int blocks = 8 * device_sms();
     if (c.dtype == SFOC_DTYPE_BF16)
         k_cube_export_bf16<<<blocks, 256, 0, st>>>(c.rm, c.H, c.W, c.z, out);
     else

@@ -251,3 +251,11 @@ def test_few_points_and_many_take_the_form_that_is_faster_for_them(lib, case, dt
         assert lib.sfoc_cube_free(c) == 0
     other.close()
     ctx.close()
+
+
+def test_launch_plans_ask_the_device_for_its_sms():
+    """Segment heights and grids that fill the chip follow the device's SM count."""
+    for name in sorted(os.listdir(CSRC)):
+        with open(os.path.join(CSRC, name)) as f:
+            code = [line.split("//")[0] for line in f]
+        assert not [c for c in code if "152" in c], name
