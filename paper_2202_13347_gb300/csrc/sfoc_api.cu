@@ -525,9 +525,9 @@ sfoc_status build_cube(sfoc_ctx* ctx, const T* d_image, int H, int W, size_t pit
 // Puts a cube into one of the context's pair slots.  The cube it replaces (of
 // another shape or type) is freed once the work queued on the stream is done
 // with it; one that a captured graph may read lives as long as the context.
-void set_pair_cube(sfoc_ctx* ctx, sfoc_cube** slot, sfoc_cube* cube) {
+// cap: the stream is being captured.
+void set_pair_cube(sfoc_ctx* ctx, sfoc_cube** slot, sfoc_cube* cube, bool cap) {
     sfoc_cube* const old = *slot;
-    const bool cap = capturing(ctx->stream);
     *slot = cube;
     cube->in_graph = cube->in_graph || cap;
     if (!old || old == cube) return;
@@ -544,7 +544,7 @@ sfoc_status build_pair_cube(sfoc_ctx* ctx, const float* d_image, int H, int W, c
                             sfoc_cube** slot) {
     sfoc_cube* cube = *slot;
     const sfoc_status s = build_cube(ctx, d_image, H, W, (size_t)W, nullptr, 0, 0, p, &cube);
-    if (s == SFOC_OK) set_pair_cube(ctx, slot, cube);
+    if (s == SFOC_OK) set_pair_cube(ctx, slot, cube, capturing(ctx->stream));
     return s;
 }
 
@@ -587,7 +587,8 @@ sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, 
     // the workspace grows only where a single build would have it grow as well
     const bool grows = at[2] > ctx->ws_bytes;
     if (grows && std::max(at[1], at[2] - at[1]) <= ctx->ws_bytes) return SFOC_OK;
-    if ((grows || !fits[0] || !fits[1]) && capturing(ctx->stream)) return SFOC_OK;
+    const bool cap = capturing(ctx->stream);
+    if ((grows || !fits[0] || !fits[1]) && cap) return SFOC_OK;
     sfoc_status s = SFOC_OK;
     for (int k = 0; k < 2; ++k) {
         sfoc_cube* c = *cube[k];
@@ -600,7 +601,7 @@ sfoc_status build_small_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int Wr, 
                 return s;
             }
         }
-        set_pair_cube(ctx, cube[k], c);
+        set_pair_cube(ctx, cube[k], c, cap);
     }
     s = ensure_ws(ctx, at[2]);
     if (s == SFOC_ERR_OOM) return SFOC_OK;  // one image's workspace may still fit
