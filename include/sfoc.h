@@ -219,6 +219,10 @@ SFOC_API sfoc_status sfoc_params_default(sfoc_params* p);
  * The cube holds z = 2*n_orient channels (first-order then second-order
  * orientations), each normalised per group, plus per-pixel sums over
  * channels of g and g^2 used for the integral images of Eq. 14.
+ * Device memory of a cube, per pixel (rows padded to 32 pixels but for the
+ * chunks): F32 4 z bytes; BF16 (12 channels) 64 for the chunks of 8 in both
+ * pixel orders, which the tensor-core forms read, and 24 for the planes, which
+ * the Fourier forms read; for both 8 for the sums and 16 for the integral images.
  */
 SFOC_API sfoc_status sfoc_build(sfoc_ctx* ctx, const float* d_image, int H, int W, size_t pitch_elems,
                        const double* scales, int n_scales, int n_orient, const sfoc_params* p,
@@ -294,8 +298,10 @@ SFOC_API sfoc_status sfoc_cube_free(sfoc_cube* cube);
  * kernel (opts->corr_path), R_S and R_SS from the reference cube's integral
  * images (Eq. 14-16: exact 64-bit sums of the per-pixel channel sums rounded
  * to multiples of 2^-28, built on first use and kept with the cube), R_T and
- * R_TT from the same sums over the template, the variances in FP64.  Ties go
- * to the smallest dy, then the smallest dx.  The workspace grows to
+ * R_TT from the same sums over the template; the variance of a window from an
+ * exact integer product rounded to FP32 (2^-22 of its value), the template's in
+ * FP64, rounded to FP32, and the quotient in FP32.  Ties go to the smallest dy,
+ * then the smallest dx.  The workspace grows to
  * sfoc_match_workspace_bytes(n, R) if it is smaller.
  * Errors: SFOC_ERR_INVALID_ARG for a NULL cube, NULL points or output with
  * n > 0, n < 0, m < 1, R < 0 or an unknown corr_path; SFOC_ERR_SHAPE when

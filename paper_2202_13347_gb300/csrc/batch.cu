@@ -167,7 +167,7 @@ cudaError_t enqueue_build(sfoc_ctx* ctx, BatchPlan* p, cudaStream_t s) {
     for (size_t i = 0; i < p->img.size(); ++i) {  // parameters without a batched kernel: one image at a time
         const ImgJob& j = p->img[i];
         StageScope sc(ctx, ST_STEER, 1 + smooth_launch_count(p->sm));
-        e = launch_sfoc_steer(static_cast<const float*>(j.img), j.H, j.W, j.pitch, j.F, j.fpitch, p->st, 0, s);
+        e = launch_sfoc_steer(static_cast<const float*>(j.img), j.H, j.W, j.pitch, j.F, j.fpitch, p->st, s);
         if (e == cudaSuccess) e = launch_sfoc_smooth(j.F, j.fpitch, j.H, j.W, p->sm, p->cubes[i]->c, s);
         if (e != cudaSuccess) return e;
     }

@@ -139,9 +139,9 @@ __device__ __forceinline__ const ImgJob& img_job(const ImgPair& one, const ImgJo
 
 // ---- kernel launchers (return cudaError_t of the launch) ----------------
 cudaError_t launch_sfoc_steer(const float* img, int H, int W, size_t pitch, float* F, size_t fpitch,
-                              const SteerTaps& tp, int z_first, cudaStream_t st);
+                              const SteerTaps& tp, cudaStream_t st);
 cudaError_t launch_sfoc_steer(const uint16_t* img, int H, int W, size_t pitch, float* F, size_t fpitch,
-                              const SteerTaps& tp, int z_first, cudaStream_t st);
+                              const SteerTaps& tp, cudaStream_t st);
 cudaError_t launch_sfoc_smooth(const float* F, size_t fpitch, int H, int W, const SmoothTaps& tp, Cube& c,
                                cudaStream_t st);
 // Batched build of several float images with the paper's radii and rates

@@ -14,8 +14,10 @@
 //                   in exact 96-bit integers: mnz R_SS - R_S^2 (the
 //                   variance times mnz) and, for the uncentred correlation
 //                   forms, R_S R_T (the mean correction of the numerator);
-//                   each is rounded to FP32 once, then NCC = num / sqrt(vS vT)
-//                   in FP32; a warp-shuffle argmax with the (NCC desc, dy
+//                   each is converted to FP32 (two roundings, relative error
+//                   below 2^-23) and scaled by 2^-56 / mnz in FP32 (two more, the
+//                   factor's and the product's), then NCC = num / sqrt(vS vT) in
+//                   FP32; a warp-shuffle argmax with the (NCC desc, dy
 //                   asc, dx asc) order and a 3-point parabola per axis.  No
 //                   FP64 per offset: GB300 runs it at a small fraction of its
 //                   FP32 rate, and the integer products cost a few 32-bit

@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(kStThreads, 2)
             asm volatile("bar.sync %0, %1;" ::"r"(kFull + b), "n"(kStThreads) : "memory");
             const float* done = s_done + (size_t)b * kStChan * U * kStW + (warp - kStChan) * kStW + 2 * lane;
             uint4* chunk = s_chunk + (size_t)b * U * G::CP + (warp - kStChan) * G::CP + 2 * lane;
-auto finish = [&](auto vec) {
+            auto finish = [&](auto vec) {
 #pragma unroll
                 for (int v = 0; v < U / kStFin; ++v)
                     if (yb + v * kStFin < y1 && gx < W)
@@ -979,12 +979,12 @@ cudaError_t launch_steer_any(const T* img, int H, int W, size_t pitch, float* F,
 }  // namespace
 
 cudaError_t launch_sfoc_steer(const float* img, int H, int W, size_t pitch, float* F, size_t fpitch,
-                              const SteerTaps& tp, int /*z_first*/, cudaStream_t st) {
+                              const SteerTaps& tp, cudaStream_t st) {
     return launch_steer_any(img, H, W, pitch, F, fpitch, tp, st);
 }
 
 cudaError_t launch_sfoc_steer(const uint16_t* img, int H, int W, size_t pitch, float* F, size_t fpitch,
-                              const SteerTaps& tp, int /*z_first*/, cudaStream_t st) {
+                              const SteerTaps& tp, cudaStream_t st) {
     return launch_steer_any(img, H, W, pitch, F, fpitch, tp, st);
 }
 

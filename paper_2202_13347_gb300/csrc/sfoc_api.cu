@@ -507,7 +507,7 @@ sfoc_status build_cube(sfoc_ctx* ctx, const T* d_image, int H, int W, size_t pit
     cudaError_t e;
     {
         StageScope sc(ctx, ST_STEER, 1);
-        e = launch_sfoc_steer(d_image, H, W, pitch_elems, F, fpitch, st, z, ctx->stream);
+        e = launch_sfoc_steer(d_image, H, W, pitch_elems, F, fpitch, st, ctx->stream);
     }
     if (e == cudaSuccess) {
         StageScope sc(ctx, ST_SMOOTH, smooth_launch_count(sm));
@@ -1396,7 +1396,7 @@ sfoc_status sfoc_build_static(sfoc_ctx* ctx, const float* d_image, int H, int W,
     const SteerTaps st = make_steer(p);
     const SmoothTaps sm = make_smooth(p);
     ctx->launches += 1 + smooth_launch_count(sm);
-    e = launch_sfoc_steer(d_image, H, W, pitch_elems, F, fpitch, st, z, ctx->stream);
+    e = launch_sfoc_steer(d_image, H, W, pitch_elems, F, fpitch, st, ctx->stream);
     if (e == cudaSuccess) e = launch_sfoc_smooth(F, fpitch, H, W, sm, c, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "sfoc kernels");
     return SFOC_OK;

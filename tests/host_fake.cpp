@@ -136,10 +136,10 @@ FAKE cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t a, cudaEvent_t b) {
 // ---- the launchers ----------------------------------------------------------
 
 namespace sfoc {
-cudaError_t launch_sfoc_steer(const float*, int, int, size_t, float*, size_t, const SteerTaps&, int, cudaStream_t) {
+cudaError_t launch_sfoc_steer(const float*, int, int, size_t, float*, size_t, const SteerTaps&, cudaStream_t) {
     return count("steer");
 }
-cudaError_t launch_sfoc_steer(const uint16_t*, int, int, size_t, float*, size_t, const SteerTaps&, int, cudaStream_t) {
+cudaError_t launch_sfoc_steer(const uint16_t*, int, int, size_t, float*, size_t, const SteerTaps&, cudaStream_t) {
     return count("steer");
 }
 cudaError_t launch_sfoc_smooth(const float*, size_t, int, int, const SmoothTaps&, Cube&, cudaStream_t) {
