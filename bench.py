@@ -50,9 +50,10 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12   # SMs x FP32 lanes x 2 flop 
 FFT_SIZES = (64, 128)  # transform sides of SFOC_CORR_FFT (the smallest with m + 2R <= L); AUTO adds 96, 160, 192, 224
 # DRAM bytes (read + write) per processed point of a correlation kernel on
 # the 2048x2048 workload (m = 81, R = 20), keyed by (form, correlation path),
-# from one ncu capture of the kernel as it stands (the band form: 87.12 MB
-# read + 4.61 MB written for the autotuner's 304-point launch); absent where
-# none is current.  A launch's traffic is this times the points it processed.
+# from one ncu capture (the band form: 87.12 MB read + 4.61 MB written for the
+# autotuner's 304-point launch, taken before its waiting warps slept; the 1000
+# points of a step since then: 270.0 + 11.4 MB, 7 % less a point); absent where
+# there is none.  A launch's traffic is this times the points it processed.
 CORR_TRAFFIC_PER_POINT_SAR2048 = {("bf16", 5): (87.118848e6 + 4.611072e6) / 304}
 
 
@@ -704,10 +705,11 @@ def run_batch_form(b, torch, ctx, pairs, form, steps, warmup, corr_name="auto"):
 
 
 # DRAM bytes per processed point of a band-form class, by (template side,
-# band instance NQ), from ncu captures of the kernel as it stands, each of the
-# 2048x2048 pair's 1000 points matched with forced band form at one (m, R):
-# m = 101, R = 40 (851 processed; 745.06 MB read + 44.46 MB written per
-# launch) and m = 81, R = 36 (879 points in bounds; 359.81 MB + 30.00 MB).  A
+# band instance NQ), from ncu captures, each of the 2048x2048 pair's 1000 points
+# matched with forced band form at one (m, R): m = 101, R = 40 (851 processed;
+# 745.06 MB read + 44.46 MB written per launch) and m = 81, R = 36 (879 points in
+# bounds; 359.81 MB + 30.00 MB).  They were taken before the kernel's waiting
+# warps slept; since then 690.65 + 43.06 and 368.27 + 29.74 MB (7 % less, 2 % more).  A
 # batched class of the same template side and instance gets this times its
 # processed points (its radii range over R 33-40).
 BAND_TRAFFIC_PER_POINT = {(101, 6): (745.062144e6 + 44.461312e6) / 851,
@@ -964,7 +966,7 @@ def short_line(line):
     out["forms"] = {f: form(s) for f, s in line["forms"].items()}
     out["peaks"] = {k: v for k, v in line["peaks"].items() if k != "microbench"}
     drop = {"e2e": ("sync_call", "plans_built_in_timed_calls"), "cpu_baseline": ("sfoc_sample",),
-            "config": ("pixels_per_rank",)}
+            "config": ("pixels_per_rank",), "parity": ("note",)}
     for key, names in drop.items():
         if line[key]:
             out[key] = {k: v[:5] if isinstance(v, list) else v for k, v in line[key].items() if k not in names}
