@@ -326,9 +326,12 @@ static int tune_waves(int n, int sms) {
 
 // A candidate's time for w points per SM from its times for one (t1) and for
 // K > 1 (tK).  Most forms run one CTA per SM and take as much longer for every
-// further point; two of the Fourier sides run two points together on an SM, side
-// 96 four, with 0.25, 0.7 and 1 of the fourth's extra time for the second to
-// fourth (m = 41, R = 25: 123, 155, 215 and 253 us; BF16 cubes 145, 182, 248, 290).
+// further point: evenly between the two, in proportion beyond (where a form's small
+// CTAs leave the chip idle up to K points per SM, as the direct kernel's do for a
+// small m and R, the slope of the two says nothing about more).  Two of the
+// Fourier sides run two points together on an SM, side 96 four, with 0.25, 0.7 and
+// 1 of the fourth's extra time for the second to fourth (m = 41, R = 25: 123, 155,
+// 215 and 253 us; BF16 cubes 145, 182, 248, 290).
 static double tune_predict(int path, int option, double t1, double tK, int K, int w) {
     if (path == SFOC_CORR_FFT && (option == 64 || option == 160)) {
         const double t2 = K == 2 ? tK : K == 3 ? tK - t1 : tK / 2;
@@ -338,7 +341,7 @@ static double tune_predict(int path, int option, double t1, double tK, int K, in
         static const double extra[kTuneWaves] = {0.0, 0.25, 0.7, 1.0};
         return t1 + extra[w - 1] / extra[K - 1] * (tK - t1);
     }
-    return t1 + (w - 1) * (tK - t1) / (K - 1);
+    return w > K ? tK * w / K : t1 + (w - 1) * (tK - t1) / (K - 1);
 }
 
 const TuneEntry* autotune_pair(sfoc_ctx* ctx, int dtype, int family, MatchJob one) {

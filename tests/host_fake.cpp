@@ -61,6 +61,7 @@ FAKE void fk_capturing(int on) { g_capturing = on != 0; }
 FAKE int fk_count(const char* name) { return g_count.count(name) ? g_count[name] : 0; }
 FAKE void fk_reset() { g_count.clear(); }
 FAKE int fk_last_form() { return g_last_form; }
+FAKE void fk_no_costs() { g_cost.clear(); }
 FAKE void fk_cost(int form, int waves, double ms) { g_cost[form][waves] = ms; }
 
 // ---- the runtime ------------------------------------------------------------

@@ -214,6 +214,7 @@ def test_few_points_and_many_take_the_form_that_is_faster_for_them(lib, case, dt
     it (a first call of up to a point per SM knows only that and keeps its choice)."""
     ctx = Ctx(lib)
     forms = COSTS[case]
+    lib.fk_no_costs()
     for (path, side), by_waves in forms.items():
         for w, ms in by_waves.items():
             lib.fk_cost(1000 * path + side, w, ms)
@@ -250,6 +251,21 @@ def test_few_points_and_many_take_the_form_that_is_faster_for_them(lib, case, dt
     for c in cubes:
         assert lib.sfoc_cube_free(c) == 0
     other.close()
+    ctx.close()
+
+
+def test_a_sample_that_leaves_the_chip_idle_promises_nothing_for_more_points(lib):
+    """The direct kernel runs three points of m = 15, R = 1 on an SM at a time: 304
+    points take no longer than 152, which says nothing about 608."""
+    ctx = Ctx(lib)
+    lib.fk_no_costs()
+    for (path, side), by_waves in {(FFT, 64): (0.028, 0.038), (FFT, 128): (0.075,), (DIRECT, 0): (0.0567, 0.0568, 0.0589)}.items():
+        for w, ms in enumerate(by_waves):
+            lib.fk_cost(1000 * path + side, w + 1, ms)
+    cubes = [ctx.build(400, 400) for _ in range(2)]
+    assert [ctx.match(*cubes, n, 15, 1) for n in (304, 100, 608, 1216, 5000)] == [1000 * FFT + 64] * 5
+    for c in cubes:
+        assert lib.sfoc_cube_free(c) == 0
     ctx.close()
 
 
