@@ -146,8 +146,6 @@ void free_cube_mem(Cube& c);
 sfoc_status build_integral(sfoc_ctx* ctx, Cube& c);
 inline size_t roundup(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t align256(size_t v) { return roundup(v, 256); }
-// the library's SM count of the context's device
-int sm_count(int device);
 
 // Correlation dispatch for one pair (the points of `one`): `path` is a
 // concrete sfoc_corr_path (DIRECT_F32, FFT, TC_TOEPLITZ, TC_COLUMN,

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 
 #include "../../include/sfoc.h"
@@ -27,12 +28,23 @@ constexpr int kMaxRadius = 63;
 // A separable 2-D kernel a(x) b(y) is applied as a horizontal pass with a
 // and a vertical pass with b; "odd" taps satisfy t(-q) = -t(q) and "even"
 // taps t(-q) = t(q), so only q = 0..K are stored.
-// SMs of the current device: the launchers' plans fill them
-inline int device_sms() {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+// SMs of a device, asked once: the launchers' plans fill them
+inline int sm_count(int device) {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
+    const bool slot = device >= 0 && device < kDevices;
+    int sms = slot ? known[device].load(std::memory_order_relaxed) : 0;
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 148;
+        if (slot) known[device].store(sms, std::memory_order_relaxed);
+    }
     return sms;
+}
+// of the current device
+inline int device_sms() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return sm_count(dev);
 }
 
 struct SteerTaps {

@@ -49,12 +49,6 @@ bool capturing(cudaStream_t s) {
     return cs != cudaStreamCaptureStatusNone;
 }
 
-int sm_count(int device) {
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    return sms;
-}
-
 static cudaEvent_t pool_event(sfoc_ctx* c) {
     if (!c->pool.empty()) {
         cudaEvent_t e = c->pool.back();
@@ -543,11 +537,11 @@ void set_pair_cube(sfoc_ctx* ctx, sfoc_cube** slot, sfoc_cube* cube, bool cap) {
 }
 
 // sfoc_build of a dense image into a pair slot
-sfoc_status build_pair_cube(sfoc_ctx* ctx, const float* d_image, int H, int W, const sfoc_params* p,
+sfoc_status build_pair_cube(sfoc_ctx* ctx, const float* d_image, int H, int W, const sfoc_params* p, bool cap,
                             sfoc_cube** slot) {
     sfoc_cube* cube = *slot;
     const sfoc_status s = build_cube(ctx, d_image, H, W, (size_t)W, nullptr, 0, 0, p, &cube);
-    if (s == SFOC_OK) set_pair_cube(ctx, slot, cube, capturing(ctx->stream));
+    if (s == SFOC_OK) set_pair_cube(ctx, slot, cube, cap);
     return s;
 }
 
@@ -1084,9 +1078,10 @@ sfoc_status fastncc_register_pair(sfoc_ctx* ctx, const float* d_ref, int Hr, int
     sfoc_status s = build_small_pair(ctx, d_ref, Hr, Wr, d_sen, Hs, Ws, p, &both);
     if (s != SFOC_OK) return s;
     if (!both) {
-        s = build_pair_cube(ctx, d_ref, Hr, Wr, p, &ctx->pair_ref);
+        const bool cap = capturing(ctx->stream);
+        s = build_pair_cube(ctx, d_ref, Hr, Wr, p, cap, &ctx->pair_ref);
         if (s != SFOC_OK) return s;
-        s = build_pair_cube(ctx, d_sen, Hs, Ws, p, &ctx->pair_sen);
+        s = build_pair_cube(ctx, d_sen, Hs, Ws, p, cap, &ctx->pair_sen);
         if (s != SFOC_OK) return s;
     }
     return fastncc_match(ctx, ctx->pair_ref, ctx->pair_sen, d_points, n, template_size, search_radius, opts, d_out);
@@ -1147,11 +1142,12 @@ sfoc_status fastncc_register_pair_host(sfoc_ctx* ctx, const float* h_ref, int Hr
         return st;
     };
     if (e != cudaSuccess) return drained(cuda_fail(ctx, e, "host to device copy"));
-    sfoc_status s = build_pair_cube(ctx, d_ref, Hr, Wr, p, &ctx->pair_ref);
+    // (a call that waits for its results is never captured)
+    sfoc_status s = build_pair_cube(ctx, d_ref, Hr, Wr, p, false, &ctx->pair_ref);
     if (s != SFOC_OK) return drained(s);
     e = cudaStreamWaitEvent(ctx->stream, ctx->ev_copied, 0);
     if (e != cudaSuccess) return drained(cuda_fail(ctx, e, "cudaStreamWaitEvent"));
-    s = build_pair_cube(ctx, d_sen, Hs, Ws, p, &ctx->pair_sen);
+    s = build_pair_cube(ctx, d_sen, Hs, Ws, p, false, &ctx->pair_sen);
     if (s == SFOC_OK)
         s = fastncc_match(ctx, ctx->pair_ref, ctx->pair_sen, d_pts, n, template_size, search_radius, opts, d_out);
     if (s != SFOC_OK) return drained(s);

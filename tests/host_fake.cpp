@@ -97,7 +97,7 @@ FAKE cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cuda
 FAKE cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
 FAKE cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 FAKE cudaError_t cudaGetDeviceCount(int* n) { return *n = 1, cudaSuccess; }
-FAKE cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = kSms, cudaSuccess; }
+FAKE cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = kSms, count("attribute"); }
 FAKE cudaError_t cudaGetLastError() { return cudaSuccess; }
 FAKE const char* cudaGetErrorString(cudaError_t) { return "fake"; }
 FAKE cudaError_t cudaGetSymbolAddress(void** p, const void*) { return *p = nullptr, cudaErrorUnknown; }

@@ -269,6 +269,19 @@ def test_a_sample_that_leaves_the_chip_idle_promises_nothing_for_more_points(lib
     ctx.close()
 
 
+def test_the_sm_count_is_asked_once(ctx):
+    """Not on every call: small calls wait for the host."""
+    cubes = [ctx.build(300, 300) for _ in range(2)]
+    ctx.match(*cubes, 200, 41, 10)
+    ctx.L.fk_reset()
+    for n in (10, 200, 1000):
+        ctx.match(*cubes, n, 41, 10)
+        ctx.ok(ctx.pair((300, 300), (300, 300)))
+    assert ctx.L.fk_count(b"attribute") == 0
+    for c in cubes:
+        assert ctx.L.sfoc_cube_free(c) == 0
+
+
 def test_launch_plans_ask_the_device_for_its_sms():
     """Segment heights and grids that fill the chip follow the device's SM count."""
     for name in sorted(os.listdir(CSRC)):
